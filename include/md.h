@@ -407,11 +407,17 @@ md_status md_get_step(md_ctx *ctx, int64_t *step);
 /* ---- tuning (runtime control; no counterpart in the paper) ---------------
  * md_tuning_list: writes up to cap entries of the compiled kernel
  * configurations into list (may be NULL) and returns their number.
- * md_set_tuning: uses the given configuration from now on.
- * md_get_tuning: the configuration in use.
+ * md_set_tuning: uses the given configuration of the step kernel from now on.
+ * Until then (and after md_autotune, if it was the fastest) a context without
+ * ionizing clusters or target slices takes the step that evaluates each pair
+ * of records once for both, where it has room for its partial sums (12 bytes
+ * per 1024 or 1536 pairs, at most 16 GB); its sums have another order.
+ * md_get_tuning: the step kernel configuration in use, or the one that would
+ * be without that step.
  * md_autotune: times every configuration over `steps` steps on the
  * context's own state (restored afterwards), with jsplit 0 and, for the two
- * fastest, jsplit -2 and -4 (no ionizing cluster), and keeps the fastest; the
+ * fastest, jsplit -2 and -4 (no ionizing cluster), then the step that takes
+ * each pair once, and keeps the fastest; the
  * per-configuration best mean step times in ms go to times_ms (cap entries,
  * may be NULL; -1 for a configuration not timed). */
 int32_t md_tuning_list(md_tuning *list, int32_t cap);

@@ -40,6 +40,14 @@ struct KernelConfig {
 
 const KernelConfig* step_configs(int* count);
 
+// One step with each pair evaluated once (md_mutual.cu): the pair sums and the
+// push.  det: with the detector epilogue; pot: a diagnostic step; mi: with the
+// minimum-image twin (pot and mi exclude one another).
+cudaError_t launch_mut_step(const MutArgs& a, int grid, bool det, bool pot, bool mi,
+                            cudaStream_t s);
+// (resident CTAs per SM of the pair kernel; block: records per i-block)
+cudaError_t mut_blocks_per_sm(int block, bool pot, bool mi, int* out);
+
 // Field (and potential) at nt targets from ns sources (FP32/Kahan direct sum),
 // with the sources split as a.nseg / a.seg_len / a.part say.
 cudaError_t launch_field(const FieldArgs& a, bool potential, cudaStream_t s);

@@ -130,6 +130,19 @@ struct md_ctx {
 
   cudaGraphExec_t graph = nullptr;
 
+  // the step with each pair evaluated once (md_mutual.cu): its work list and
+  // partial sums, while `mut_on`
+  bool forced = false;  // md_set_tuning or md_autotune chose: no automatic choice
+  bool mut_on = false;
+  md::MutUnit* d_mut_units = nullptr;
+  int* d_mut_first = nullptr;
+  md::MutBlk* d_mut_blks = nullptr;
+  int mut_shares = 0, mut_blks = 0, mut_grid = 0, mut_block = 0;
+  double* d_mut_ipart = nullptr;
+  float* d_mut_jpart = nullptr;
+  double* d_mut_jphi = nullptr;   // allocated by the first diagnostic step
+  long long mut_jrecs = 0;        // records of all rows of jpart
+
   // ionization
   std::vector<md::IonDev> ion;
   std::vector<long long> ion_out_off;  // per cluster, into d_ion_out / d_ion_fired
@@ -395,6 +408,28 @@ cudaError_t launch_step_of(const md_ctx* c, const md::KernelConfig& k, const md:
     return c->det_on ? k.launch_step_mi_det(a, c->grid, s) : k.launch_step_mi(a, c->grid, s);
   }
   return c->det_on ? k.launch_step_det(a, c->grid, s) : k.launch_step(a, c->grid, s);
+}
+
+md::MutArgs mut_args(md_ctx* c) {
+  md::MutArgs a;
+  a.s = step_args(c);
+  a.units = c->d_mut_units;
+  a.share_first = c->d_mut_first;
+  a.n_shares = c->mut_shares;
+  a.blks = c->d_mut_blks;
+  a.n_blks = c->mut_blks;
+  a.block = c->mut_block;
+  a.ipart = c->d_mut_ipart;
+  a.jpart = c->d_mut_jpart;
+  a.jphi = c->d_mut_jphi;
+  return a;
+}
+
+// The kernels of one step of a context.
+cudaError_t launch_one_step(md_ctx* c, const md::KernelConfig& k, const md::StepArgs& a,
+                            cudaStream_t s) {
+  if (c->mut_on) return md::launch_mut_step(mut_args(c), c->mut_grid, c->det_on, false, c->any_mi, s);
+  return launch_step_of(c, k, a, s);
 }
 
 cudaError_t blocks_per_sm_of(const md_ctx* c, const md::KernelConfig& k, int* bps) {
@@ -665,6 +700,135 @@ md_status configure(md_ctx* c, int cfg, int ctas_per_sm, int jsplit) {
   return MD_OK;
 }
 
+void mut_off(md_ctx* c) {
+  if (c->mut_on) destroy_graph(c);
+  c->mut_on = false;
+  cudaFree(c->d_mut_units);
+  cudaFree(c->d_mut_first);
+  cudaFree(c->d_mut_blks);
+  cudaFree(c->d_mut_ipart);
+  cudaFree(c->d_mut_jpart);
+  cudaFree(c->d_mut_jphi);
+  c->d_mut_units = nullptr;
+  c->d_mut_first = nullptr;
+  c->d_mut_blks = nullptr;
+  c->d_mut_ipart = nullptr;
+  c->d_mut_jpart = nullptr;
+  c->d_mut_jphi = nullptr;
+}
+
+// Rows of jpart at most: 16 GB (1.6M records in one cluster); a larger context
+// keeps the step kernel.
+constexpr long long kMutMaxRecs = (16LL << 30) / 12;
+// Records from which a cluster with minimum-image forces takes it.  Another
+// order of the sums moves next step's FP32 positions by an ulp here and there,
+// and a pair half a box apart then takes its other image: a kick of up to
+// 8 K_C dt / L^2.  At the density of a solid cluster that stays below 1e-3 of a
+// 10 eV electron's momentum from 11000 records on; smaller periodic clusters
+// keep the step kernel and its order.
+constexpr long long kMutMinImageRecords = 11000;
+constexpr long long kMutBigRecords = 40000;
+constexpr long long kMutMinTiles = 2;
+
+// Sets up the step with each pair evaluated once, if the context can take it
+// (no ionizing cluster, no target slice, room for the partial sums); otherwise
+// the configured step kernel stays.
+md_status mut_configure(md_ctx* c) {
+  MD_CUDA(cudaStreamSynchronize(c->stream));
+  mut_off(c);
+  if (c->any_ion || c->any_slice) return MD_OK;
+  for (int ci = 0; ci < c->n_clusters; ++ci)
+    if (c->min_image[ci] && c->cl[ci].n < kMutMinImageRecords) return MD_OK;
+  // 12 targets per thread (fewer shuffles and loads per pair) once the largest
+  // cluster has kMutBigRecords, else 8 (smaller blocks, so less of the
+  // one-sided work and of the padding)
+  const long long B = c->max_n >= kMutBigRecords ? 128 * 12 : 128 * 8;
+  constexpr long long T = md::kMutTile;
+  int bps = 0;
+  MD_CUDA(md::mut_blocks_per_sm(static_cast<int>(B), false, c->any_mi, &bps));
+  if (bps < 1) return MD_OK;
+  const long long slots = static_cast<long long>(bps) * c->sm_count;
+  std::vector<md::MutBlk> blks;
+  long long jrecs = 0, weight = 0;
+  for (int ci = 0; ci < c->n_clusters; ++ci) {
+    const long long n = c->cl[ci].n_pad, nb = (n + B - 1) / B;
+    const long long base = jrecs;
+    for (long long b = 0; b < nb; ++b) {
+      const long long nt = (n - b * B + T - 1) / T, own = std::min(nt, B / T);
+      blks.push_back({ci, static_cast<int>(b), 0, 0, base});
+      jrecs += std::max(0LL, n - (b + 1) * B);
+      weight += md::kMutWeightOwn * own + md::kMutWeightPair * (nt - own);
+    }
+  }
+  if (jrecs > kMutMaxRecs || blks.size() > (1u << 27)) return MD_OK;
+  // Shares in rounds of one per resident CTA: a round takes three eighths of
+  // the work that is left.  The CTAs of an SM do not advance alike (one share
+  // each, all equal: 10.8 ms per step at 200k records; eight rounds of equal
+  // shares 9.8; these 9.6; half of what is left per round 10.2), and a share
+  // keeps at least kMutMinTiles tiles because each of its units writes a
+  // partial sum of every target of its block (19k records: 0.150 ms with 2,
+  // 0.165 with 3).
+  std::vector<long long> cut;  // the shares' ends, in weight
+  for (long long left = weight, at = 0; left > 0;) {
+    const long long w = std::max<long long>(kMutMinTiles * md::kMutWeightPair,
+                                            (3 * left + 8 * slots - 1) / (8 * slots));
+    for (long long k = 0; k < slots && left > 0; ++k) {
+      const long long take = std::min(left, w);
+      at += take;
+      left -= take;
+      cut.push_back(at);
+    }
+  }
+  std::vector<md::MutUnit> units;
+  std::vector<int> first(cut.size() + 1, 0);
+  long long w = 0;
+  size_t share = 0;
+  for (md::MutBlk& bk : blks) {
+    const long long n = c->cl[bk.cluster].n_pad, b = bk.block;
+    const long long nt = (n - b * B + T - 1) / T;
+    const long long jrow = bk.jbase + b * n - B * (b * (b + 1) / 2);
+    bk.unit0 = static_cast<int>(units.size());
+    for (long long t = 0; t < nt; ++t) {
+      const size_t before = share;
+      while (share + 1 < cut.size() && w >= cut[share]) ++share;
+      if (t == 0 || share != before) {
+        units.push_back({bk.cluster, bk.block, static_cast<int>(t), 0, jrow});
+        ++first[share + 1];
+      }
+      ++units.back().nt;
+      w += t < B / T ? md::kMutWeightOwn : md::kMutWeightPair;
+    }
+    bk.units = static_cast<int>(units.size()) - bk.unit0;
+  }
+  const long long G = static_cast<long long>(cut.size());
+  for (size_t i = 1; i < first.size(); ++i) first[i] += first[i - 1];
+  cudaError_t e = dev_alloc(&c->d_mut_jpart, 3 * static_cast<size_t>(jrecs));
+  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_ipart, 4 * static_cast<size_t>(B) * units.size());
+  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_units, units.size());
+  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_first, first.size());
+  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_blks, blks.size());
+  if (e != cudaSuccess) {  // no room: the step kernel needs none of this
+    cudaGetLastError();
+    mut_off(c);
+    return MD_OK;
+  }
+  MD_CUDA(cudaMemcpyAsync(c->d_mut_units, units.data(), units.size() * sizeof(md::MutUnit),
+                          cudaMemcpyHostToDevice, c->stream));
+  MD_CUDA(cudaMemcpyAsync(c->d_mut_first, first.data(), first.size() * sizeof(int),
+                          cudaMemcpyHostToDevice, c->stream));
+  MD_CUDA(cudaMemcpyAsync(c->d_mut_blks, blks.data(), blks.size() * sizeof(md::MutBlk),
+                          cudaMemcpyHostToDevice, c->stream));
+  MD_CUDA(cudaStreamSynchronize(c->stream));
+  c->mut_shares = static_cast<int>(G);
+  c->mut_blks = static_cast<int>(blks.size());
+  c->mut_grid = static_cast<int>(std::min(G, slots));
+  c->mut_jrecs = jrecs;
+  c->mut_block = static_cast<int>(B);
+  destroy_graph(c);
+  c->mut_on = true;
+  return MD_OK;
+}
+
 // Default before autotuning: 128 threads x 4 i-particles per thread, scalar.
 int default_config(md_ctx* c) {
   (void)c;
@@ -829,7 +993,7 @@ md_status launch_steps_direct(md_ctx* c, int n) {
       if (e == cudaSuccess) e = launch_ion_pushes(c, a, c->stream);
       if (e != cudaSuccess) return cuda_fail(e, "ionization launch");
     }
-    cudaError_t e = launch_step_of(c, cfgs[c->cfg], a, c->stream);
+    cudaError_t e = launch_one_step(c, cfgs[c->cfg], a, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");
   }
   return MD_OK;
@@ -847,7 +1011,7 @@ md_status build_graph(md_ctx* c) {
     for (int s = 0; s < kGraphSteps && e == cudaSuccess; ++s) {
       if (c->any_ion) e = launch_ion_all(c, 0, cs);
       if (c->any_ion && e == cudaSuccess) e = launch_ion_pushes(c, a, cs);
-      if (e == cudaSuccess) e = launch_step_of(c, cfgs[c->cfg], a, cs);
+      if (e == cudaSuccess) e = launch_one_step(c, cfgs[c->cfg], a, cs);
     }
     cudaError_t e2 = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = e2;
@@ -866,6 +1030,7 @@ void free_ctx(md_ctx* c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream);
   destroy_graph(c);
+  mut_off(c);
   cudaFree(c->d_cl);
   for (auto p : c->d_posq) cudaFree(p);
   for (auto p : c->d_x) cudaFree(p);
@@ -1342,7 +1507,8 @@ md_status populate(md_ctx* c, int32_t n_clusters, Fill fill, md_ctx** out) {
       return st;
     }
   }
-  const md_status st = configure(c, default_config(c), 0, 0);
+  md_status st = configure(c, default_config(c), 0, 0);
+  if (st == MD_OK) st = mut_configure(c);
   if (st != MD_OK) {
     free_ctx(c);
     return st;
@@ -1674,7 +1840,8 @@ static md_status md_set_slice_body(md_ctx* c, int32_t cluster, int64_t i_begin, 
   for (int ci = 0; ci < c->n_clusters; ++ci)
     any = any || c->slice_b[ci] > 0 || c->slice_e[ci] < c->cl[ci].n_pad;
   c->any_slice = any;
-  return configure(c, c->cfg, c->ctas_per_sm, c->jsplit);
+  const md_status st = configure(c, c->cfg, c->ctas_per_sm, c->jsplit);
+  return st == MD_OK && !c->forced ? mut_configure(c) : st;
 }
 
 md_status md_set_slice(md_ctx* c, int32_t cluster, int64_t i_begin, int64_t i_end) {
@@ -1878,7 +2045,9 @@ static md_status md_step_diag_body(md_ctx* c, md_diag* out) {
   if (st != MD_OK) return st;
   const size_t nt = static_cast<size_t>(c->n_total);
   if (!c->d_diag_rec) MD_CUDA(dev_alloc(&c->d_diag_rec, 6 * nt));
-  if (c->nseg_used > 1 && c->part_phi_seg < c->nseg_used) {
+  if (c->mut_on) {
+    if (!c->d_mut_jphi) MD_CUDA(dev_alloc(&c->d_mut_jphi, static_cast<size_t>(c->mut_jrecs)));
+  } else if (c->nseg_used > 1 && c->part_phi_seg < c->nseg_used) {
     cudaFree(c->d_part_phi);
     c->d_part_phi = nullptr;
     MD_CUDA(dev_alloc(&c->d_part_phi, static_cast<size_t>(c->nseg_used) * nt));
@@ -1890,7 +2059,13 @@ static md_status md_step_diag_body(md_ctx* c, md_diag* out) {
   md::StepArgs a = step_args(c);
   a.diag_rec = c->d_diag_rec;
   a.part_phi = c->d_part_phi;
-  MD_CUDA(k.launch_step_pot(a, c->grid, c->stream));
+  if (c->mut_on) {
+    md::MutArgs ma = mut_args(c);
+    ma.s = a;
+    MD_CUDA(md::launch_mut_step(ma, c->mut_grid, false, true, false, c->stream));
+  } else {
+    MD_CUDA(k.launch_step_pot(a, c->grid, c->stream));
+  }
   for (int ci = 0; ci < c->n_clusters; ++ci) {
     md::DiagArgs d;
     d.c = slice_view(c, ci);
@@ -2027,7 +2202,12 @@ static md_status md_set_tuning_body(md_ctx* c, const md_tuning* t) {
         (t->min_blocks < 0 || cfgs[i].min_blocks == t->min_blocks)) {
       if (t->ctas_per_sm < 0) return fail(MD_ERR_ARG, "ctas_per_sm < 0");
       MD_CUDA(cudaStreamSynchronize(c->stream));
-      return configure(c, i, t->ctas_per_sm, t->jsplit);
+      const md_status st = configure(c, i, t->ctas_per_sm, t->jsplit);
+      if (st == MD_OK) {
+        c->forced = true;
+        mut_off(c);
+      }
+      return st;
     }
   }
   return fail(MD_ERR_ARG, "no compiled configuration threads=%d r=%d tile=%d packed=%d",
@@ -2157,6 +2337,8 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   cudaMemcpyAsync(&step0, c->d_step, sizeof(step0), cudaMemcpyDeviceToHost, s);
   cudaStreamSynchronize(s);
   const int cfg0 = c->cfg, cps0 = c->ctas_per_sm, js0 = c->jsplit;
+  const bool mut0 = c->mut_on;
+  mut_off(c);
   int n = 0;
   const md::KernelConfig* cfgs = md::step_configs(&n);
   cudaEvent_t e0, e1;
@@ -2168,9 +2350,11 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   std::vector<double> by_cfg(static_cast<size_t>(n), -1.0);
   // one trial: configuration i with source split js, timed over `steps`
   // steps from the saved state (restored afterwards)
+  // (i < 0: the step with each pair evaluated once)
+  bool best_mut = false;
   auto trial = [&](int i, int js) {
-    st = configure(c, i, 0, js);
-    if (st != MD_OK) return;
+    st = i < 0 ? mut_configure(c) : configure(c, i, 0, js);
+    if (st != MD_OK || (i < 0 && !c->mut_on)) return;
     st = launch_steps_direct(c, 1);  // warm-up
     if (st != MD_OK) return;
     cudaEventRecord(e0, s);
@@ -2180,11 +2364,14 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
     float ms = 0.f;
     cudaEventElapsedTime(&ms, e0, e1);
     const double per = ms / steps;
-    if (by_cfg[i] < 0.0 || per < by_cfg[i]) by_cfg[i] = per;
+    if (i >= 0 && (by_cfg[i] < 0.0 || per < by_cfg[i])) by_cfg[i] = per;
     if (per < best) {
       best = per;
-      best_cfg = i;
-      best_js = js;
+      best_mut = i < 0;
+      if (i >= 0) {
+        best_cfg = i;
+        best_js = js;
+      }
     }
     if (st == MD_OK) st = check_device_error(c);
     for (auto& b : bufs) cudaMemcpyAsync(b.dev, b.copy, b.bytes, cudaMemcpyDeviceToDevice, s);
@@ -2211,6 +2398,7 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
       for (int sh : kAutoShares)
         if (st == MD_OK) trial(order[k], -sh);
   }
+  if (st == MD_OK) trial(-1, 0);
   if (times_ms)
     for (int i = 0; i < n && i < cap; ++i) times_ms[i] = by_cfg[i];
   cudaEventDestroy(e0);
@@ -2218,8 +2406,11 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   release();
   if (st != MD_OK) {
     configure(c, cfg0, cps0, js0);
+    if (mut0) mut_configure(c);
     return st;
   }
+  if (!best_mut) mut_off(c);
+  c->forced = !best_mut;
   return configure(c, best_cfg, 0, best_js);
 }
 

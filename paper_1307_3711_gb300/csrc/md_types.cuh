@@ -124,6 +124,46 @@ struct StepArgs {
   const unsigned char* min_image;
 };
 
+// The step with each pair evaluated once (md_mutual.cu): sources per tile, the
+// weights of a mutual and of a one-sided tile in the cut into shares (14 and 11
+// FP32 operations per pair, and the shuffles).
+constexpr int kMutTile = 128;
+constexpr int kMutWeightPair = 4;
+constexpr int kMutWeightOwn = 3;
+
+// A run of source tiles [t0, t0 + nt) of one i-block; tile t holds the
+// cluster's records from the block's first + t * kMutTile on, so the tiles of
+// the first i-block's length are the block's own.
+struct MutUnit {
+  int cluster;
+  int block;
+  int t0;
+  int nt;
+  long long jrow;  // first column of the block's row of `jpart`, in records
+};
+
+// One i-block of the push: its units, and the start of its cluster's rows.
+struct MutBlk {
+  int cluster;
+  int block;
+  int unit0;
+  int units;
+  long long jbase;
+};
+
+struct MutArgs {
+  StepArgs s;
+  const MutUnit* units;
+  const int* share_first;  // first unit of every share, n_shares + 1
+  int n_shares;
+  const MutBlk* blks;
+  int n_blks;
+  int block;      // records per i-block
+  double* ipart;  // [unit][3, or 4 with the potential][block]
+  float* jpart;   // per block: [3][records after the block]
+  double* jphi;   // per block: [records after the block] (diagnostic steps)
+};
+
 // Cell list of the electrons near the ions, for the local moments of the
 // ionization pass (clusters without minimum-image forces): cells of side
 // 1.01 r_loc, hashed into kCellBuckets buckets, the electrons of each bucket
