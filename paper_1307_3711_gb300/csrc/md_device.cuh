@@ -254,17 +254,21 @@ __device__ __forceinline__ double envelope(double t, int kind, double tau) {
 // Eqs. 4-9 at time t: linear E = A sin t x, B = A sin t y; circular adds
 // E_y = A sin(t + 3pi/2) = -A cos t and B_x = A sin(t + pi/2) = A cos t.
 // out = (a_x, a_y, a_z, b_x, b_y, b_z).
-__device__ __forceinline__ void laser_field(const ClusterDev& c, double t, float* out) {
-  const double amp = c.a0 * envelope(t, c.env, c.tau);
-  double sn, cs;
-  sincos(t, &sn, &cs);
-  const double circ = c.pol ? 1.0 : 0.0;
+__device__ __forceinline__ void laser_of(double amp, double sn, double cs, int pol, float* out) {
+  const double circ = pol ? 1.0 : 0.0;
   out[0] = static_cast<float>(amp * sn);
   out[1] = static_cast<float>(-circ * amp * cs);
   out[2] = 0.0f;
   out[3] = static_cast<float>(circ * amp * cs);
   out[4] = static_cast<float>(amp * sn);
   out[5] = 0.0f;
+}
+
+__device__ __forceinline__ void laser_field(const ClusterDev& c, double t, float* out) {
+  const double amp = c.a0 * envelope(t, c.env, c.tau);
+  double sn, cs;
+  sincos(t, &sn, &cs);
+  laser_of(amp, sn, cs, c.pol, out);
 }
 
 // ---------------------------------------------------------------- Boris --
@@ -1110,21 +1114,31 @@ __device__ __forceinline__ void detect(unsigned long long* hist, unsigned char* 
   if (-b1 >= cc) atomicAdd(h + 3 * nb1 + bin, 1ull);
 }
 
+// The integrator state of one record.
+// (push_record loads it; push_loaded takes it from a caller that loaded it early.)
 // Laser + Boris kick (FP32 increment) + FP64 drift + boundary for record i
 // with Coulomb field (ex, ey, ez); writes x, u and the next j-stream entry.
 // DIAG (diagnostic steps): also the record's diagnostics at t_n, as
 // k_diag_partial forms them from the same kick: status (1 active, 2
 // non-finite; inactive records are left at 0), kinetic energy at the
 // integer-time u = u^{n-1/2} + du/2, potential energy w z phi / 2, momentum.
+struct RecState {
+  double X, Y, Z, Ux, Uy, Uz;
+  float qm;
+};
+
+__device__ __forceinline__ RecState load_state(const StepArgs& a, long long i) {
+  return {a.x[i], a.y[i], a.z[i], a.ux[i], a.uy[i], a.uz[i], a.qm[i]};
+}
+
 template <bool DET, bool DIAG = false>
-__device__ __forceinline__ void push_record(const StepArgs& a, const ClusterDev& c, long long i,
-                                            double ex, double ey, double ez, const float* las,
-                                            double t_next, const float4* cur, float4* nxt,
-                                            double phi = 0.0) {
-  if (!MD_IN_RANGE(a.err, i, c.off, c.off + c.n_pad)) return;
-  double X = a.x[i], Y = a.y[i], Z = a.z[i];
-  double Ux = a.ux[i], Uy = a.uy[i], Uz = a.uz[i];
-  const float h = 0.5f * static_cast<float>(c.dt) * a.qm[i];
+__device__ __forceinline__ void push_loaded(const StepArgs& a, const ClusterDev& c, long long i,
+                                            const RecState& st, double ex, double ey, double ez,
+                                            const float* las, double t_next, const float4* cur,
+                                            float4* nxt, double phi = 0.0) {
+  double X = st.X, Y = st.Y, Z = st.Z;
+  double Ux = st.Ux, Uy = st.Uy, Uz = st.Uz;
+  const float h = 0.5f * static_cast<float>(c.dt) * st.qm;
   float dux, duy, duz;
   boris_increment(static_cast<float>(Ux), static_cast<float>(Uy), static_cast<float>(Uz),
                   static_cast<float>(ex) + las[0], static_cast<float>(ey) + las[1],
@@ -1162,8 +1176,8 @@ __device__ __forceinline__ void push_record(const StepArgs& a, const ClusterDev&
     Z = wrap_periodic(Z, c.box);
   }
   if constexpr (DET) {
-    if (c.det_nbins > 0 && a.det_hist && a.qm[i] > 0.0f)
-      detect(a.det_hist, a.det_crossed, c, i, a.x[i], a.y[i], a.z[i], X, Y, Z, Ux, Uy, Uz,
+    if (c.det_nbins > 0 && a.det_hist && st.qm > 0.0f)
+      detect(a.det_hist, a.det_crossed, c, i, st.X, st.Y, st.Z, X, Y, Z, Ux, Uy, Uz,
              a.mass[i], a.err);
   }
   a.x[i] = X;
@@ -1181,6 +1195,15 @@ __device__ __forceinline__ void push_record(const StepArgs& a, const ClusterDev&
     v.z = static_cast<float>(Uz);
     a.vel[i] = v;
   }
+}
+
+template <bool DET, bool DIAG = false>
+__device__ __forceinline__ void push_record(const StepArgs& a, const ClusterDev& c, long long i,
+                                            double ex, double ey, double ez, const float* las,
+                                            double t_next, const float4* cur, float4* nxt,
+                                            double phi = 0.0) {
+  if (!MD_IN_RANGE(a.err, i, c.off, c.off + c.n_pad)) return;
+  push_loaded<DET, DIAG>(a, c, i, load_state(a, i), ex, ey, ez, las, t_next, cur, nxt, phi);
 }
 
 // Sum of the n partials p[k stride] (C components each, k = 0 .. n - 1) of

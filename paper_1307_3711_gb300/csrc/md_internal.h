@@ -48,6 +48,11 @@ cudaError_t launch_mut_step(const MutArgs& a, int grid, bool det, bool pot, bool
 // (resident CTAs per SM of the pair kernel; block: records per i-block)
 cudaError_t mut_blocks_per_sm(int block, bool pot, bool mi, int* out);
 
+// One step of clusters of a few thousand records (md_small.cu): n_blks CTAs of
+// `targets` (16 or 32) targets; blks may be nullptr for a single cluster.
+cudaError_t launch_small_step(const StepArgs& a, const SmallBlk* blks, int n_blks, int targets,
+                              bool det, bool pot, cudaStream_t s);
+
 // Field (and potential) at nt targets from ns sources (FP32/Kahan direct sum),
 // with the sources split as a.nseg / a.seg_len / a.part say.
 cudaError_t launch_field(const FieldArgs& a, bool potential, cudaStream_t s);

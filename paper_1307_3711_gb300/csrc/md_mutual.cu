@@ -10,8 +10,8 @@
 // 13.2 ms per step at 200k records), so only fewer operands make a large step
 // faster.  Here one evaluation of the displacement and of 1/r^3 feeds the sums
 // of both records: 34 operands for four interactions, 36 cycles with the
-// shuffles: 9.6 ms at 200k records, 2.50 against 3.41 at 100k, 0.71 against
-// 0.91 at 50k, 0.150 against 0.20 at 19k.  (Unrolling by 1, 2 or 8 steps,
+// shuffles: 9.5 ms at 200k records, 2.46 against 3.41 at 100k, 0.67 against
+// 0.91 at 50k, 0.123 against 0.20 at 19k.  (Unrolling by 1, 2 or 8 steps,
 // prefetching the next source, one scalar instead of two packed partial sums
 // of a source, tiles of 256 sources and 6, 10, 14 or 16 targets per thread
 // were slower or no faster.)
@@ -28,7 +28,7 @@
 //   * The four warps' sums of a source are added and written to `jpart`, one
 //     FP32 value per component, block I and later record; the targets' sums
 //     (Kahan, folded once per tile) go to `ipart` per work unit.  k_mut_push
-//     adds a record's partials in order in FP64 and pushes it.  The traffic is
+//     adds a record's partials in a fixed order and pushes it.  The traffic is
 //     12 bytes per i-block and later record each way: 0.24 GB written and read
 //     per step at 200k records, 1 % of its time.
 //   * Work units are runs of tiles of one i-block, cut into equal shares of the
@@ -432,8 +432,9 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
           }
         }
       }
-      // this unit's partial field at its targets, -(s - c) of sum Q (x_j - x_i)/r^3
-      double* ip = a.ipart + (POT ? 4 : 3) * static_cast<long long>(kBlock) * u;
+      // this unit's Kahan sums and compensations at its targets (of
+      // sum Q (x_j - x_i)/r^3, and of the potential)
+      float2* ip = a.ipart + (POT ? 4 : 3) * static_cast<long long>(kBlock) * u;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int k = tid + r * kMutThreads;
@@ -443,8 +444,7 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
           float s0, s1, c0, c1;
           f2_unpack(ks.v[kc][r >> 1][tid], s0, s1);
           f2_unpack(ks.v[cc][r >> 1][tid], c0, c1);
-          const double v = (r & 1) ? static_cast<double>(s1) - c1 : static_cast<double>(s0) - c0;
-          __stcg(ip + c * kBlock + k, c < 3 ? -v : v);
+          __stcg(ip + c * kBlock + k, (r & 1) ? make_float2(s1, c1) : make_float2(s0, c0));
         }
       }
       __syncthreads();  // s_un, s_c and ks are rewritten by the next unit
@@ -452,82 +452,101 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
   }
 }
 
-// The push of every record: its partials in a fixed order (the units of its
-// i-block, then the earlier blocks' mutual sums), laser, kick, drift.  Runs
-// after k_mut_pairs, whose ticket it resets; its last CTA advances the step.
-constexpr int kPushThreads = 128;
+// The push of every record: its partials in a fixed order, laser, kick, drift.
+// Runs after k_mut_pairs, whose ticket it resets; its last CTA advances the
+// step.  A CTA takes 32 records: warp w adds the work units and the earlier
+// blocks' rows w, w + 8, ... in Kahan-compensated FP32, and the first warp adds
+// the eight sums in FP64 and pushes.  136 us at 200k records and 14 at 19k
+// (0.3 GB of partials at 200k); one thread per record with FP64 adds, which the
+// narrow FP64 pipe bounds, took 240 and 32.
+constexpr int kPushRec = 32;
+constexpr int kPushWarps = 8;
 
 template <bool DET, bool POT>
-__global__ void __launch_bounds__(kPushThreads) k_mut_push(const MutArgs a) {
+__global__ void __launch_bounds__(32 * kPushWarps) k_mut_push(const MutArgs a) {
+  constexpr int C = POT ? 4 : 3;
+  __shared__ double s_e[C][kPushWarps][kPushRec];
   __shared__ ClusterDev s_c;
   __shared__ float s_las[6];
-  __shared__ MutBlk s_b;
   const long long step = __ldcg(a.s.step);
   // a wait of k_mut_pairs ran out: its partials are incomplete, push nothing
   if (__ldcg(a.s.err) & kErrTimeout) return;
-  const int per = a.block / kPushThreads;
-  if (threadIdx.x == 0) {
-    s_b = a.blks[blockIdx.x / per];
-    s_c = a.s.cl[s_b.cluster];
-    laser_field(s_c, s_c.t0 + static_cast<double>(step) * s_c.dt, s_las);
+  const int per = a.block / kPushRec;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const MutBlk b = a.blks[blockIdx.x / per];
+  const ClusterDev* cl = a.s.cl + b.cluster;
+  const int n_pad = cl->n_pad;
+  const int k = static_cast<int>(blockIdx.x % per) * kPushRec + lane;  // in the block
+  const long long j = static_cast<long long>(b.block) * a.block + k;   // in the cluster
+  const bool live = j < n_pad;
+  RecState st;
+  if (warp == kPushWarps - 1) {
+    if (lane == 0) {
+      s_c = *cl;
+      laser_field(s_c, s_c.t0 + static_cast<double>(step) * s_c.dt, s_las);
+    }
+    __syncwarp();
   }
-  __syncthreads();
-  const int k = static_cast<int>(blockIdx.x % per) * kPushThreads + threadIdx.x;  // in the block
-  const long long j = static_cast<long long>(s_b.block) * a.block + k;           // in the cluster
-  if (j < s_c.n_pad) {
-    double e[POT ? 4 : 3];
-    constexpr int C = POT ? 4 : 3;
+  if (live) {
+    if (warp == 0) st = load_state(a.s, cl->off + j);
+    float s[3] = {0.f, 0.f, 0.f}, c[3] = {0.f, 0.f, 0.f};
+    double ph = 0.0;
+    const float2* ip = a.ipart + C * static_cast<long long>(a.block) * b.unit0 + k;
+#pragma unroll 2
+    for (int p = warp; p < b.units; p += kPushWarps) {
+      const float2* q = ip + static_cast<long long>(p) * C * a.block;
 #pragma unroll
-    for (int c = 0; c < C; ++c) e[c] = 0.0;
-    const double* ip = a.ipart + C * static_cast<long long>(a.block) * s_b.unit0 + k;
-    for (int p = 0; p < s_b.units; ++p, ip += C * a.block) {
-#pragma unroll
-      for (int c = 0; c < C; ++c) e[c] += __ldcg(ip + c * a.block);
+      for (int m = 0; m < 3; ++m) {
+        // the units sum x_j - x_i: their field has the other sign
+        const float2 v = __ldcg(q + m * a.block);
+        kahan_add(s[m], c[m], -v.x);
+        kahan_add(s[m], c[m], v.y);
+      }
+      if constexpr (POT) {
+        const float2 v = __ldcg(q + 3 * a.block);
+        ph += static_cast<double>(v.x) - v.y;
+      }
     }
     // row I: the records after block I, `later` of them, three components apart
-    long long later = s_c.n_pad - a.block;
-    const float* jr = a.jpart + 3 * s_b.jbase;
-    const double* pr = POT ? a.jphi + s_b.jbase : nullptr;
-    long long col = j - a.block;
-    constexpr int kFly = 8;  // rows in flight
-    for (int I0 = 0; I0 < s_b.block; I0 += kFly) {
-      float v[kFly][3];
-      double ph[POT ? kFly : 1];
+#pragma unroll 4
+    for (int I = warp; I < b.block; I += kPushWarps) {
+      const long long skipped = static_cast<long long>(I) * n_pad -
+                                static_cast<long long>(a.block) * I * (I + 1) / 2;
+      const long long later = n_pad - static_cast<long long>(I + 1) * a.block;
+      const long long col = j - static_cast<long long>(I + 1) * a.block;
+      const float* row = a.jpart + 3 * (b.jbase + skipped) + col;
 #pragma unroll
-      for (int q = 0; q < kFly; ++q) {
-        if (I0 + q < s_b.block) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) v[q][c] = __ldcg(jr + c * later + col);
-          if constexpr (POT) ph[q] = __ldcg(pr + col);
-          jr += 3 * later;
-          if constexpr (POT) pr += later;
-          later -= a.block;
-          col -= a.block;
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < kFly; ++q) {
-        if (I0 + q < s_b.block) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) e[c] += static_cast<double>(v[q][c]);
-          if constexpr (POT) e[3] += ph[q];
-        }
-      }
+      for (int m = 0; m < 3; ++m) kahan_add(s[m], c[m], __ldcg(row + m * later));
+      if constexpr (POT) ph += __ldcg(a.jphi + b.jbase + skipped + col);
     }
-    const float4* __restrict__ cur = (step & 1) ? a.s.posq1 : a.s.posq0;
-    float4* __restrict__ nxt = (step & 1) ? a.s.posq0 : a.s.posq1;
-    const double t_next = s_c.t0 + static_cast<double>(step + 1) * s_c.dt;
-    const long long i = s_c.off + j;
-    if constexpr (POT) {
-      // the potential without the record's own term
-      const double ph = e[3] - static_cast<double>(cur[i].w * rsqrt_mufu(s_c.eps2));
-      push_record<DET, true>(a.s, s_c, i, e[0], e[1], e[2], s_las, t_next, cur, nxt, ph);
-    } else {
-      push_record<DET>(a.s, s_c, i, e[0], e[1], e[2], s_las, t_next, cur, nxt);
-    }
+#pragma unroll
+    for (int m = 0; m < 3; ++m) s_e[m][warp][lane] = static_cast<double>(s[m]) - c[m];
+    if constexpr (POT) s_e[3][warp][lane] = ph;
   }
-  if (threadIdx.x == 0) {
-    const unsigned prev = atomicAdd(a.s.done, 1u);
+  __syncthreads();
+  if (warp == 0) {
+    if (live) {
+      double e[C];
+#pragma unroll
+      for (int m = 0; m < C; ++m) {
+        e[m] = 0.0;
+#pragma unroll
+        for (int w = 0; w < kPushWarps; ++w) e[m] += s_e[m][w][lane];
+      }
+      const float4* __restrict__ cur = (step & 1) ? a.s.posq1 : a.s.posq0;
+      float4* __restrict__ nxt = (step & 1) ? a.s.posq0 : a.s.posq1;
+      const double t_next = s_c.t0 + static_cast<double>(step + 1) * s_c.dt;
+      const long long i = s_c.off + j;
+      if constexpr (POT) {
+        // the potential without the record's own term
+        const double phi = e[3] - static_cast<double>(cur[i].w * rsqrt_mufu(s_c.eps2));
+        push_loaded<DET, true>(a.s, s_c, i, st, e[0], e[1], e[2], s_las, t_next, cur, nxt, phi);
+      } else {
+        push_loaded<DET>(a.s, s_c, i, st, e[0], e[1], e[2], s_las, t_next, cur, nxt);
+      }
+    }
+  } else if (threadIdx.x == 32) {
+    const unsigned prev = atomicAdd(a.s.done, 1u);  // every warp here has read the step
     if (prev == gridDim.x - 1) {
       atomicExch(a.s.ticket, 0u);
       atomicExch(a.s.done, 0u);
@@ -575,13 +594,13 @@ cudaError_t launch_mut_step(const MutArgs& a, int grid, bool det, bool pot, bool
     return cudaErrorInvalidValue;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const unsigned g = static_cast<unsigned>(a.n_blks) * static_cast<unsigned>(a.block / kPushThreads);
+  const unsigned g = static_cast<unsigned>(a.n_blks) * static_cast<unsigned>(a.block / kPushRec);
   if (det)
-    k_mut_push<true, false><<<g, kPushThreads, 0, s>>>(a);
+    k_mut_push<true, false><<<g, 32 * kPushWarps, 0, s>>>(a);
   else if (pot)
-    k_mut_push<false, true><<<g, kPushThreads, 0, s>>>(a);
+    k_mut_push<false, true><<<g, 32 * kPushWarps, 0, s>>>(a);
   else
-    k_mut_push<false, false><<<g, kPushThreads, 0, s>>>(a);
+    k_mut_push<false, false><<<g, 32 * kPushWarps, 0, s>>>(a);
   return cudaGetLastError();
 }
 

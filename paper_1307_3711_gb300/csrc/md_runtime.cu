@@ -138,10 +138,14 @@ struct md_ctx {
   int* d_mut_first = nullptr;
   md::MutBlk* d_mut_blks = nullptr;
   int mut_shares = 0, mut_blks = 0, mut_grid = 0, mut_block = 0;
-  double* d_mut_ipart = nullptr;
+  float2* d_mut_ipart = nullptr;
   float* d_mut_jpart = nullptr;
   double* d_mut_jphi = nullptr;   // allocated by the first diagnostic step
   long long mut_jrecs = 0;        // records of all rows of jpart
+  // the step of a few thousand records (md_small.cu), while small_targets > 0
+  int small_targets = 0;
+  int small_ctas = 0;
+  md::SmallBlk* d_small_blks = nullptr;  // (more than one cluster)
 
   // ionization
   std::vector<md::IonDev> ion;
@@ -428,6 +432,9 @@ md::MutArgs mut_args(md_ctx* c) {
 // The kernels of one step of a context.
 cudaError_t launch_one_step(md_ctx* c, const md::KernelConfig& k, const md::StepArgs& a,
                             cudaStream_t s) {
+  if (c->small_targets)
+    return md::launch_small_step(a, c->d_small_blks, c->small_ctas, c->small_targets, c->det_on,
+                                 false, s);
   if (c->mut_on) return md::launch_mut_step(mut_args(c), c->mut_grid, c->det_on, false, c->any_mi, s);
   return launch_step_of(c, k, a, s);
 }
@@ -700,9 +707,12 @@ md_status configure(md_ctx* c, int cfg, int ctas_per_sm, int jsplit) {
   return MD_OK;
 }
 
-void mut_off(md_ctx* c) {
-  if (c->mut_on) destroy_graph(c);
+void auto_off(md_ctx* c) {
+  if (c->mut_on || c->small_targets) destroy_graph(c);
   c->mut_on = false;
+  c->small_targets = 0;
+  cudaFree(c->d_small_blks);
+  c->d_small_blks = nullptr;
   cudaFree(c->d_mut_units);
   cudaFree(c->d_mut_first);
   cudaFree(c->d_mut_blks);
@@ -730,13 +740,51 @@ constexpr long long kMutMinImageRecords = 11000;
 constexpr long long kMutBigRecords = 40000;
 constexpr long long kMutMinTiles = 2;
 
-// Sets up the step with each pair evaluated once, if the context can take it
-// (no ionizing cluster, no target slice, room for the partial sums); otherwise
-// the configured step kernel stays.
-md_status mut_configure(md_ctx* c) {
+// Pairs (records squared, summed over the clusters) up to which the small step
+// is taken: 24.6 us per step at 5000 records against 31 with each pair once,
+// 42.3 against 41.2 at 8000, 66 against 55 at 10000.
+constexpr double kSmallMaxPairs = 9.0e3 * 9.0e3;
+
+// The small step, if the context is that small: 16 or 32 targets per CTA,
+// whichever leaves the busiest SM fewer targets (equal: 32, whose CTAs stage
+// the sources half as often).
+md_status small_configure(md_ctx* c) {
+  double pairs = 0.0;
+  for (const md::ClusterDev& cl : c->cl) pairs += static_cast<double>(cl.n_pad) * cl.n_pad;
+  if (c->any_mi || pairs > kSmallMaxPairs) return MD_OK;
+  long long ctas[2] = {0, 0}, load[2];
+  for (int k = 0; k < 2; ++k) {
+    const long long per = k ? 32 : 16;
+    for (const md::ClusterDev& cl : c->cl) ctas[k] += (cl.n_pad + per - 1) / per;
+    load[k] = (ctas[k] + c->sm_count - 1) / c->sm_count * per;
+  }
+  const int pick = load[1] <= load[0] ? 1 : 0;
+  const int per = pick ? 32 : 16;
+  if (c->n_clusters > 1) {
+    std::vector<md::SmallBlk> blks;
+    for (int ci = 0; ci < c->n_clusters; ++ci)
+      for (int t = 0; t < c->cl[ci].n_pad; t += per) blks.push_back({ci, t});
+    MD_CUDA(dev_alloc(&c->d_small_blks, blks.size()));
+    MD_CUDA(cudaMemcpyAsync(c->d_small_blks, blks.data(), blks.size() * sizeof(md::SmallBlk),
+                            cudaMemcpyHostToDevice, c->stream));
+    MD_CUDA(cudaStreamSynchronize(c->stream));
+  }
+  destroy_graph(c);
+  c->small_ctas = static_cast<int>(ctas[pick]);
+  c->small_targets = per;
+  return MD_OK;
+}
+
+// Sets up the step that suits the context's size, if it can take it (no
+// ionizing cluster, no target slice): the small step, or each pair evaluated
+// once if there is room for the partial sums; otherwise the configured step
+// kernel stays.
+md_status auto_configure(md_ctx* c) {
   MD_CUDA(cudaStreamSynchronize(c->stream));
-  mut_off(c);
+  auto_off(c);
   if (c->any_ion || c->any_slice) return MD_OK;
+  const md_status small = small_configure(c);
+  if (small != MD_OK || c->small_targets) return small;
   for (int ci = 0; ci < c->n_clusters; ++ci)
     if (c->min_image[ci] && c->cl[ci].n < kMutMinImageRecords) return MD_OK;
   // 12 targets per thread (fewer shuffles and loads per pair) once the largest
@@ -749,7 +797,7 @@ md_status mut_configure(md_ctx* c) {
   if (bps < 1) return MD_OK;
   const long long slots = static_cast<long long>(bps) * c->sm_count;
   std::vector<md::MutBlk> blks;
-  long long jrecs = 0, weight = 0;
+  long long jrecs = 0, weight = 0, tiles = 0;
   for (int ci = 0; ci < c->n_clusters; ++ci) {
     const long long n = c->cl[ci].n_pad, nb = (n + B - 1) / B;
     const long long base = jrecs;
@@ -758,6 +806,7 @@ md_status mut_configure(md_ctx* c) {
       blks.push_back({ci, static_cast<int>(b), 0, 0, base});
       jrecs += std::max(0LL, n - (b + 1) * B);
       weight += md::kMutWeightOwn * own + md::kMutWeightPair * (nt - own);
+      tiles += nt;
     }
   }
   if (jrecs > kMutMaxRecs || blks.size() > (1u << 27)) return MD_OK;
@@ -765,12 +814,14 @@ md_status mut_configure(md_ctx* c) {
   // the work that is left.  The CTAs of an SM do not advance alike (one share
   // each, all equal: 10.8 ms per step at 200k records; eight rounds of equal
   // shares 9.8; these 9.6; half of what is left per round 10.2), and a share
-  // keeps at least kMutMinTiles tiles because each of its units writes a
-  // partial sum of every target of its block (19k records: 0.150 ms with 2,
-  // 0.165 with 3).
+  // keeps at least kMutMinTiles tiles, or a fortieth of a CTA's work, because
+  // each of its units writes a partial sum of every target of its block (19k
+  // records: 0.150 ms with 2, 0.165 with 3).
+  const long long min_tiles = std::max<long long>(
+      kMutMinTiles, weight / (md::kMutWeightPair * 40 * slots));
   std::vector<long long> cut;  // the shares' ends, in weight
   for (long long left = weight, at = 0; left > 0;) {
-    const long long w = std::max<long long>(kMutMinTiles * md::kMutWeightPair,
+    const long long w = std::max<long long>(min_tiles * md::kMutWeightPair,
                                             (3 * left + 8 * slots - 1) / (8 * slots));
     for (long long k = 0; k < slots && left > 0; ++k) {
       const long long take = std::min(left, w);
@@ -780,7 +831,11 @@ md_status mut_configure(md_ctx* c) {
     }
   }
   std::vector<md::MutUnit> units;
-  std::vector<int> first(cut.size() + 1, 0);
+  std::vector<int> first(1, 0);
+  // few tiles: one to a share, so that no CTA gets two while another has none
+  // (54.8 against 67.6 us per step at 10000 records, 193 against 212 at 25000,
+  // no difference at 36000)
+  const bool single = tiles <= 8 * slots;
   long long w = 0;
   size_t share = 0;
   for (md::MutBlk& bk : blks) {
@@ -789,18 +844,22 @@ md_status mut_configure(md_ctx* c) {
     const long long jrow = bk.jbase + b * n - B * (b * (b + 1) / 2);
     bk.unit0 = static_cast<int>(units.size());
     for (long long t = 0; t < nt; ++t) {
-      const size_t before = share;
-      while (share + 1 < cut.size() && w >= cut[share]) ++share;
-      if (t == 0 || share != before) {
+      bool next = single || (t == 0 && b == 0 && units.empty());
+      while (share + 1 < cut.size() && w >= cut[share]) {
+        ++share;
+        next = true;
+      }
+      if (next) first.push_back(0);
+      if (next || t == 0) {
         units.push_back({bk.cluster, bk.block, static_cast<int>(t), 0, jrow});
-        ++first[share + 1];
+        ++first.back();
       }
       ++units.back().nt;
       w += t < B / T ? md::kMutWeightOwn : md::kMutWeightPair;
     }
     bk.units = static_cast<int>(units.size()) - bk.unit0;
   }
-  const long long G = static_cast<long long>(cut.size());
+  const long long G = static_cast<long long>(first.size()) - 1;
   for (size_t i = 1; i < first.size(); ++i) first[i] += first[i - 1];
   cudaError_t e = dev_alloc(&c->d_mut_jpart, 3 * static_cast<size_t>(jrecs));
   if (e == cudaSuccess) e = dev_alloc(&c->d_mut_ipart, 4 * static_cast<size_t>(B) * units.size());
@@ -809,7 +868,7 @@ md_status mut_configure(md_ctx* c) {
   if (e == cudaSuccess) e = dev_alloc(&c->d_mut_blks, blks.size());
   if (e != cudaSuccess) {  // no room: the step kernel needs none of this
     cudaGetLastError();
-    mut_off(c);
+    auto_off(c);
     return MD_OK;
   }
   MD_CUDA(cudaMemcpyAsync(c->d_mut_units, units.data(), units.size() * sizeof(md::MutUnit),
@@ -1030,7 +1089,7 @@ void free_ctx(md_ctx* c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream);
   destroy_graph(c);
-  mut_off(c);
+  auto_off(c);
   cudaFree(c->d_cl);
   for (auto p : c->d_posq) cudaFree(p);
   for (auto p : c->d_x) cudaFree(p);
@@ -1508,7 +1567,7 @@ md_status populate(md_ctx* c, int32_t n_clusters, Fill fill, md_ctx** out) {
     }
   }
   md_status st = configure(c, default_config(c), 0, 0);
-  if (st == MD_OK) st = mut_configure(c);
+  if (st == MD_OK) st = auto_configure(c);
   if (st != MD_OK) {
     free_ctx(c);
     return st;
@@ -1841,7 +1900,7 @@ static md_status md_set_slice_body(md_ctx* c, int32_t cluster, int64_t i_begin, 
     any = any || c->slice_b[ci] > 0 || c->slice_e[ci] < c->cl[ci].n_pad;
   c->any_slice = any;
   const md_status st = configure(c, c->cfg, c->ctas_per_sm, c->jsplit);
-  return st == MD_OK && !c->forced ? mut_configure(c) : st;
+  return st == MD_OK && !c->forced ? auto_configure(c) : st;
 }
 
 md_status md_set_slice(md_ctx* c, int32_t cluster, int64_t i_begin, int64_t i_end) {
@@ -2047,7 +2106,7 @@ static md_status md_step_diag_body(md_ctx* c, md_diag* out) {
   if (!c->d_diag_rec) MD_CUDA(dev_alloc(&c->d_diag_rec, 6 * nt));
   if (c->mut_on) {
     if (!c->d_mut_jphi) MD_CUDA(dev_alloc(&c->d_mut_jphi, static_cast<size_t>(c->mut_jrecs)));
-  } else if (c->nseg_used > 1 && c->part_phi_seg < c->nseg_used) {
+  } else if (!c->small_targets && c->nseg_used > 1 && c->part_phi_seg < c->nseg_used) {
     cudaFree(c->d_part_phi);
     c->d_part_phi = nullptr;
     MD_CUDA(dev_alloc(&c->d_part_phi, static_cast<size_t>(c->nseg_used) * nt));
@@ -2063,6 +2122,9 @@ static md_status md_step_diag_body(md_ctx* c, md_diag* out) {
     md::MutArgs ma = mut_args(c);
     ma.s = a;
     MD_CUDA(md::launch_mut_step(ma, c->mut_grid, false, true, false, c->stream));
+  } else if (c->small_targets) {
+    MD_CUDA(md::launch_small_step(a, c->d_small_blks, c->small_ctas, c->small_targets, false, true,
+                                  c->stream));
   } else {
     MD_CUDA(k.launch_step_pot(a, c->grid, c->stream));
   }
@@ -2205,7 +2267,7 @@ static md_status md_set_tuning_body(md_ctx* c, const md_tuning* t) {
       const md_status st = configure(c, i, t->ctas_per_sm, t->jsplit);
       if (st == MD_OK) {
         c->forced = true;
-        mut_off(c);
+        auto_off(c);
       }
       return st;
     }
@@ -2337,8 +2399,8 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   cudaMemcpyAsync(&step0, c->d_step, sizeof(step0), cudaMemcpyDeviceToHost, s);
   cudaStreamSynchronize(s);
   const int cfg0 = c->cfg, cps0 = c->ctas_per_sm, js0 = c->jsplit;
-  const bool mut0 = c->mut_on;
-  mut_off(c);
+  const bool auto0 = c->mut_on || c->small_targets;
+  auto_off(c);
   int n = 0;
   const md::KernelConfig* cfgs = md::step_configs(&n);
   cudaEvent_t e0, e1;
@@ -2350,11 +2412,11 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   std::vector<double> by_cfg(static_cast<size_t>(n), -1.0);
   // one trial: configuration i with source split js, timed over `steps`
   // steps from the saved state (restored afterwards)
-  // (i < 0: the step with each pair evaluated once)
-  bool best_mut = false;
+  // (i < 0: the step that auto_configure sets up)
+  bool best_auto = false;
   auto trial = [&](int i, int js) {
-    st = i < 0 ? mut_configure(c) : configure(c, i, 0, js);
-    if (st != MD_OK || (i < 0 && !c->mut_on)) return;
+    st = i < 0 ? auto_configure(c) : configure(c, i, 0, js);
+    if (st != MD_OK || (i < 0 && !c->mut_on && !c->small_targets)) return;
     st = launch_steps_direct(c, 1);  // warm-up
     if (st != MD_OK) return;
     cudaEventRecord(e0, s);
@@ -2367,7 +2429,7 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
     if (i >= 0 && (by_cfg[i] < 0.0 || per < by_cfg[i])) by_cfg[i] = per;
     if (per < best) {
       best = per;
-      best_mut = i < 0;
+      best_auto = i < 0;
       if (i >= 0) {
         best_cfg = i;
         best_js = js;
@@ -2406,11 +2468,11 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   release();
   if (st != MD_OK) {
     configure(c, cfg0, cps0, js0);
-    if (mut0) mut_configure(c);
+    if (auto0) auto_configure(c);
     return st;
   }
-  if (!best_mut) mut_off(c);
-  c->forced = !best_mut;
+  if (!best_auto) auto_off(c);
+  c->forced = !best_auto;
   return configure(c, best_cfg, 0, best_js);
 }
 

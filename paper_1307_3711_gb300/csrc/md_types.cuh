@@ -159,9 +159,15 @@ struct MutArgs {
   const MutBlk* blks;
   int n_blks;
   int block;      // records per i-block
-  double* ipart;  // [unit][3, or 4 with the potential][block]
+  float2* ipart;  // [unit][3, or 4 with the potential][block]: Kahan sum, compensation
   float* jpart;   // per block: [3][records after the block]
   double* jphi;   // per block: [records after the block] (diagnostic steps)
+};
+
+// One CTA of the small step (md_small.cu): its cluster and first target.
+struct SmallBlk {
+  int cluster;
+  int t0;
 };
 
 // Cell list of the electrons near the ions, for the local moments of the

@@ -1,8 +1,9 @@
-"""The step that evaluates each pair of records once (contexts whose kernel
-configuration is not forced): record counts around its i-blocks, tiles and
-chunks, one and many charges per block, several clusters, the diagnostic and
-the minimum-image twin, against the FP64 oracle and against the step kernel
-that sums every pair for either record."""
+"""The steps of contexts whose kernel configuration is not forced (the small
+step, and the step that evaluates each pair of records once): record counts
+around their target groups, i-blocks, tiles and chunks, one and many charges
+per block, several clusters, the diagnostic and the minimum-image twin, against
+the FP64 oracle and against the step kernel that sums every pair for either
+record."""
 import os
 
 import numpy as np
@@ -58,7 +59,8 @@ def _kick(md, recs, forced=None, **kw):
 
 
 @pytest.mark.parametrize("charges", ["species", "one", "mixed"])
-@pytest.mark.parametrize("n", [1, 2, 16, 127, 129, 1023, 1024, 1025, 1041, 2049, 3071, 5000])
+@pytest.mark.parametrize("n", [1, 2, 16, 17, 33, 1023, 1025, 4095, 4097, 8995, 9217, 10241,
+                               11279])
 def test_kick_follows_oracle_around_block_and_tile_edges(md, n, charges):
     recs = _gas(n, charges, n)
     x, u, z, mass, w = recs
@@ -85,10 +87,11 @@ def test_large_blocks_follow_oracle(md, n):
     assert summary(force_error(got[idx], e64))["p99"] <= FORCE_P99
 
 
-def test_clusters_of_one_launch_are_independent(md):
+@pytest.mark.parametrize("largest", [3000, 9600])
+def test_clusters_of_one_launch_are_independent(md, largest):
     """Uneven clusters together and alone: the same kicks to FP32 order."""
     sets = [_gas(n, ch, 50 + n) for n, ch in
-            ((700, "mixed"), (4100, "species"), (1, "one"), (2100, "one"), (9000, "species"))]
+            ((700, "mixed"), (4100, "species"), (1, "one"), (1040, "one"), (largest, "species"))]
     with md.Context([_cfg(md) for _ in sets], [md.HostParticles(*s) for s in sets]) as ctx:
         ctx.step(1)
         together = [ctx.get_particles(k).u - sets[k][1] for k in range(len(sets))]
@@ -100,7 +103,7 @@ def test_clusters_of_one_launch_are_independent(md):
         assert np.abs(du - alone).max() <= 1e-5 * scale
 
 
-@pytest.mark.parametrize("n,charges", [(1500, "mixed"), (5000, "species"), (45000, "species")])
+@pytest.mark.parametrize("n,charges", [(1500, "mixed"), (5000, "species"), (9300, "mixed"), (45000, "species")])
 def test_diagnostic_step_and_repeats(md, n, charges):
     """md_step_diag takes the same step, bit for bit, as md_step and reports
     the diagnostics at its start; a second context repeats the bits."""
