@@ -601,6 +601,8 @@ void equal_shares(md_ctx* c, long long per, int tile, long long G, std::vector<m
   plan_shares(blks, tile, G, units, first, max_parts);
 }
 
+int default_config(md_ctx* c);
+
 // Work units (cluster, i-block, source piece) and their shares.  jsplit < 0
 // without ionizing clusters: equal shares, -jsplit per resident CTA.
 // Otherwise every i-block's sources are split into segments (jsplit of them,
@@ -631,7 +633,20 @@ md_status configure(md_ctx* c, int cfg, int ctas_per_sm, int jsplit) {
     for (int ci = 0; ci < c->n_clusters; ++ci)
       ib += static_cast<int>((c->cl[ci].n_pad + per - 1) / per);
   } else {
-    const int S = jsplit > 0 ? jsplit : choose_split(c, per, k.tile, slots);
+    // the default configuration of a context with ionization takes the split
+    // of its scalar twin (the same i-blocks and tiles), and so its bits
+    long long split_slots = slots;
+    if (jsplit == 0 && ctas_per_sm == 0 && !c->forced && cfg == default_config(c) && k.packed) {
+      const md::KernelConfig* twin = nullptr;
+      for (int i = 0; i < ncfg; ++i)
+        if (cfgs[i].threads == k.threads && cfgs[i].r == k.r && cfgs[i].tile == k.tile &&
+            !cfgs[i].packed)
+          twin = &cfgs[i];
+      int tb = 0;
+      if (twin) MD_CUDA(blocks_per_sm_of(c, *twin, &tb));
+      if (tb > 0) split_slots = static_cast<long long>(tb) * c->sm_count;
+    }
+    const int S = jsplit > 0 ? jsplit : choose_split(c, per, k.tile, split_slots);
     jsplit = std::max(jsplit, 0);
     struct Work {
       long long cost;
@@ -888,13 +903,18 @@ md_status auto_configure(md_ctx* c) {
   return MD_OK;
 }
 
-// Default before autotuning: 128 threads x 4 i-particles per thread, scalar.
+// Default before autotuning: 128 threads x 4 i-particles per thread, tile 512;
+// packed in contexts with ionization and no image forces (the scalar kernel's
+// bits, split as for it: 60.7 against 65.9 ms per step at 425k live records),
+// scalar otherwise.
 int default_config(md_ctx* c) {
-  (void)c;
+  const bool packed = c->any_ion && !c->any_mi;
   int ncfg = 0;
   const md::KernelConfig* cfgs = md::step_configs(&ncfg);
   for (int i = 0; i < ncfg; ++i)
-    if (cfgs[i].threads == 128 && cfgs[i].r == 4 && !cfgs[i].packed) return i;
+    if (cfgs[i].threads == 128 && cfgs[i].r == 4 && cfgs[i].tile == 512 &&
+        cfgs[i].packed == (packed ? 1 : 0))
+      return i;
   return 0;
 }
 
@@ -2264,11 +2284,13 @@ static md_status md_set_tuning_body(md_ctx* c, const md_tuning* t) {
         (t->min_blocks < 0 || cfgs[i].min_blocks == t->min_blocks)) {
       if (t->ctas_per_sm < 0) return fail(MD_ERR_ARG, "ctas_per_sm < 0");
       MD_CUDA(cudaStreamSynchronize(c->stream));
+      const bool was = c->forced;
+      c->forced = true;
       const md_status st = configure(c, i, t->ctas_per_sm, t->jsplit);
-      if (st == MD_OK) {
-        c->forced = true;
+      if (st == MD_OK)
         auto_off(c);
-      }
+      else
+        c->forced = was;
       return st;
     }
   }
@@ -2399,8 +2421,9 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   cudaMemcpyAsync(&step0, c->d_step, sizeof(step0), cudaMemcpyDeviceToHost, s);
   cudaStreamSynchronize(s);
   const int cfg0 = c->cfg, cps0 = c->ctas_per_sm, js0 = c->jsplit;
-  const bool auto0 = c->mut_on || c->small_targets;
+  const bool auto0 = c->mut_on || c->small_targets, forced0 = c->forced;
   auto_off(c);
+  c->forced = true;  // every trial takes its own split
   int n = 0;
   const md::KernelConfig* cfgs = md::step_configs(&n);
   cudaEvent_t e0, e1;
@@ -2467,13 +2490,15 @@ static md_status md_autotune_body(md_ctx* c, int32_t steps, double* times_ms, in
   cudaEventDestroy(e1);
   release();
   if (st != MD_OK) {
+    c->forced = forced0;
     configure(c, cfg0, cps0, js0);
     if (auto0) auto_configure(c);
     return st;
   }
   if (!best_auto) auto_off(c);
+  st = configure(c, best_cfg, 0, best_js);
   c->forced = !best_auto;
-  return configure(c, best_cfg, 0, best_js);
+  return st;
 }
 
 md_status md_autotune(md_ctx* c, int32_t steps, double* times_ms, int32_t cap) {
