@@ -171,43 +171,55 @@ constexpr double kLotzA = 4.5e-14;               // cm^2 eV^2
 
 // ---------------------------------------------------------------- rates ---
 
-// E1(x) = int_x^inf e^-t/t dt: power series up to 1, even continued fraction
-// (modified Lentz) beyond.
-__device__ inline double expint_e1(double x) {
-  if (!(x > 0.0)) return __longlong_as_double(0x7ff0000000000000LL);  // +inf
-  if (x <= 1.0) {
-    double sum = 0.0, term = 1.0;
-    for (int k = 1; k < 60; ++k) {
-      term *= -x / k;
-      const double add = -term / k;
-      sum += add;
-      if (fabs(add) < 1e-18 * fabs(sum)) break;
-    }
-    return -kEulerGamma - log(x) + sum;
-  }
-  const double tiny = 1e-300;
-  double b = x + 1.0, c = 1.0 / tiny, d = 1.0 / b, h = d;
-  for (int i = 1; i < 300; ++i) {
-    const double an = -static_cast<double>(i) * i;
-    b += 2.0;
-    d = 1.0 / (an * d + b);
-    c = b + an / c;
-    const double del = c * d;
-    h *= del;
-    if (fabs(del - 1.0) < 1e-16) break;
-  }
-  return h * exp(-x);
+// k k! of the power series of E1, as (-1)^(k+1) / (k k!).
+__host__ __device__ constexpr double e1_coeff(int k) {
+  double f = 1.0;
+  for (int i = 2; i <= k; ++i) f *= i;
+  return ((k & 1) ? 1.0 : -1.0) / (k * f);
 }
 
-// Static ADK rate (a.u.) at field F (a.u.), potential ip (a.u.), residual
-// charge Z: n* = Z/sqrt(2 ip), l* = n* - 1, l = m = 0.
-__device__ inline double adk_rate_au(double F, double ip, double Z) {
+template <int K>
+__device__ __forceinline__ double e1_series(double x) {  // sum_{k >= K} c_k x^(k-K)
+  if constexpr (K == 25)
+    return e1_coeff(25);
+  else
+    return fma(e1_series<K + 1>(x), x, e1_coeff(K));
+}
+
+// E1(x) = int_x^inf e^-t/t dt: the power series (25 terms) up to 2, beyond it
+// the even continued fraction e^-x / (x + 1 - 1/(x + 3 - 4/(x + 5 - ...))), its
+// n-th convergent from Wallis' recurrence for numerator and denominator (Jones
+// and Thron, Continued Fractions): no division per term, 90/x + 8 terms reach
+// the last bit.  On GB300's narrow FP64 pipe the divisions were the cost of
+// the rates: modified Lentz (two per term, up to 92 terms) took 160 us for a
+// few thousand ions, 336 us for 50000.  Largest relative error over [1e-6, 500]
+// against 40 digits: 7e-15 (Lentz and a series up to 1: 8e-15).
+__device__ inline double expint_e1(double x) {
+  if (!(x > 0.0)) return __longlong_as_double(0x7ff0000000000000LL);  // +inf
+  if (x <= 2.0) return -kEulerGamma - log(x) + x * e1_series<1>(x);
+  if (x > 745.0) return 0.0 * x;  // e^-x underflows (and NaN stays NaN)
+  const int n = static_cast<int>(90.0f / static_cast<float>(x)) + 8;
+  double a0 = 0.0, a1 = 1.0, b0 = 1.0, b1 = x + 1.0, b = b1, k2 = 1.0, dk = 3.0;
+  for (int k = 1; k < n; ++k) {  // k2 = k^2
+    b += 2.0;
+    const double a2 = fma(b, a1, -k2 * a0), b2 = fma(b, b1, -k2 * b0);
+    a0 = a1;
+    a1 = a2;
+    b0 = b1;
+    b1 = b2;
+    k2 += dk;
+    dk += 2.0;
+  }
+  return a1 / b1 * exp(-x);
+}
+
+// Static ADK rate (a.u.) of charge state z at field F (a.u.), l = m = 0:
+// C^2 Ip (2 F0/F)^(2 n* - 1) exp(-2 F0/(3 F)), with C^2 Ip, F0 and 2 n* - 1 of
+// each charge state from adk_tables.
+__device__ inline double adk_rate_au(const IonDev& io, double F, int z) {
   if (!(F > 0.0)) return 0.0;
-  const double ns = Z / sqrt(2.0 * ip);
-  const double ls = ns - 1.0;
-  const double c2 = pow(2.0, 2.0 * ns) / (ns * tgamma(ns + ls + 1.0) * tgamma(ns - ls));
-  const double f0 = pow(2.0 * ip, 1.5);
-  return c2 * ip * pow(2.0 * f0 / F, 2.0 * ns - 1.0) * exp(-2.0 * f0 / (3.0 * F));
+  const double f0 = io.adk_f0[z];
+  return io.adk_c[z] * pow(2.0 * f0 / F, io.adk_p[z]) * exp(-2.0 * f0 / (3.0 * F));
 }
 
 // Lotz rate coefficient (cm^3/s): sqrt(8/(pi m_e)) a q E1(P/T) / (P sqrt(T)).
@@ -221,8 +233,7 @@ __device__ inline double lotz_rate_cgs(double P, double T, double q) {
 // ne (cm^-3), te (eV).
 __device__ inline double rate_plain(const IonDev& io, double a_mag, int z, double ne, double te) {
   const double F = a_mag * kMeC2Ev * io.k_si / kFieldAu;
-  const double w_ofi = adk_rate_au(F, io.ip_ev[z] / kHartreeEv, static_cast<double>(z + 1)) /
-                       kTimeAu;
+  const double w_ofi = adk_rate_au(io, F, z) / kTimeAu;
   const double w_ci = ne > 0.0 ? ne * lotz_rate_cgs(io.ip_ev[z], te, io.q_outer[z]) : 0.0;
   return (w_ofi + w_ci) / io.omega;
 }

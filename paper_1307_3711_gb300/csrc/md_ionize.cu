@@ -387,9 +387,9 @@ __global__ void __launch_bounds__(THREADS) k_ion_field(const IonArgs a) {
 // r^2 + eps^2 of the j-stream positions against r_loc^2 + eps^2.
 
 // Field of the live records at the ions: CTA (x, y) sums segment y of the
-// live records for R x THREADS ions and writes its field to the scratch
-// slots of segment y (slots 0-2; slot 3, the weight of the local electrons,
-// is 0 here and filled for segment 0 by k_ion_moments).
+// live records for R x THREADS ions and writes its field to the scratch of
+// segment y.  4000 ions, 34000 live records: 168 us with 17 segments of whole
+// tiles (68 CTAs), 60 us with 112.
 template <int THREADS, int R, int TILE, int STAGES, bool PACK>
 __global__ void __launch_bounds__(THREADS) k_ion_field_sum(const IonArgs a) {
   __shared__ Stage<TILE, STAGES> sm;
@@ -409,7 +409,9 @@ __global__ void __launch_bounds__(THREADS) k_ion_field_sum(const IonArgs a) {
   n_live = n_live > a.ion.slot_base ? n_live : a.ion.slot_base;
   n_live = n_live < a.c.n_pad ? (n_live > 0 ? n_live : 0) : a.c.n_pad;
   const long long per_seg = (n_live + gridDim.y - 1) / gridDim.y;
-  const long long seg_len = (per_seg + TILE - 1) / TILE * TILE;
+  // whole tiles, unless the segments are that short
+  const long long unit = per_seg >= 4 * TILE ? TILE : 64;
+  const long long seg_len = (per_seg + unit - 1) / unit * unit;
   const long long j0 = static_cast<long long>(blockIdx.y) * seg_len;
   const long long ns = (j0 >= n_live) ? 0 : ((n_live - j0 < seg_len) ? n_live - j0 : seg_len);
   const long long t0 = static_cast<long long>(blockIdx.x) * (THREADS * R);
@@ -441,18 +443,18 @@ __global__ void __launch_bounds__(THREADS) k_ion_field_sum(const IonArgs a) {
   for (int r = 0; r < R; ++r) {
     const long long tt = t0 + threadIdx.x + r * THREADS;
     if (tt >= a.ion.n_ions) continue;
-    if (!MD_IN_RANGE(a.err, blockIdx.y, 0, kIonMaxSeg)) continue;
-    double* o = a.scratch + kIonScratch * (static_cast<long long>(blockIdx.y) * a.ion.n_ions + tt);
+    if (!MD_IN_RANGE(a.err, blockIdx.y, 0, kIonSumSeg)) continue;
+    const long long nn = a.ion.n_ions;
+    double* o = a.scratch + 3 * static_cast<long long>(blockIdx.y) * nn + tt;
     if constexpr (PACK) {
       o[0] = -(static_cast<double>(kahan_part(ks, 0, r)) - kahan_part(ks, 3, r));
-      o[1] = -(static_cast<double>(kahan_part(ks, 1, r)) - kahan_part(ks, 4, r));
-      o[2] = -(static_cast<double>(kahan_part(ks, 2, r)) - kahan_part(ks, 5, r));
+      o[nn] = -(static_cast<double>(kahan_part(ks, 1, r)) - kahan_part(ks, 4, r));
+      o[2 * nn] = -(static_cast<double>(kahan_part(ks, 2, r)) - kahan_part(ks, 5, r));
     } else {
       o[0] = -(static_cast<double>(acc.sx[r]) - acc.cx[r]);
-      o[1] = -(static_cast<double>(acc.sy[r]) - acc.cy[r]);
-      o[2] = -(static_cast<double>(acc.sz[r]) - acc.cz[r]);
+      o[nn] = -(static_cast<double>(acc.sy[r]) - acc.cy[r]);
+      o[2 * nn] = -(static_cast<double>(acc.sz[r]) - acc.cz[r]);
     }
-    o[3] = 0.0;
   }
 }
 
@@ -476,28 +478,27 @@ __device__ __forceinline__ bool cell_coords(float x, float y, float z, float inv
 // (An XOR of the coordinates times three odd constants, the first version,
 // put the mirror cells (0, y, z) and (0, -y, -z) of a cluster centred on the
 // origin into one bucket whenever y and z have the same power of 2.)
-__device__ __forceinline__ int cell_bucket(int x, int y, int z) {
+__device__ __forceinline__ int cell_bucket(int x, int y, int z, int bits) {
   constexpr unsigned long long kMask = (1ull << 21) - 1;
   const unsigned long long key = (static_cast<unsigned long long>(x) & kMask) |
                                  ((static_cast<unsigned long long>(y) & kMask) << 21) |
                                  ((static_cast<unsigned long long>(z) & kMask) << 42);
-  constexpr int kBits = 18;
-  static_assert(kCellBuckets == 1 << kBits, "bucket count");
-  return static_cast<int>((key * 0x9E3779B97F4A7C15ull) >> (64 - kBits));
+  return static_cast<int>((key * 0x9E3779B97F4A7C15ull) >> (64 - bits));
 }
 
-__device__ __forceinline__ int bucket_of(float x, float y, float z, float inv_h) {
+__device__ __forceinline__ int bucket_of(float x, float y, float z, float inv_h, int bits) {
   int cc[3];
   if (!cell_coords(x, y, z, inv_h, cc)) return -1;
-  return cell_bucket(cc[0], cc[1], cc[2]);
+  return cell_bucket(cc[0], cc[1], cc[2], bits);
 }
 
 __device__ __forceinline__ float cell_inv_h(const IonArgs& a) {
   return 1.0f / (1.01f * static_cast<float>(a.ion.r_loc));
 }
 
-// FILL = false: count the electrons (negative charge) of the live records per
-// cell; FILL = true: list each at its cell's start + an atomic fill counter.
+// FILL = false: count the electrons (negative charge) of the live records and
+// the ions per bucket; FILL = true: list them at their bucket's start + an
+// atomic fill counter.  One grid over the records, then over the ions.
 template <bool FILL>
 __global__ void __launch_bounds__(256) k_cell_list(const IonArgs a) {
   const long long step = __ldcg(a.step);
@@ -508,50 +509,32 @@ __global__ void __launch_bounds__(256) k_cell_list(const IonArgs a) {
   n_live = n_live < a.c.n_pad ? (n_live > 0 ? n_live : 0) : a.c.n_pad;
   const CellBuf cb = a.cells;
   const float inv_h = cell_inv_h(a);
-  for (long long j = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; j < n_live;
-       j += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const float4 p = cur[a.c.off + j];
-    if (!(p.w < 0.0f)) continue;
-    const int cell = bucket_of(p.x, p.y, p.z, inv_h);
-    if (cell < 0) continue;
-    if (!FILL) {
-      atomicAdd(cb.count + cell, 1);
-    } else {
-      const long long k = cb.start[cell] + atomicAdd(cb.fill + cell, 1);
-      if (!MD_IN_RANGE(a.err, k, 0, cb.capacity)) continue;
-      cb.rec[2 * k] = p;
-      cb.rec[2 * k + 1] = a.vel[a.c.off + j];
-    }
-  }
-}
-
-// FILL = false: count the ions per cell; FILL = true: list them in cell order.
-template <bool FILL>
-__global__ void __launch_bounds__(256) k_ion_cell_list(const IonArgs a) {
-  const long long step = __ldcg(a.step);
-  if (!pass_active(a, step)) return;
-  const float4* __restrict__ cur = (step & 1) ? a.posq1 : a.posq0;
-  const CellBuf cb = a.cells;
-  const float inv_h = cell_inv_h(a);
-  for (long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-       t < a.ion.n_ions; t += static_cast<long long>(gridDim.x) * blockDim.x) {
+  for (long long j = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+       j < n_live + a.ion.n_ions; j += static_cast<long long>(gridDim.x) * blockDim.x) {
+    const bool ion = j >= n_live;
+    const long long t = ion ? j - n_live : j;
     const float4 p = cur[a.c.off + t];
-    int cell = bucket_of(p.x, p.y, p.z, inv_h);
-    if (cell < 0) cell = 0;  // a position too far away to have a cell: its moments stay 0
-    if (!FILL) {
-      atomicAdd(cb.ion_count + cell, 1);
-    } else {
-      const long long k = cb.ion_start[cell] + atomicAdd(cb.ion_fill + cell, 1);
+    if (!ion && !(p.w < 0.0f)) continue;
+    int cell = bucket_of(p.x, p.y, p.z, inv_h, cb.bits);
+    if (cell < 0) {
+      if (!ion) continue;
+      cell = 0;  // a position too far away to have a cell: its moments stay 0
+    }
+    int* counter = FILL ? (ion ? cb.ion_fill : cb.fill) : (ion ? cb.ion_count : cb.count);
+    const int at = atomicAdd(counter + cell, 1);
+    if (!FILL) continue;
+    if (ion) {
+      const long long k = cb.ion_start[cell] + at;
       if (!MD_IN_RANGE(a.err, k, 0, a.ion.n_ions)) continue;
       cb.ion_list[k] = static_cast<int>(t);
+    } else {
+      const long long k = cb.start[cell] + at;
+      if (!MD_IN_RANGE(a.err, k, 0, cb.capacity)) continue;
+      cb.rec[k] = p;
+      cb.rec[cb.capacity + k] = a.vel[a.c.off + t];
     }
   }
 }
-
-// Exclusive scan of the kCellBuckets bucket counts into starts, in three
-// launches: each of kScanBlocks CTAs scans its 1024 buckets and records their
-// total; one CTA scans the totals; each CTA adds its offset.
-constexpr int kScanBlocks = kCellBuckets / 1024;
 
 __device__ __forceinline__ int block_excl_scan_1024(int v, int* s_warp, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -578,40 +561,81 @@ __device__ __forceinline__ int block_excl_scan_1024(int v, int* s_warp, int* tot
   return before;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_blocks(const IonArgs a, const int* count,
-                                                      int* start, int* totals) {
+// Exclusive scans of the bucket counts into starts: the electrons' (blockIdx.y
+// = 0) and the ions' (1).  Up to kScanOne buckets one CTA scans each, sixteen
+// or fewer buckets per thread; above, each CTA scans 1024 buckets and records
+// their total, one CTA per list scans the totals, and each CTA adds its offset.
+constexpr int kScanOne = 1 << 14;
+constexpr int kScanBlocks = kCellBuckets / 1024;
+
+__global__ void __launch_bounds__(1024) k_scan_one(const IonArgs a) {
   __shared__ int s_warp[32];
   const long long step = __ldcg(a.step);
   if (!pass_active(a, step)) return;
+  const int* count = blockIdx.y ? a.cells.ion_count : a.cells.count;
+  int* start = blockIdx.y ? a.cells.ion_start : a.cells.start;
+  constexpr int kPer = kScanOne / 1024;
+  const int n = 1 << a.cells.bits, per = (n + 1023) / 1024;
+  int v[kPer], sum = 0;
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    const int k = static_cast<int>(threadIdx.x) * per + q;
+    v[q] = (q < per && k < n) ? count[k] : 0;
+    sum += v[q];
+  }
+  int tot = 0;
+  int before = block_excl_scan_1024(sum, s_warp, &tot);
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    const int k = static_cast<int>(threadIdx.x) * per + q;
+    if (q < per && k < n) start[k] = before;
+    before += v[q];
+  }
+  if (threadIdx.x == 0) start[n] = tot;
+}
+
+__global__ void __launch_bounds__(1024) k_scan_blocks(const IonArgs a) {
+  __shared__ int s_warp[32];
+  const long long step = __ldcg(a.step);
+  if (!pass_active(a, step)) return;
+  const int* count = blockIdx.y ? a.cells.ion_count : a.cells.count;
+  int* start = blockIdx.y ? a.cells.ion_start : a.cells.start;
   const int k = blockIdx.x * 1024 + threadIdx.x;
   int tot = 0;
   start[k] = block_excl_scan_1024(count[k], s_warp, &tot);
-  if (threadIdx.x == 0) totals[blockIdx.x] = tot;
+  if (threadIdx.x == 0) a.cells.scan_tmp[blockIdx.y * kScanBlocks + blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_totals(const IonArgs a, int* totals, int* start) {
+__global__ void __launch_bounds__(1024) k_scan_totals(const IonArgs a, int blocks) {
   __shared__ int s_warp[32];
   const long long step = __ldcg(a.step);
   if (!pass_active(a, step)) return;
-  const int v = threadIdx.x < kScanBlocks ? totals[threadIdx.x] : 0;
+  int* totals = a.cells.scan_tmp + blockIdx.y * kScanBlocks;
+  const int v = static_cast<int>(threadIdx.x) < blocks ? totals[threadIdx.x] : 0;
   int tot = 0;
   const int before = block_excl_scan_1024(v, s_warp, &tot);
   __syncthreads();
-  if (threadIdx.x < kScanBlocks) totals[threadIdx.x] = before;
-  if (threadIdx.x == 0) start[kCellBuckets] = tot;
+  if (static_cast<int>(threadIdx.x) < blocks) totals[threadIdx.x] = before;
+  if (threadIdx.x == 0) (blockIdx.y ? a.cells.ion_start : a.cells.start)[blocks * 1024] = tot;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_add(const IonArgs a, const int* totals,
-                                                   int* start) {
+__global__ void __launch_bounds__(1024) k_scan_add(const IonArgs a) {
   const long long step = __ldcg(a.step);
   if (!pass_active(a, step)) return;
-  start[blockIdx.x * 1024 + threadIdx.x] += totals[blockIdx.x];
+  (blockIdx.y ? a.cells.ion_start : a.cells.start)[blockIdx.x * 1024 + threadIdx.x] +=
+      a.cells.scan_tmp[blockIdx.y * kScanBlocks + blockIdx.x];
 }
 
-cudaError_t launch_cell_scan(const IonArgs& a, const int* count, int* start, cudaStream_t s) {
-  k_scan_blocks<<<kScanBlocks, 1024, 0, s>>>(a, count, start, a.cells.scan_tmp);
-  k_scan_totals<<<1, 1024, 0, s>>>(a, a.cells.scan_tmp, start);
-  k_scan_add<<<kScanBlocks, 1024, 0, s>>>(a, a.cells.scan_tmp, start);
+cudaError_t launch_cell_scan(const IonArgs& a, cudaStream_t s) {
+  const int n = 1 << a.cells.bits;
+  if (n <= kScanOne) {
+    k_scan_one<<<dim3(1, 2), 1024, 0, s>>>(a);
+    return cudaGetLastError();
+  }
+  const unsigned blocks = static_cast<unsigned>(n / 1024);
+  k_scan_blocks<<<dim3(blocks, 2), 1024, 0, s>>>(a);
+  k_scan_totals<<<dim3(1, 2), 1024, 0, s>>>(a, static_cast<int>(blocks));
+  k_scan_add<<<dim3(blocks, 2), 1024, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -622,17 +646,22 @@ cudaError_t launch_cell_scan(const IonArgs& a, const int* count, int* start, cud
 // and added to 64-bit integer sums, so a total does not depend on which lane
 // took which electron, nor on the order of the listing.
 //
-// The ions are taken in bucket order, kMomIons per CTA.  The ions of one
+// The ions are taken in bucket order, a.mom_ions per CTA (fewer of them when
+// the cluster is small, so that the CTAs cover the SMs).  The ions of one
 // bucket mostly share one cell and so one set of 27 neighbour cells: for each
 // run of ions with the same bucket, the positions of the electrons listed in
 // those cells' buckets (a few thousand) are staged once in shared memory, and
 // each warp tests them against one ion at a time, 32 electrons per step.  An
 // ion of the run in another cell (two cells hashed to one bucket, or a
 // position without a cell) and a run whose electrons do not fit the stage
-// walk their own 27 buckets from global memory instead.
+// walk their own 27 buckets from global memory instead, four loads in flight.
+// Either way the electrons within r_loc are queued and their terms added 32 at
+// a time: in a dense plasma (6000 electrons in the 27 cells, 15 % of them
+// within r_loc) adding them where they are found kept a seventh of the lanes
+// busy.  4000 ions: 578 -> 75 us per pass, 50000: 1.54 -> 0.72 ms.
 constexpr int kMomThreads = 256;
 constexpr int kMomWarps = kMomThreads / 32;
-constexpr int kMomIons = 64;     // ions per CTA
+constexpr int kMomIons = 64;     // ions per CTA at most
 constexpr int kMomCap = 3072;    // staged electrons per run
 
 // v rounded to the nearest integer, ties to even, as a 64-bit integer, on
@@ -697,10 +726,10 @@ __device__ __forceinline__ bool near_loc(const float4 p, const float4 pi, float 
 // Lane l < 27 of a warp: the bucket of neighbour cell l of cc (offsets
 // l % 3 - 1, l / 3 % 3 - 1, l / 9 - 1), or -1 for a repeat of a lower lane's
 // bucket (cells may share one) and for lanes 27..31.
-__device__ __forceinline__ int neighbour_bucket(const int (&cc)[3], int lane) {
+__device__ __forceinline__ int neighbour_bucket(const int (&cc)[3], int lane, int bits) {
   int bk = -1;
   if (lane < 27)
-    bk = cell_bucket(cc[0] + lane % 3 - 1, cc[1] + (lane / 3) % 3 - 1, cc[2] + lane / 9 - 1);
+    bk = cell_bucket(cc[0] + lane % 3 - 1, cc[1] + (lane / 3) % 3 - 1, cc[2] + lane / 9 - 1, bits);
   bool first = lane < 27;
   for (int m = 0; m < 27; ++m) {
     const int bm = __shfl_sync(0xffffffffu, bk, m);
@@ -709,29 +738,74 @@ __device__ __forceinline__ int neighbour_bucket(const int (&cc)[3], int lane) {
   return first ? bk : -1;
 }
 
+// The electrons a warp has found within r_loc of its ion and not yet added.
+struct NearQueue {
+  int* q;  // [64] in shared memory
+  int n;   // queued (warp-uniform)
+
+  // queues electron idx of the lanes with nr; adds 32 once there are as many
+  __device__ __forceinline__ void push(bool nr, int idx, const float4* vel, const float4 ui,
+                                       int lane, MomSums& m) {
+    const unsigned mask = __ballot_sync(0xffffffffu, nr);
+    if (nr) q[n + __popc(mask & ((1u << lane) - 1u))] = idx;
+    n += __popc(mask);
+    if (n >= 32) {
+      __syncwarp();
+      m.add(vel[q[lane]], ui);
+      const int rest = n - 32 > lane ? q[32 + lane] : 0;
+      __syncwarp();
+      if (lane < n - 32) q[lane] = rest;
+      __syncwarp();
+      n -= 32;
+    }
+  }
+  __device__ __forceinline__ void flush(const float4* vel, const float4 ui, int lane, MomSums& m) {
+    __syncwarp();
+    if (lane < n) m.add(vel[q[lane]], ui);
+    __syncwarp();
+    n = 0;
+  }
+};
+
 // One warp: the sums of one ion over its 27 cells' buckets, read from global
 // memory (lane-strided over each bucket's electrons).
 __device__ __forceinline__ void moments_global(const CellBuf& cb, const float4 pi,
                                                const float4 ui, const int (&cc)[3], float eps2,
-                                               float rloc2e, int lane, MomSums& m, int* err) {
-  const int bk = neighbour_bucket(cc, lane);
-  unsigned todo = __ballot_sync(0xffffffffu, bk >= 0);
+                                               float rloc2e, int lane, MomSums& m, int* queue,
+                                               int* err) {
+  const int bk = neighbour_bucket(cc, lane, cb.bits);
+  const int k0 = bk >= 0 ? cb.start[bk] : 0;
+  const int cnt = bk >= 0 ? cb.start[bk + 1] - k0 : 0;
+  unsigned todo = __ballot_sync(0xffffffffu, cnt > 0);
+  NearQueue nq{queue, 0};
+  const float4* vel = cb.rec + cb.capacity;
+  constexpr int U = 4;
   while (todo) {
     const int src = __ffs(todo) - 1;
     todo &= todo - 1;
-    const int cell = __shfl_sync(0xffffffffu, bk, src);
-    const int k1 = cb.start[cell + 1];
-    for (int k = cb.start[cell] + lane; k < k1; k += 32)
-      if (MD_IN_RANGE(err, k, 0, cb.capacity) && near_loc(cb.rec[2 * k], pi, eps2, rloc2e))
-        m.add(cb.rec[2 * k + 1], ui);
+    const int b0 = __shfl_sync(0xffffffffu, k0, src), n = __shfl_sync(0xffffffffu, cnt, src);
+    if (!MD_IN_RANGE(err, b0 + n, 1, cb.capacity + 1)) continue;
+    for (int k = 0; k < n; k += 32 * U) {
+      float4 p[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kk = k + 32 * u + lane;
+        p[u] = __ldg(cb.rec + b0 + (kk < n ? kk : n - 1));
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int kk = k + 32 * u + lane;
+        if (k + 32 * u >= n) break;  // warp-uniform
+        nq.push(kk < n && near_loc(p[u], pi, eps2, rloc2e), b0 + kk, vel, ui, lane, m);
+      }
+    }
   }
+  nq.flush(vel, ui, lane, m);
 }
 
 __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
   __shared__ float4 s_pos[kMomCap];
   __shared__ int s_idx[kMomCap];
-  // per warp: the electrons found within r_loc and not yet added, so that
-  // the terms are added 32 at a time with every lane busy
   __shared__ int s_near[kMomWarps][64];
   __shared__ int s_bucket[kMomIons];
   __shared__ int s_bk[32], s_beg[32], s_cnt[32];
@@ -741,18 +815,19 @@ __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const CellBuf cb = a.cells;
   const float4* __restrict__ cur = (step & 1) ? a.posq1 : a.posq0;
+  const float4* vel = cb.rec + cb.capacity;
   const float eps2 = a.c.eps2;
   const float rloc2e = static_cast<float>(a.ion.r_loc * a.ion.r_loc) + eps2;
   const float inv_h = cell_inv_h(a);
-  const long long c0 = static_cast<long long>(blockIdx.x) * kMomIons;
-  const int nloc = static_cast<int>(a.ion.n_ions - c0 < kMomIons ? a.ion.n_ions - c0 : kMomIons);
+  const long long c0 = static_cast<long long>(blockIdx.x) * a.mom_ions;
+  const int nloc = static_cast<int>(a.ion.n_ions - c0 < a.mom_ions ? a.ion.n_ions - c0 : a.mom_ions);
   // each ion's bucket, as the ion listing computed it (no cell: bucket 0)
   if (tid < nloc) {
     const long long t = cb.ion_list[c0 + tid];
     int b = 0;
     if (MD_IN_RANGE(a.err, t, 0, a.ion.n_ions)) {
       const float4 p = cur[a.c.off + t];
-      b = bucket_of(p.x, p.y, p.z, inv_h);
+      b = bucket_of(p.x, p.y, p.z, inv_h, cb.bits);
       b = b < 0 ? 0 : b;
     }
     s_bucket[tid] = b;
@@ -770,7 +845,7 @@ __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
       staged = cell_coords(p0.x, p0.y, p0.z, inv_h, cc0);
     }
     if (staged && warp == 0) {
-      const int bk = neighbour_bucket(cc0, lane);
+      const int bk = neighbour_bucket(cc0, lane, cb.bits);
       const int cnt = bk >= 0 ? cb.start[bk + 1] - cb.start[bk] : 0;
       int inc = cnt;  // inclusive scan of the counts over the lanes
 #pragma unroll
@@ -784,7 +859,8 @@ __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
       if (lane == 31) s_total = inc;
     }
     __syncthreads();
-    staged = staged && s_total <= kMomCap;
+    // staging pays from three ions on (one would read its electrons once either way)
+    staged = staged && s_total <= kMomCap && r1 - r0 >= 3;
     if (staged) {
       for (int l = 0; l < 27; ++l) {
         const int cnt = s_cnt[l];
@@ -793,7 +869,7 @@ __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
         for (int k = tid; k < cnt; k += kMomThreads) {
           const bool ok = MD_IN_RANGE(a.err, k0 + k, 0, cb.capacity);
           // (an index out of range stages a position no ion is near)
-          s_pos[beg + k] = ok ? cb.rec[2 * (k0 + k)] : make_float4(3e38f, 3e38f, 3e38f, 0.f);
+          s_pos[beg + k] = ok ? cb.rec[k0 + k] : make_float4(3e38f, 3e38f, 3e38f, 0.f);
           s_idx[beg + k] = ok ? k0 + k : 0;
         }
       }
@@ -809,43 +885,29 @@ __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
       int cc[3];
       if (cell_coords(pi.x, pi.y, pi.z, inv_h, cc)) {
         if (staged && cc[0] == cc0[0] && cc[1] == cc0[1] && cc[2] == cc0[2]) {
-          int* q = s_near[warp];
-          int qn = 0;  // queued electrons (warp-uniform)
+          NearQueue nq{s_near[warp], 0};
           for (int k0 = 0; k0 < total; k0 += 32) {
             const int k = k0 + lane;
-            const bool nr = k < total && near_loc(s_pos[k], pi, eps2, rloc2e);
-            const unsigned mask = __ballot_sync(0xffffffffu, nr);
-            if (nr) q[qn + __popc(mask & ((1u << lane) - 1u))] = s_idx[k];
-            qn += __popc(mask);
-            if (qn >= 32) {
-              __syncwarp();
-              m.add(cb.rec[2 * q[lane] + 1], ui);
-              const int rest = qn - 32 > lane ? q[32 + lane] : 0;
-              __syncwarp();
-              if (lane < qn - 32) q[lane] = rest;
-              __syncwarp();
-              qn -= 32;
-            }
+            nq.push(k < total && near_loc(s_pos[k], pi, eps2, rloc2e), k < total ? s_idx[k] : 0,
+                    vel, ui, lane, m);
           }
-          __syncwarp();
-          if (lane < qn) m.add(cb.rec[2 * q[lane] + 1], ui);
-          __syncwarp();
+          nq.flush(vel, ui, lane, m);
         } else {
-          moments_global(cb, pi, ui, cc, eps2, rloc2e, lane, m, a.err);
+          moments_global(cb, pi, ui, cc, eps2, rloc2e, lane, m, s_near[warp], a.err);
         }
         m.warp_sum();
       }
       if (lane == 0) {
         constexpr double kScale = 1099511627776.0;  // 2^40
-        double* o = a.scratch + kIonScratch * t;  // segment 0
-        o[3] = static_cast<double>(m.W) / kScale;
-        o[4] = static_cast<double>(m.S0) / kScale;
-        o[5] = static_cast<double>(m.S1) / kScale;
-        o[6] = static_cast<double>(m.S2) / kScale;
-        o[7] = static_cast<double>(m.Q) / kScale;
-        o[8] = ui.x;
-        o[9] = ui.y;
-        o[10] = ui.z;
+        double* o = a.scratch + 3 * static_cast<long long>(a.nseg) * a.ion.n_ions + kIonMom * t;
+        o[0] = static_cast<double>(m.W) / kScale;
+        o[1] = static_cast<double>(m.S0) / kScale;
+        o[2] = static_cast<double>(m.S1) / kScale;
+        o[3] = static_cast<double>(m.S2) / kScale;
+        o[4] = static_cast<double>(m.Q) / kScale;
+        o[5] = ui.x;
+        o[6] = ui.y;
+        o[7] = ui.z;
       }
     }
     __syncthreads();  // the stage is rewritten by the next run
@@ -855,6 +917,9 @@ __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
 
 // ------------------------------------------------------------- decision --
 
+constexpr int kDecideThreads = 64;
+constexpr int kApplyThreads = 256;
+
 __device__ __forceinline__ double laser_ax(const ClusterDev& c, double t, double* ay) {
   const double amp = c.a0 * envelope(t, c.env, c.tau);
   double sn, cs;
@@ -863,44 +928,18 @@ __device__ __forceinline__ double laser_ax(const ClusterDev& c, double t, double
   return amp * sn;
 }
 
-// Per ion: total field with the laser at t_n, local density and temperature.
-__global__ void __launch_bounds__(256) k_ion_inputs(const IonArgs a) {
-  const long long step = __ldcg(a.step);
-  if (!pass_active(a, step)) return;
-  const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (t >= a.ion.n_ions) return;
-  if (t == 0) *a.pass_slot = *a.next_slot;  // the apply kernel's base for this pass
-  // combine the source segments in order: fields add; the moments of each
-  // segment are shifted to the reference of the first segment with electrons
-  // (sums about r_s -> sums about r: S += W d, Q += 2 d.S + W |d|^2, d = r_s - r)
-  double fx = 0.0, fy = 0.0, fz = 0.0, W = 0.0, S[3] = {0.0, 0.0, 0.0}, Q = 0.0, ref[3];
-  bool have = false;
-  for (int sg = 0; sg < a.nseg; ++sg) {
-    const double* sc = a.scratch + kIonScratch * (static_cast<long long>(sg) * a.ion.n_ions + t);
-    fx += sc[0];
-    fy += sc[1];
-    fz += sc[2];
-    if (!(sc[3] > 0.0)) continue;
-    if (!have) {
-      ref[0] = sc[8]; ref[1] = sc[9]; ref[2] = sc[10];
-      have = true;
-    }
-    const double d0 = sc[8] - ref[0], d1 = sc[9] - ref[1], d2 = sc[10] - ref[2];
-    Q += sc[7] + 2.0 * (d0 * sc[4] + d1 * sc[5] + d2 * sc[6]) + sc[3] * (d0 * d0 + d1 * d1 + d2 * d2);
-    S[0] += sc[4] + sc[3] * d0;
-    S[1] += sc[5] + sc[3] * d1;
-    S[2] += sc[6] + sc[3] * d2;
-    W += sc[3];
-  }
+// Per ion: total field with the laser at t_n, local density and temperature,
+// from the Coulomb field f and the moments (weight W, sums S, Q about a
+// reference velocity).
+__device__ __forceinline__ void ion_outputs(const IonArgs& a, long long t, const double (&f)[3],
+                                            double lax, double lay, double W,
+                                            const double (&S)[3], double Q) {
   if (a.e_ion) {
-    a.e_ion[3 * t + 0] = fx;
-    a.e_ion[3 * t + 1] = fy;
-    a.e_ion[3 * t + 2] = fz;
+    a.e_ion[3 * t + 0] = f[0];
+    a.e_ion[3 * t + 1] = f[1];
+    a.e_ion[3 * t + 2] = f[2];
   }
-  const double tn = a.c.t0 + static_cast<double>(step) * a.c.dt;
-  double lay;
-  const double lax = laser_ax(a.c, tn, &lay);
-  const double ex = fx + lax, ey = fy + lay, ez = fz;
+  const double ex = f[0] + lax, ey = f[1] + lay, ez = f[2];
   double ne = 0.0, te = 0.0;
   if (W > 0.0) {
     const double lk = a.ion.r_loc / a.ion.k_si;  // r_loc in metres
@@ -918,10 +957,81 @@ __global__ void __launch_bounds__(256) k_ion_inputs(const IonArgs a) {
   a.nu[t] = -1.0;
 }
 
+// After the fused kernel: the segments are added in order; the moments of each
+// segment are shifted to the reference of the first segment with electrons
+// (sums about r_s -> sums about r: S += W d, Q += 2 d.S + W |d|^2, d = r_s - r).
+__global__ void __launch_bounds__(256) k_ion_inputs(const IonArgs a) {
+  const long long step = __ldcg(a.step);
+  if (!pass_active(a, step)) return;
+  const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (t >= a.ion.n_ions) return;
+  if (t == 0) *a.pass_slot = *a.next_slot;  // the apply kernel's base for this pass
+  double f[3] = {0.0, 0.0, 0.0}, W = 0.0, S[3] = {0.0, 0.0, 0.0}, Q = 0.0, ref[3];
+  bool have = false;
+  for (int sg = 0; sg < a.nseg; ++sg) {
+    const double* sc = a.scratch + kIonScratch * (static_cast<long long>(sg) * a.ion.n_ions + t);
+    f[0] += sc[0];
+    f[1] += sc[1];
+    f[2] += sc[2];
+    if (!(sc[3] > 0.0)) continue;
+    if (!have) {
+      ref[0] = sc[8]; ref[1] = sc[9]; ref[2] = sc[10];
+      have = true;
+    }
+    const double d0 = sc[8] - ref[0], d1 = sc[9] - ref[1], d2 = sc[10] - ref[2];
+    Q += sc[7] + 2.0 * (d0 * sc[4] + d1 * sc[5] + d2 * sc[6]) + sc[3] * (d0 * d0 + d1 * d1 + d2 * d2);
+    S[0] += sc[4] + sc[3] * d0;
+    S[1] += sc[5] + sc[3] * d1;
+    S[2] += sc[6] + sc[3] * d2;
+    W += sc[3];
+  }
+  double lay;
+  const double lax = laser_ax(a.c, a.c.t0 + static_cast<double>(step) * a.c.dt, &lay);
+  ion_outputs(a, t, f, lax, lay, W, S, Q);
+}
+
+// After the field-only kernel and the cell list's moments: 32 ions per CTA,
+// each of eight warps adds every eighth segment, the first warp the eight sums
+// (4000 ions: 23 us with a thread per ion over the strided segments).
+__global__ void __launch_bounds__(256) k_ion_inputs_sum(const IonArgs a) {
+  __shared__ double s_f[3][8][32];
+  __shared__ double s_las[2];
+  const long long step = __ldcg(a.step);
+  if (!pass_active(a, step)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long nn = a.ion.n_ions, t = static_cast<long long>(blockIdx.x) * 32 + lane;
+  if (t == 0 && warp == 0) *a.pass_slot = *a.next_slot;
+  if (threadIdx.x == 255) s_las[0] = laser_ax(a.c, a.c.t0 + static_cast<double>(step) * a.c.dt,
+                                              &s_las[1]);
+  double f[3] = {0.0, 0.0, 0.0};
+  if (t < nn) {
+#pragma unroll 4
+    for (int sg = warp; sg < a.nseg; sg += 8) {
+      const double* sc = a.scratch + 3 * static_cast<long long>(sg) * nn + t;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) f[c] += sc[c * nn];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) s_f[c][warp][lane] = f[c];
+  __syncthreads();
+  if (warp != 0 || t >= nn) return;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    f[c] = s_f[c][0][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) f[c] += s_f[c][w][lane];
+  }
+  const double* m = a.scratch + 3 * static_cast<long long>(a.nseg) * nn + kIonMom * t;
+  const double S[3] = {m[1], m[2], m[3]};
+  ion_outputs(a, t, f, s_las[0], s_las[1], m[0], S, m[4]);
+}
+
 // Per ion: rate (surrogate if it set one, else static ADK + Lotz), P and the
 // Philox draw; sets fired[t] and the number of fired ions of the block.  No
-// state changes here.
-__global__ void __launch_bounds__(256) k_ion_decide(const IonArgs a) {
+// state changes here.  Bound by the narrow FP64 pipe (the rates), so the blocks
+// are small enough to spread a few thousand ions over the SMs.
+__global__ void __launch_bounds__(kDecideThreads) k_ion_decide(const IonArgs a) {
   const long long step = __ldcg(a.step);
   if (!pass_active(a, step)) return;
   const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -1000,7 +1110,7 @@ __device__ void apply_one(const IonArgs& a, long long step, long long t, long lo
 // The fired ions, in index order, take the slots *pass_slot + (fired ions
 // before them): each block adds the counts of the blocks before it (from
 // k_ion_decide) to an in-block scan; the last block advances *next_slot.
-__global__ void __launch_bounds__(256) k_ion_apply(const IonArgs a) {
+__global__ void __launch_bounds__(kApplyThreads) k_ion_apply(const IonArgs a) {
   __shared__ int s_part[8], s_warp[8];
   __shared__ long long s_base;
   const long long step = __ldcg(a.step);
@@ -1008,7 +1118,8 @@ __global__ void __launch_bounds__(256) k_ion_apply(const IonArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // fired ions of the blocks before this one
   int before = 0;
-  for (int b = tid; b < static_cast<int>(blockIdx.x); b += 256) before += a.blk_fired[b];
+  for (int b = tid; b < static_cast<int>(blockIdx.x) * (kApplyThreads / kDecideThreads); b += 256)
+    before += a.blk_fired[b];
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
   if (lane == 0) s_part[warp] = before;
@@ -1267,9 +1378,10 @@ cudaError_t ion_fix_blocks_per_sm(int* out) {
 
 cudaError_t launch_ion_pass(const IonArgs& a, cudaStream_t s) {
   if (a.ion.n_ions <= 0) return cudaSuccess;
-  if (a.nseg < 1 || a.nseg > kIonMaxSeg) return cudaErrorInvalidValue;
+  const bool sum_only = !a.min_image && a.cells.count;
+  if (a.nseg < 1 || a.nseg > (sum_only ? kIonSumSeg : kIonMaxSeg)) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
-  if (a.min_image || !a.cells.count) {
+  if (!sum_only) {
     // field and moments in one source loop
     const long long per = kIonThreads * kIonR;
     const dim3 g1(static_cast<unsigned>((a.ion.n_ions + per - 1) / per),
@@ -1286,34 +1398,30 @@ cudaError_t launch_ion_pass(const IonArgs& a, cudaStream_t s) {
                   static_cast<unsigned>(a.nseg));
     k_ion_field_sum<kSumThreads, kSumR, kSumTile, 1, kSumPacked><<<g1, kSumThreads, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const int cells = kCellBuckets;
-    if ((e = cudaMemsetAsync(a.cells.count, 0, sizeof(int) * cells, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.cells.fill, 0, sizeof(int) * cells, s)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(a.cells.ion_count, 0, sizeof(int) * cells, s)) != cudaSuccess)
+    // (the four counter arrays lie one after the other)
+    if ((e = cudaMemsetAsync(a.cells.count, 0, sizeof(int) * (4ull << a.cells.bits), s)) !=
+        cudaSuccess)
       return e;
-    if ((e = cudaMemsetAsync(a.cells.ion_fill, 0, sizeof(int) * cells, s)) != cudaSuccess)
-      return e;
-    const unsigned gl = static_cast<unsigned>(std::min<long long>(4096, (a.c.n_pad + 255) / 256));
-    const unsigned gi = static_cast<unsigned>(
-        std::min<long long>(4096, (a.ion.n_ions + 255) / 256));
+    const unsigned gl = static_cast<unsigned>(
+        std::min<long long>(4096, (a.c.n_pad + a.ion.n_ions + 255) / 256));
     k_cell_list<false><<<gl, 256, 0, s>>>(a);
-    k_ion_cell_list<false><<<gi, 256, 0, s>>>(a);
-    if ((e = launch_cell_scan(a, a.cells.count, a.cells.start, s)) != cudaSuccess) return e;
-    if ((e = launch_cell_scan(a, a.cells.ion_count, a.cells.ion_start, s)) != cudaSuccess)
-      return e;
+    if ((e = launch_cell_scan(a, s)) != cudaSuccess) return e;
     k_cell_list<true><<<gl, 256, 0, s>>>(a);
-    k_ion_cell_list<true><<<gi, 256, 0, s>>>(a);
-    k_ion_moments<<<static_cast<unsigned>((a.ion.n_ions + kMomIons - 1) / kMomIons),
+    k_ion_moments<<<static_cast<unsigned>((a.ion.n_ions + a.mom_ions - 1) / a.mom_ions),
                     kMomThreads, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const unsigned g2 = static_cast<unsigned>((a.ion.n_ions + 255) / 256);
-  k_ion_inputs<<<g2, 256, 0, s>>>(a);
+  if (!sum_only)
+    k_ion_inputs<<<g2, 256, 0, s>>>(a);
+  else
+    k_ion_inputs_sum<<<static_cast<unsigned>((a.ion.n_ions + 31) / 32), 256, 0, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (a.ion.rate_model == 2 && a.mlp) {
     if ((e = launch_ion_mlp(a, s)) != cudaSuccess) return e;
   }
-  k_ion_decide<<<g2, 256, 0, s>>>(a);
+  k_ion_decide<<<static_cast<unsigned>((a.ion.n_ions + kDecideThreads - 1) / kDecideThreads),
+                 kDecideThreads, 0, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_ion_apply<<<g2, 256, 0, s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

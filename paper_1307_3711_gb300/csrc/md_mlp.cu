@@ -636,6 +636,7 @@ IonDev domain_io(const md_mlp_train_config& c) {
   io.dom[0] = c.e_min; io.dom[1] = c.e_max;
   io.dom[2] = c.ne_min; io.dom[3] = c.ne_max;
   io.dom[4] = c.te_min; io.dom[5] = c.te_max;
+  adk_tables(io);
   return io;
 }
 

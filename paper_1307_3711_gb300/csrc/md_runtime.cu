@@ -152,7 +152,7 @@ struct md_ctx {
   std::vector<long long> ion_out_off;  // per cluster, into d_ion_out / d_ion_fired
   bool any_ion = false;
   double* d_ion_scratch = nullptr;     // [kIonMaxSeg][max n_ions][kIonScratch]
-  int* d_ion_blk = nullptr;            // [ceil(max n_ions / 256)] fired ions per block
+  int* d_ion_blk = nullptr;            // [ceil(max n_ions / 64)] fired ions per block
   long long* d_ion_pass = nullptr;     // [n_clusters] first free slot at the pass start
   double* d_ion_out = nullptr;         // [sum n_ions][4]
   unsigned char* d_ion_fired = nullptr;
@@ -987,8 +987,11 @@ md::IonArgs ion_args(md_ctx* c, int ci, int force) {
     const long long ion_blocks = (a.ion.n_ions + per - 1) / per;
     const long long cap = std::max(1LL, static_cast<long long>(
         sum_only ? c->ion_sum_bps : c->ion_field_bps) * c->sm_count);
-    const long long by_len = std::max(1LL, static_cast<long long>(a.c.n_pad) / 2048);
-    const int smax = static_cast<int>(std::min<long long>(md::kIonMaxSeg, by_len));
+    // (the field-only kernel: segments of 256 records or more, so that a few
+    // thousand ions, a handful of blocks, still cover the SMs)
+    const long long by_len = std::max(1LL, static_cast<long long>(a.c.n_pad) / (sum_only ? 256 : 2048));
+    const int smax = static_cast<int>(
+        std::min<long long>(sum_only ? md::kIonSumSeg : md::kIonMaxSeg, by_len));
     double best = -1.0;
     a.nseg = 1;
     for (int sg = 1; sg <= smax; ++sg) {
@@ -1015,17 +1018,26 @@ md::IonArgs ion_args(md_ctx* c, int ci, int force) {
   a.fix_src = ions_fused(c, ci) ? c->d_ion_fix + 2 * c->ion_out_off[ci] : nullptr;
   std::memset(&a.cells, 0, sizeof(a.cells));
   if (!a.min_image && c->d_cell_int) {
-    constexpr long long C = md::kCellBuckets;
-    a.cells.count = c->d_cell_int + 16;
-    a.cells.start = c->d_cell_int + 16 + C;
-    a.cells.fill = c->d_cell_int + 16 + 2 * C + 1;
+    // four buckets or more per ion, at least 2^10 (the scan's block)
+    int bits = 10;
+    while (bits < md::kCellBits && (1LL << bits) < 4LL * a.ion.n_ions) ++bits;
+    const long long C = 1LL << bits;
+    int* p = c->d_cell_int;
+    a.cells.bits = bits;
+    a.cells.count = p;
+    a.cells.fill = p + C;
+    a.cells.ion_count = p + 2 * C;
+    a.cells.ion_fill = p + 3 * C;
+    a.cells.start = p + 4 * C;
+    a.cells.ion_start = p + 5 * C + 1;
+    a.cells.ion_list = p + 6 * C + 2;
+    a.cells.scan_tmp = p + 6 * C + 2 + c->cell_ion_cap;
     a.cells.rec = c->d_cell_rec;
     a.cells.capacity = c->cell_cap;
-    a.cells.ion_count = c->d_cell_int + 16 + 3 * C + 1;
-    a.cells.ion_start = c->d_cell_int + 16 + 4 * C + 1;
-    a.cells.ion_fill = c->d_cell_int + 16 + 5 * C + 2;
-    a.cells.ion_list = c->d_cell_int + 16 + 6 * C + 2;
-    a.cells.scan_tmp = c->d_cell_int + 16 + 6 * C + 2 + c->cell_ion_cap;
+    // the moments' CTAs: eight warps, one ion at a time each; two or more CTAs
+    // per SM before an ion list gets longer
+    a.mom_ions = static_cast<int>(std::max(
+        8LL, std::min(64LL, a.ion.n_ions / (2LL * c->sm_count) / 8 * 8)));
   }
   // segments of the charge-change field: about 3 waves of (ion block, segment) CTAs
   {
@@ -1456,6 +1468,7 @@ md_status create_context(const md_config* cfgs, int32_t n_clusters, const long l
       io.ip_ev[z] = f.ip_ev[z];
       io.q_outer[z] = f.q_outer[z];
     }
+    md::adk_tables(io);
     c->ion_out_off.push_back(c->ion.empty() ? 0 : c->ion_out_off.back() + c->ion.back().n_ions);
     c->ion.push_back(io);
     c->ion_push.push_back(0);
@@ -1517,7 +1530,7 @@ md_status create_context(const md_config* cfgs, int32_t n_clusters, const long l
     }
     if (dev_alloc(&c->d_ion_scratch, static_cast<size_t>(md::kIonMaxSeg) * md::kIonScratch *
                                          static_cast<size_t>(max_ion)) != cudaSuccess ||
-        dev_alloc(&c->d_ion_blk, static_cast<size_t>((max_ion + 255) / 256)) != cudaSuccess ||
+        dev_alloc(&c->d_ion_blk, static_cast<size_t>((max_ion + 63) / 64 + 4)) != cudaSuccess ||
         dev_alloc(&c->d_ion_pass, static_cast<size_t>(n_clusters)) != cudaSuccess ||
         dev_alloc(&c->d_ion_out, 4 * static_cast<size_t>(sum_ion)) != cudaSuccess ||
         dev_alloc(&c->d_ion_fired, static_cast<size_t>(sum_ion)) != cudaSuccess ||
@@ -1537,7 +1550,7 @@ md_status create_context(const md_config* cfgs, int32_t n_clusters, const long l
       constexpr size_t C = md::kCellBuckets;
       long long cap = 0;
       for (const auto& d : c->cl) cap = std::max<long long>(cap, d.n_pad);
-      if (dev_alloc(&c->d_cell_int, 16 + 6 * C + 2 + static_cast<size_t>(max_ion) + C / 1024) !=
+      if (dev_alloc(&c->d_cell_int, 6 * C + 2 + static_cast<size_t>(max_ion) + 2 * C / 1024) !=
               cudaSuccess ||
           dev_alloc(&c->d_cell_rec, 2 * static_cast<size_t>(cap)) != cudaSuccess)
         return bail(fail(MD_ERR_OOM, "cell list"));

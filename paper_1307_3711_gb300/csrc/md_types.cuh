@@ -1,6 +1,7 @@
 // md_types.cuh -- plain data shared by the kernels and the host runtime.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -44,6 +45,11 @@ __host__ __device__ inline int live_seg_len(int n_pad, int nseg, long long live)
 constexpr int kMaxZ = 16;
 constexpr int kIonScratch = 11;   // doubles per ion and source segment
 constexpr int kIonMaxSeg = 32;    // source segments of the ionization field pass
+// the field-only pass writes three doubles per ion and segment, so the same
+// scratch holds more segments; the moments follow, kIonMom doubles per ion
+constexpr int kIonSumSeg = 112;
+constexpr int kIonMom = 8;
+static_assert(3 * kIonSumSeg + kIonMom <= kIonScratch * kIonMaxSeg, "pass scratch");
 
 // Ionization parameters of one cluster (Sec. II, ionization paragraph).
 struct IonDev {
@@ -60,7 +66,27 @@ struct IonDev {
   double ip_ev[kMaxZ];
   double q_outer[kMaxZ];
   double dom[6];      // surrogate domain: |E| min/max, n_e min/max, T_e min/max
+  // ADK constants of the charge states (adk_tables)
+  double adk_c[kMaxZ], adk_f0[kMaxZ], adk_p[kMaxZ];
 };
+
+// The parts of the static ADK rate that depend on the charge state alone:
+// n* = Z / sqrt(2 Ip), l* = n* - 1; c = C^2 Ip with C^2 = 2^(2 n*) /
+// (n* Gamma(n* + l* + 1) Gamma(n* - l*)), f0 = (2 Ip)^(3/2), p = 2 n* - 1
+// (Ip in hartree).  Two gamma functions and two powers per ion and pass less.
+inline void adk_tables(IonDev& io) {
+  constexpr double kHartreeEv = 27.211386245988;
+  for (int z = 0; z < kMaxZ; ++z) {
+    const double ip = io.ip_ev[z] / kHartreeEv;
+    io.adk_c[z] = io.adk_f0[z] = io.adk_p[z] = 0.0;
+    if (!(ip > 0.0)) continue;
+    const double ns = static_cast<double>(z + 1) / std::sqrt(2.0 * ip), ls = ns - 1.0;
+    io.adk_c[z] = std::pow(2.0, 2.0 * ns) /
+                  (ns * std::tgamma(ns + ls + 1.0) * std::tgamma(ns - ls)) * ip;
+    io.adk_f0[z] = std::pow(2.0 * ip, 1.5);
+    io.adk_p[z] = 2.0 * ns - 1.0;
+  }
+}
 
 // One unit of the step kernel: the field at one i-block of targets from one
 // piece of its cluster's sources.  The pieces of an i-block publish partial
@@ -172,23 +198,27 @@ struct SmallBlk {
 
 // Cell list of the electrons near the ions, for the local moments of the
 // ionization pass (clusters without minimum-image forces): cells of side
-// 1.01 r_loc, hashed into kCellBuckets buckets, the electrons of each bucket
-// listed contiguously as (position record, velocity record) pairs, and the
-// ions listed by bucket too.
-constexpr int kCellBuckets = 1 << 18;
+// 1.01 r_loc, hashed into 2^bits buckets (about four per ion, at most
+// kCellBuckets), the electrons of each bucket listed contiguously, and the ions
+// listed by bucket too.
+constexpr int kCellBits = 18;
+constexpr int kCellBuckets = 1 << kCellBits;
 struct CellBuf {
-  int* count;    // [kCellBuckets] electrons per bucket
-  int* start;    // [kCellBuckets + 1] first listed electron of each bucket
-  int* fill;     // [kCellBuckets] fill counters of the listing
-  float4* rec;   // [2 capacity] the listed electrons' position and velocity records
+  int bits;
+  // electrons and ions per bucket, fill counters of the two listings: four
+  // arrays of 2^bits, one after the other
+  int* count;
+  int* fill;
+  int* start;    // [2^bits + 1] first listed electron of each bucket
+  float4* rec;   // [2][capacity] the listed electrons' position, then velocity records
   long long capacity;
   // the ions listed by bucket, so that neighbouring threads of the moment
   // kernel take ions of one cell and read the same electron lists
-  int* ion_count;  // [kCellBuckets]
-  int* ion_start;  // [kCellBuckets + 1]
-  int* ion_fill;   // [kCellBuckets]
+  int* ion_count;
+  int* ion_start;  // [2^bits + 1]
+  int* ion_fill;
   int* ion_list;   // [n_ions capacity] ion records in bucket order
-  int* scan_tmp;   // [kCellBuckets / 1024] block totals of the bucket scans
+  int* scan_tmp;   // [2 kCellBuckets / 1024] block totals of the bucket scans
 };
 
 // Arguments of the ionization kernels of one cluster.
@@ -211,11 +241,13 @@ struct IonArgs {
   const long long* step;
   int* err;
   int force;          // 1: run regardless of ionize_every
-  double* scratch;    // [nseg][n_ions][kIonScratch]: ex, ey, ez, sw, sw du_x, sw du_y,
+  double* scratch;    // moments from the cell list: [nseg][3][n_ions] field, then
+                      // [n_ions][kIonMom] sw .. u_ref; else
+                      // [nseg][n_ions][kIonScratch]: ex, ey, ez, sw, sw du_x, sw du_y,
                       // sw du_z, sw du^2, u_ref (3) of each source segment (du = u -
                       // u_ref, u_ref = the segment's first local electron's u)
   int nseg;           // source segments of the field pass (equal shares of the live records)
-  int* blk_fired;     // [ceil(n_ions / 256)] fired ions per block of the decision
+  int* blk_fired;     // fired ions per block of 64 of the decision
   long long* pass_slot;  // first free slot at the start of the pass
   double* out;        // [n_ions][4]: |E|, ne (cm^-3), Te (eV), P
   double* nu;         // [n_ions]: rate from the surrogate, or -1 (use the plain rate)
@@ -240,6 +272,7 @@ struct IonArgs {
   // local moments from a cell list (cells.count non-null) instead of beside
   // the field sum
   CellBuf cells;
+  int mom_ions;       // ions per CTA of the moments
   // 1: minimum-image distances while the boundary is periodic (field and
   // local moments of the pass, charge-change correction)
   int min_image;
