@@ -646,23 +646,17 @@ cudaError_t launch_cell_scan(const IonArgs& a, cudaStream_t s) {
 // and added to 64-bit integer sums, so a total does not depend on which lane
 // took which electron, nor on the order of the listing.
 //
-// The ions are taken in bucket order, a.mom_ions per CTA (fewer of them when
-// the cluster is small, so that the CTAs cover the SMs).  The ions of one
-// bucket mostly share one cell and so one set of 27 neighbour cells: for each
-// run of ions with the same bucket, the positions of the electrons listed in
-// those cells' buckets (a few thousand) are staged once in shared memory, and
-// each warp tests them against one ion at a time, 32 electrons per step.  An
-// ion of the run in another cell (two cells hashed to one bucket, or a
-// position without a cell) and a run whose electrons do not fit the stage
-// walk their own 27 buckets from global memory instead, four loads in flight.
-// Either way the electrons within r_loc are queued and their terms added 32 at
-// a time: in a dense plasma (6000 electrons in the 27 cells, 15 % of them
-// within r_loc) adding them where they are found kept a seventh of the lanes
-// busy.  4000 ions: 578 -> 75 us per pass, 50000: 1.54 -> 0.72 ms.
+// A warp takes one ion, the ions in bucket order, so that the warps of a CTA
+// read mostly the same buckets and meet in L1: the electrons of the 27 cells'
+// buckets, four loads in flight, those within r_loc queued and their terms
+// added 32 at a time.  In a dense plasma (8000 electrons in the 27 cells, 15 %
+// of them within r_loc) adding them where they are found kept a seventh of the
+// lanes busy.  Per pass, us: 4000 ions 73 (578 with the electrons of a cell
+// staged in shared memory and added where found, 139 staged and queued), 50000
+// ions 650 (1540, 1115), 200000 atoms with 334000 electrons 790 (staged and
+// queued 798), with 89000 electrons 171 (234).
 constexpr int kMomThreads = 256;
 constexpr int kMomWarps = kMomThreads / 32;
-constexpr int kMomIons = 64;     // ions per CTA at most
-constexpr int kMomCap = 3072;    // staged electrons per run
 
 // v rounded to the nearest integer, ties to even, as a 64-bit integer, on
 // the integer pipe (for |v| < 2^62).  From the binary32 layout: v = m 2^s
@@ -769,7 +763,7 @@ struct NearQueue {
 
 // One warp: the sums of one ion over its 27 cells' buckets, read from global
 // memory (lane-strided over each bucket's electrons).
-__device__ __forceinline__ void moments_global(const CellBuf& cb, const float4 pi,
+__device__ __forceinline__ void moments_of(const CellBuf& cb, const float4 pi,
                                                const float4 ui, const int (&cc)[3], float eps2,
                                                float rloc2e, int lane, MomSums& m, int* queue,
                                                int* err) {
@@ -804,114 +798,37 @@ __device__ __forceinline__ void moments_global(const CellBuf& cb, const float4 p
 }
 
 __global__ void __launch_bounds__(kMomThreads) k_ion_moments(const IonArgs a) {
-  __shared__ float4 s_pos[kMomCap];
-  __shared__ int s_idx[kMomCap];
   __shared__ int s_near[kMomWarps][64];
-  __shared__ int s_bucket[kMomIons];
-  __shared__ int s_bk[32], s_beg[32], s_cnt[32];
-  __shared__ int s_total;
   const long long step = __ldcg(a.step);
   if (!pass_active(a, step)) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const CellBuf cb = a.cells;
   const float4* __restrict__ cur = (step & 1) ? a.posq1 : a.posq0;
-  const float4* vel = cb.rec + cb.capacity;
   const float eps2 = a.c.eps2;
   const float rloc2e = static_cast<float>(a.ion.r_loc * a.ion.r_loc) + eps2;
-  const float inv_h = cell_inv_h(a);
-  const long long c0 = static_cast<long long>(blockIdx.x) * a.mom_ions;
-  const int nloc = static_cast<int>(a.ion.n_ions - c0 < a.mom_ions ? a.ion.n_ions - c0 : a.mom_ions);
-  // each ion's bucket, as the ion listing computed it (no cell: bucket 0)
-  if (tid < nloc) {
-    const long long t = cb.ion_list[c0 + tid];
-    int b = 0;
-    if (MD_IN_RANGE(a.err, t, 0, a.ion.n_ions)) {
-      const float4 p = cur[a.c.off + t];
-      b = bucket_of(p.x, p.y, p.z, inv_h, cb.bits);
-      b = b < 0 ? 0 : b;
-    }
-    s_bucket[tid] = b;
+  const long long q = static_cast<long long>(blockIdx.x) * kMomWarps + warp;
+  if (q >= a.ion.n_ions) return;
+  const long long t = cb.ion_list[q];
+  if (!MD_IN_RANGE(a.err, t, 0, a.ion.n_ions)) return;  // warp-uniform
+  const float4 pi = cur[a.c.off + t];
+  const float4 ui = a.vel[a.c.off + t];
+  MomSums m;
+  int cc[3];
+  if (cell_coords(pi.x, pi.y, pi.z, cell_inv_h(a), cc)) {
+    moments_of(cb, pi, ui, cc, eps2, rloc2e, lane, m, s_near[warp], a.err);
+    m.warp_sum();
   }
-  __syncthreads();
-  for (int r0 = 0; r0 < nloc;) {
-    int r1 = r0 + 1;
-    while (r1 < nloc && s_bucket[r1] == s_bucket[r0]) ++r1;
-    // the run's first ion sets the staged cell
-    const long long t0 = cb.ion_list[c0 + r0];
-    int cc0[3] = {0, 0, 0};
-    bool staged = MD_IN_RANGE(a.err, t0, 0, a.ion.n_ions);
-    if (staged) {
-      const float4 p0 = cur[a.c.off + t0];
-      staged = cell_coords(p0.x, p0.y, p0.z, inv_h, cc0);
-    }
-    if (staged && warp == 0) {
-      const int bk = neighbour_bucket(cc0, lane, cb.bits);
-      const int cnt = bk >= 0 ? cb.start[bk + 1] - cb.start[bk] : 0;
-      int inc = cnt;  // inclusive scan of the counts over the lanes
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= d) inc += y;
-      }
-      s_bk[lane] = bk;
-      s_cnt[lane] = cnt;
-      s_beg[lane] = inc - cnt;
-      if (lane == 31) s_total = inc;
-    }
-    __syncthreads();
-    // staging pays from three ions on (one would read its electrons once either way)
-    staged = staged && s_total <= kMomCap && r1 - r0 >= 3;
-    if (staged) {
-      for (int l = 0; l < 27; ++l) {
-        const int cnt = s_cnt[l];
-        if (cnt == 0) continue;
-        const int k0 = cb.start[s_bk[l]], beg = s_beg[l];
-        for (int k = tid; k < cnt; k += kMomThreads) {
-          const bool ok = MD_IN_RANGE(a.err, k0 + k, 0, cb.capacity);
-          // (an index out of range stages a position no ion is near)
-          s_pos[beg + k] = ok ? cb.rec[k0 + k] : make_float4(3e38f, 3e38f, 3e38f, 0.f);
-          s_idx[beg + k] = ok ? k0 + k : 0;
-        }
-      }
-    }
-    __syncthreads();
-    const int total = staged ? s_total : 0;
-    for (int q = r0 + warp; q < r1; q += kMomWarps) {
-      const long long t = cb.ion_list[c0 + q];
-      if (!MD_IN_RANGE(a.err, t, 0, a.ion.n_ions)) continue;  // warp-uniform
-      const float4 pi = cur[a.c.off + t];
-      const float4 ui = a.vel[a.c.off + t];
-      MomSums m;
-      int cc[3];
-      if (cell_coords(pi.x, pi.y, pi.z, inv_h, cc)) {
-        if (staged && cc[0] == cc0[0] && cc[1] == cc0[1] && cc[2] == cc0[2]) {
-          NearQueue nq{s_near[warp], 0};
-          for (int k0 = 0; k0 < total; k0 += 32) {
-            const int k = k0 + lane;
-            nq.push(k < total && near_loc(s_pos[k], pi, eps2, rloc2e), k < total ? s_idx[k] : 0,
-                    vel, ui, lane, m);
-          }
-          nq.flush(vel, ui, lane, m);
-        } else {
-          moments_global(cb, pi, ui, cc, eps2, rloc2e, lane, m, s_near[warp], a.err);
-        }
-        m.warp_sum();
-      }
-      if (lane == 0) {
-        constexpr double kScale = 1099511627776.0;  // 2^40
-        double* o = a.scratch + 3 * static_cast<long long>(a.nseg) * a.ion.n_ions + kIonMom * t;
-        o[0] = static_cast<double>(m.W) / kScale;
-        o[1] = static_cast<double>(m.S0) / kScale;
-        o[2] = static_cast<double>(m.S1) / kScale;
-        o[3] = static_cast<double>(m.S2) / kScale;
-        o[4] = static_cast<double>(m.Q) / kScale;
-        o[5] = ui.x;
-        o[6] = ui.y;
-        o[7] = ui.z;
-      }
-    }
-    __syncthreads();  // the stage is rewritten by the next run
-    r0 = r1;
+  if (lane == 0) {
+    constexpr double kScale = 1099511627776.0;  // 2^40
+    double* o = a.scratch + 3 * static_cast<long long>(a.nseg) * a.ion.n_ions + kIonMom * t;
+    o[0] = static_cast<double>(m.W) / kScale;
+    o[1] = static_cast<double>(m.S0) / kScale;
+    o[2] = static_cast<double>(m.S1) / kScale;
+    o[3] = static_cast<double>(m.S2) / kScale;
+    o[4] = static_cast<double>(m.Q) / kScale;
+    o[5] = ui.x;
+    o[6] = ui.y;
+    o[7] = ui.z;
   }
 }
 
@@ -1407,7 +1324,7 @@ cudaError_t launch_ion_pass(const IonArgs& a, cudaStream_t s) {
     k_cell_list<false><<<gl, 256, 0, s>>>(a);
     if ((e = launch_cell_scan(a, s)) != cudaSuccess) return e;
     k_cell_list<true><<<gl, 256, 0, s>>>(a);
-    k_ion_moments<<<static_cast<unsigned>((a.ion.n_ions + a.mom_ions - 1) / a.mom_ions),
+    k_ion_moments<<<static_cast<unsigned>((a.ion.n_ions + kMomWarps - 1) / kMomWarps),
                     kMomThreads, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -1018,9 +1018,11 @@ md::IonArgs ion_args(md_ctx* c, int ci, int force) {
   a.fix_src = ions_fused(c, ci) ? c->d_ion_fix + 2 * c->ion_out_off[ci] : nullptr;
   std::memset(&a.cells, 0, sizeof(a.cells));
   if (!a.min_image && c->d_cell_int) {
-    // four buckets or more per ion, at least 2^10 (the scan's block)
+    // a bucket or more per ion, at least 2^10 (the scan's block): a solid
+    // cluster holds 36 ions per cell, an expanded one still under one cell per
+    // ion; cells that share a bucket only cost each other's tests
     int bits = 10;
-    while (bits < md::kCellBits && (1LL << bits) < 4LL * a.ion.n_ions) ++bits;
+    while (bits < md::kCellBits && (1LL << bits) < a.ion.n_ions) ++bits;
     const long long C = 1LL << bits;
     int* p = c->d_cell_int;
     a.cells.bits = bits;
@@ -1034,10 +1036,6 @@ md::IonArgs ion_args(md_ctx* c, int ci, int force) {
     a.cells.scan_tmp = p + 6 * C + 2 + c->cell_ion_cap;
     a.cells.rec = c->d_cell_rec;
     a.cells.capacity = c->cell_cap;
-    // the moments' CTAs: eight warps, one ion at a time each; two or more CTAs
-    // per SM before an ion list gets longer
-    a.mom_ions = static_cast<int>(std::max(
-        8LL, std::min(64LL, a.ion.n_ions / (2LL * c->sm_count) / 8 * 8)));
   }
   // segments of the charge-change field: about 3 waves of (ion block, segment) CTAs
   {

@@ -198,7 +198,7 @@ struct SmallBlk {
 
 // Cell list of the electrons near the ions, for the local moments of the
 // ionization pass (clusters without minimum-image forces): cells of side
-// 1.01 r_loc, hashed into 2^bits buckets (about four per ion, at most
+// 1.01 r_loc, hashed into 2^bits buckets (one or more per ion, at most
 // kCellBuckets), the electrons of each bucket listed contiguously, and the ions
 // listed by bucket too.
 constexpr int kCellBits = 18;
@@ -272,7 +272,6 @@ struct IonArgs {
   // local moments from a cell list (cells.count non-null) instead of beside
   // the field sum
   CellBuf cells;
-  int mom_ions;       // ions per CTA of the moments
   // 1: minimum-image distances while the boundary is periodic (field and
   // local moments of the pass, charge-change correction)
   int min_image;
