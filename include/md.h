@@ -459,10 +459,11 @@ md_status md_plan_shares(const int32_t *n_pad, int32_t n_clusters, int32_t per, 
  *         is removed), or -1 if targets are not sources
  *   e:    device double[nt][3] output field; phi: device double[nt] or NULL
  *   stream: cudaStream_t (NULL = legacy default stream).  Asynchronous.
- * When few targets would leave the GPU mostly idle, the sources are split
- * into segments whose partial fields are added in order (deterministic); the
- * partials are allocated and freed in stream order on `stream` (at most
- * 256 MB), so calls on different streams may overlap.
+ * Few targets or sources: one launch whose CTAs add their partial sums on the
+ * chip.  Otherwise the sources are split into segments whose partial fields are
+ * added in order; the partials are allocated and freed in stream order on
+ * `stream` (at most 256 MB).  Deterministic; calls on different streams may
+ * overlap.
  * Errors: MD_ERR_ARG for NULL/unaligned pointers, ns < 0, nt < 0.  A
  * device-side wait that runs out of its budget (about 2 s) leaves e/phi not
  * (completely) written and is recorded in the device's sticky field error
@@ -475,19 +476,16 @@ md_status md_coulomb_field_device(const void *src, int64_t ns, const void *tgt,
  * md_coulomb_field_device, for callers that cannot allocate device memory
  * (code inside another framework's memory pool, a graph builder that must not
  * see cudaMalloc, a plugin whose host forbids allocation).  The paper has no
- * counterpart: this is a library-interface variant.  The sources are cut into
- * up to 8 segments whose partial fields go to a fixed scratch array compiled
- * into the library (about 8.6 MB of device memory on every GPU that loads it,
- * held until the process exits); the call itself allocates nothing.
+ * counterpart: this is a library-interface variant.  The CTAs that share a
+ * target add their partial sums on the chip, so the call needs no scratch
+ * memory.
  *   Arguments, layout and ownership: as md_coulomb_field_device.
  *   Limit: nt <= 32768 targets per call (MD_ERR_ARG beyond it, nothing is
  *   launched); ns is unbounded.
- *   The first call on a device looks up the scratch array's device address on
+ *   The first call on a device looks up the error word's device address on
  *   that device; make that first call before any stream capture.
- *   Every call shares the one scratch array: calls that overlap on the GPU
- *   (other streams, other host threads) race and give wrong results, so
- *   serialise them.  Each call clears the counters it uses before its kernel.
- *   Asynchronous on `stream`. */
+ *   Calls on different streams or host threads may overlap.  Asynchronous on
+ *   `stream`. */
 md_status md_coulomb_field_device_noalloc(const void *src, int64_t ns, const void *tgt,
                                           int64_t nt, float eps2, int64_t self_offset,
                                           double *e, double *phi, void *stream);

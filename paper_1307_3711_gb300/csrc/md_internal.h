@@ -112,9 +112,16 @@ cudaError_t launch_live_init(const float4* posq0, const float4* posq1, const uns
 // Surrogate rates of the ions inside its domain (rate_model 2).
 cudaError_t launch_ion_mlp(const IonArgs& a, cudaStream_t s);
 
-// Device address of the current device's error word of the stateless field
-// calls (a file-scope device array, looked up once per device).
-md_status field_error_word(int** out);
+// The current device's error word of the stateless field calls (a file-scope
+// device array) and its number of SMs (sms may be nullptr), looked up once per
+// device.
+md_status field_device(int** err, int* sms);
+
+// Field (and potential) in one launch without scratch memory (md_probe.cu; no
+// liveness flags, no image forces), and whether that is faster than
+// launch_field with nseg segments.
+cudaError_t launch_field_direct(const FieldArgs& a, bool potential, int sms, cudaStream_t s);
+bool field_uses_probe(long long nt, long long ns, long long nseg, int sms);
 
 // Records the thread-local message returned by md_last_error() and returns
 // the status (implemented in md_runtime.cu).

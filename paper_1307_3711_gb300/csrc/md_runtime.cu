@@ -2000,6 +2000,13 @@ static md_status run_fields(md_ctx* c, int ci, bool potential) {
   const long long want = (4LL * c->field_bps * c->sm_count + blocks - 1) / blocks;
   const long long nseg = std::max(1LL, std::min({want, static_cast<long long>(kFieldMaxSeg),
                                                 a.ns / 2048}));
+  // (a periodic cluster keeps the kernel whose minimum-image twin gives the
+  // same bits where no pair needs an image)
+  if (!a.src_live && cl.boundary == MD_BOUNDARY_OPEN && a.nt > 0 &&
+      md::field_uses_probe(a.nt, a.ns, nseg, c->sm_count)) {
+    MD_CUDA(md::launch_field_direct(a, potential, c->sm_count, c->stream));
+    return MD_OK;
+  }
   if (nseg > 1) {
     a.nseg = static_cast<int>(nseg);
     a.seg_len = (a.ns + nseg - 1) / nseg;
@@ -2547,11 +2554,10 @@ static md_status md_coulomb_field_device_body(const void* src, int64_t ns, const
   if (!(eps2 > 0.0f)) return fail(MD_ERR_ARG, "eps2 must be > 0");
   // the sticky error word of the stateless field calls on this device, read
   // and cleared by md_field_device_status
-  int dev = 0;
-  MD_CUDA(cudaGetDevice(&dev));
   int* d_err = nullptr;
+  int sms = 1;
   {
-    const md_status es = md::field_error_word(&d_err);
+    const md_status es = md::field_device(&d_err, &sms);
     if (es != MD_OK) return es;
   }
   md::FieldArgs a;
@@ -2571,15 +2577,18 @@ static md_status md_coulomb_field_device_body(const void* src, int64_t ns, const
   // split the sources until about 4 waves of CTAs run (up to 64 segments of
   // at least 4 tiles, partials of at most 256 MB); the partials live in
   // stream-ordered memory, so calls on different streams do not share them
-  int bps = 1, sms = 1;
+  int bps = 1;
   MD_CUDA(md::field_blocks_per_sm(&bps));
-  MD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const long long per = md::field_targets_per_cta();
   const long long nt_ = static_cast<long long>(nt), ns_ = static_cast<long long>(ns);
   const long long blocks = (nt_ + per - 1) / per;
   const long long want = (4LL * std::max(1, bps) * sms + blocks - 1) / blocks;
   const long long by_mem = (256LL << 20) / (32LL * nt_);
   const long long nseg = std::max(1LL, std::min({want, 64LL, ns_ / 2048, by_mem}));
+  if (md::field_uses_probe(nt_, ns_, nseg, sms)) {
+    MD_CUDA(md::launch_field_direct(a, phi != nullptr, sms, st));
+    return MD_OK;
+  }
   void* part = nullptr;
   if (nseg > 1) {
     MD_CUDA(cudaMallocAsync(&part, static_cast<size_t>(32 * nseg * nt_), st));

@@ -44,8 +44,7 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
   constexpr int kTargets = TL * R;
   constexpr int kSlices = THREADS / TL;
   constexpr int C = POT ? 4 : 3;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  SmallSmem<THREADS, TL, R, POT>& S = *reinterpret_cast<SmallSmem<THREADS, TL, R, POT>*>(smem_raw);
+  __shared__ SmallSmem<THREADS, TL, R, POT> S;
 
   const int tid = threadIdx.x;
   const SmallBlk b = blks ? blks[blockIdx.x] : SmallBlk{0, static_cast<int>(blockIdx.x) * kTargets};
@@ -184,12 +183,7 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
 
 template <int THREADS, int TL, int R, bool DET, bool POT>
 cudaError_t launch_k(const StepArgs& a, const SmallBlk* blks, int n_blks, cudaStream_t s) {
-  constexpr size_t bytes = sizeof(SmallSmem<THREADS, TL, R, POT>);
-  cudaError_t e = cudaFuncSetAttribute(k_step_small<THREADS, TL, R, DET, POT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(bytes));
-  if (e != cudaSuccess) return e;
-  k_step_small<THREADS, TL, R, DET, POT><<<n_blks, THREADS + 64, bytes, s>>>(a, blks);
+  k_step_small<THREADS, TL, R, DET, POT><<<n_blks, THREADS + 64, 0, s>>>(a, blks);
   return cudaGetLastError();
 }
 

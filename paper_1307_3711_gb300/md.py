@@ -502,8 +502,8 @@ def coulomb_field_fp64_device(xs_ptr: int, qs_ptr: int, ns: int, xt_ptr: int, se
 def coulomb_field_device_noalloc(src_ptr: int, ns: int, tgt_ptr: int, nt: int, eps2: float,
                                  self_offset: int, e_ptr: int, phi_ptr: int | None,
                                  stream: int | None):
-    """As ``coulomb_field_device`` without any device allocation: its scratch
-    is a fixed array inside the library (nt <= 32768; overlapping calls race)."""
+    """As ``coulomb_field_device`` without any device allocation
+    (nt <= 32768)."""
     _check(_lib.md_coulomb_field_device_noalloc(
         C.c_void_p(src_ptr), int(ns), C.c_void_p(tgt_ptr), int(nt), float(eps2),
         int(self_offset), C.c_void_p(e_ptr), C.c_void_p(phi_ptr) if phi_ptr else None,
