@@ -82,28 +82,38 @@ __device__ __forceinline__ float dsilu(float a) {
 }
 
 // Weights of one CTA in shared memory: BF16 hidden-layer matrices (W1 padded
-// to K = 16), FP32 output layer and biases.
+// to K = 16), FP32 output layer and biases.  The rows are padded so that the
+// eight rows and four columns that the lanes of a warp read at once lie in
+// different banks (rows of 32 words met eight at a time in one bank).
+constexpr int kW1Row = 24, kW2Row = 72, kW3Row = 72;
 struct MlpWeights {
-  alignas(16) __nv_bfloat16 w1[kNH][16];
-  alignas(16) __nv_bfloat16 w2[kNH][kNH];
-  alignas(16) float w3[kNO][kNH];
+  alignas(16) __nv_bfloat16 w1[kNH][kW1Row];
+  alignas(16) __nv_bfloat16 w2[kNH][kW2Row];
+  alignas(16) float w3[kNO][kW3Row];
   float b1[kNH], b2[kNH], b3[kNO];
 };
 
-__device__ void load_weights(const float* __restrict__ p, MlpWeights& w) {
-  for (int e = threadIdx.x; e < kNH * 16; e += blockDim.x) {
-    const int n = e >> 4, k = e & 15;
-    w.w1[n][k] = __float2bfloat16_rn(k < kNI ? p[kOffW1 + n * kNI + k] : 0.0f);
+template <int THREADS>
+__device__ __forceinline__ void load_weights(const float* __restrict__ p, MlpWeights& w) {
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int e = tid; e < kNH * kNH / 2; e += THREADS) {  // pairs of a row
+    const float lo = __ldg(p + kOffW2 + 2 * e), hi = __ldg(p + kOffW2 + 2 * e + 1);
+    *reinterpret_cast<uint32_t*>(&w.w2[e >> 5][2 * (e & 31)]) = pack_bf16(lo, hi);
   }
-  for (int e = threadIdx.x; e < kNH * kNH; e += blockDim.x)
-    w.w2[e >> 6][e & 63] = __float2bfloat16_rn(p[kOffW2 + e]);
-  for (int e = threadIdx.x; e < kNO * kNH; e += blockDim.x)
-    w.w3[e >> 6][e & 63] = p[kOffW3 + e];
-  for (int e = threadIdx.x; e < kNH; e += blockDim.x) {
+#pragma unroll
+  for (int e = tid; e < kNH * 8; e += THREADS) {
+    const int n = e >> 3, k = 2 * (e & 7);
+    *reinterpret_cast<uint32_t*>(&w.w1[n][k]) =
+        k < kNI ? pack_bf16(p[kOffW1 + n * kNI + k], p[kOffW1 + n * kNI + k + 1]) : 0u;
+  }
+#pragma unroll
+  for (int e = tid; e < kNO * kNH; e += THREADS) w.w3[e >> 6][e & 63] = p[kOffW3 + e];
+  for (int e = tid; e < kNH; e += THREADS) {
     w.b1[e] = p[kOffB1 + e];
     w.b2[e] = p[kOffB2 + e];
   }
-  for (int e = threadIdx.x; e < kNO; e += blockDim.x) w.b3[e] = p[kOffB3 + e];
+  if (tid < kNO) w.b3[tid] = p[kOffB3 + tid];
 }
 
 __device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16* p) {
@@ -135,14 +145,12 @@ __device__ __forceinline__ void c_to_a(const float (&c)[8][4], uint32_t (&a)[4][
   }
 }
 
-// x: features of rows g and g+8 of this warp's tile (x_lo, x_hi: 4 values).
-// Hidden layers only: a1, h1, a2.
-__device__ __forceinline__ void forward_hidden(const MlpWeights& w, const float (&xg)[4],
-                                               const float (&xg8)[4], Fwd& f) {
+// x0, x1: this lane's A fragments of layer 1, the features 2t and 2t + 1 of rows
+// g and g + 8 of the warp's tile as BF16 (0 for t >= 2: K = 16, columns 0..3
+// real).  Hidden layers only: a1, h1, a2.
+__device__ __forceinline__ void forward_hidden(const MlpWeights& w, uint32_t x0, uint32_t x1,
+                                               Fwd& f) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  // layer 1: A = features padded to K = 16 (columns 0..3 real)
-  const uint32_t x0 = t < 2 ? pack_bf16(xg[2 * t], xg[2 * t + 1]) : 0u;
-  const uint32_t x1 = t < 2 ? pack_bf16(xg8[2 * t], xg8[2 * t + 1]) : 0u;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const float b0 = w.b1[8 * j + 2 * t], b1 = w.b1[8 * j + 2 * t + 1];
@@ -166,8 +174,9 @@ __device__ __forceinline__ void forward_hidden(const MlpWeights& w, const float 
 // All 8 outputs of rows g and g+8 (every lane of the quad gets them).
 __device__ __forceinline__ void forward(const MlpWeights& w, const float (&xg)[4],
                                         const float (&xg8)[4], Fwd& f) {
-  forward_hidden(w, xg, xg8, f);
   const int t = threadIdx.x & 3;
+  forward_hidden(w, t < 2 ? pack_bf16(xg[2 * t], xg[2 * t + 1]) : 0u,
+                 t < 2 ? pack_bf16(xg8[2 * t], xg8[2 * t + 1]) : 0u, f);
   // layer 3 in FP32: partial dot products over this lane's 16 columns of
   // rows g and g+8, summed over the quad (lanes t = 0..3)
 #pragma unroll
@@ -216,11 +225,10 @@ __device__ __forceinline__ double rate_of_output(float y) {
 
 // Output of the charge state of each row only (rows g and g+8 of the warp's
 // tile): the FP32 dot product of that row of W3, summed over the quad.
-__device__ __forceinline__ void forward_sel(const MlpWeights& w, const float (&xg)[4],
-                                            const float (&xg8)[4], int z0, int z1,
-                                            float (&ysel)[2]) {
+__device__ __forceinline__ void forward_sel(const MlpWeights& w, uint32_t x0, uint32_t x1, int z0,
+                                            int z1, float (&ysel)[2]) {
   Fwd f;
-  forward_hidden(w, xg, xg8, f);
+  forward_hidden(w, x0, x1, f);
   const int t = threadIdx.x & 3;
   float p0 = 0.0f, p1 = 0.0f;
 #pragma unroll
@@ -237,13 +245,46 @@ __device__ __forceinline__ void forward_sel(const MlpWeights& w, const float (&x
   ysel[1] = p1 + w.b3[z1];
 }
 
+// One warp, 32 samples, lane l holding sample l's inputs: the output of its
+// charge state z (clamped to the network's).  The features are formed once per
+// sample and reach the two 16-row tiles' fragments by shuffles.
+__device__ __forceinline__ float forward_32(const MlpWeights& w, const IonDev& io, bool have,
+                                            double emag, int z, double ne, double te) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int zc = z < 0 ? 0 : (z < kNO ? z : kNO - 1);
+  float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (have) features_of(io, emag, zc, ne, te, x);
+  const uint32_t f01 = pack_bf16(x[0], x[1]), f23 = pack_bf16(x[2], x[3]);
+  float y = 0.0f;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t xr[2];
+    int zr[2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int src = 16 * h + 8 * r + g;
+      const uint32_t a = __shfl_sync(0xffffffffu, f01, src), b = __shfl_sync(0xffffffffu, f23, src);
+      xr[r] = t == 0 ? a : (t == 1 ? b : 0u);
+      zr[r] = __shfl_sync(0xffffffffu, zc, src);
+    }
+    float ysel[2];
+    forward_sel(w, xr[0], xr[1], zr[0], zr[1], ysel);
+    // every lane of quad g holds rows g and g + 8: sample l = 16 h + 8 r + g
+    const int from = 4 * (lane & 7);
+    const float lo = __shfl_sync(0xffffffffu, ysel[0], from);
+    const float hi = __shfl_sync(0xffffffffu, ysel[1], from);
+    if ((lane >> 4) == h) y = (lane & 8) ? hi : lo;
+  }
+  return y;
+}
+
 // ------------------------------------------------------------ inference --
 
 __global__ void __launch_bounds__(32 * kWarps) k_mlp_forward(const float* __restrict__ p,
                                                              const float* __restrict__ feats,
                                                              long long n, float* __restrict__ y) {
   __shared__ MlpWeights w;
-  load_weights(p, w);
+  load_weights<32 * kWarps>(p, w);
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const long long tiles = (n + 15) / 16;
@@ -270,40 +311,23 @@ __global__ void __launch_bounds__(32 * kWarps) k_ion_mlp_rates(const IonArgs a) 
   const long long step = __ldcg(a.step);
   if (a.ion.rate_model != 2) return;
   if (!a.force && !(a.ion.ionize_every > 0 && step % a.ion.ionize_every == 0)) return;
-  load_weights(a.mlp, w);
+  load_weights<32 * kWarps>(a.mlp, w);
   __syncthreads();
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const long long n = a.ion.n_ions;
-  const long long tiles = (n + 15) / 16;
+  const long long tiles = (n + 31) / 32;
   for (long long tile = static_cast<long long>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
        tile < tiles; tile += static_cast<long long>(gridDim.x) * kWarps) {
-    const long long s[2] = {tile * 16 + g, tile * 16 + g + 8};
-    float x[2][4];
-    int zs[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      zs[h] = -1;
-      x[h][0] = x[h][1] = x[h][2] = x[h][3] = 0.0f;
-      if (s[h] < n) {
-        const double* o = a.out + 4 * s[h];
-        zs[h] = a.zq[a.c.off + s[h]];
-        features_of(a.ion, o[0], zs[h] < 0 ? 0 : (zs[h] < kNO ? zs[h] : kNO - 1), o[1], o[2],
-                    x[h]);
-      }
-    }
-    float ysel[2];
-    forward_sel(w, x[0], x[1], zs[0] < 0 ? 0 : (zs[0] < kNO ? zs[0] : kNO - 1),
-                zs[1] < 0 ? 0 : (zs[1] < kNO ? zs[1] : kNO - 1), ysel);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (t != 0 || s[h] >= n || zs[h] < 0 || zs[h] >= a.ion.zmax) continue;
-      const double* o = a.out + 4 * s[h];
-      const bool inside = o[0] >= a.ion.dom[0] && o[0] <= a.ion.dom[1] &&
-                          (o[1] == 0.0 || (o[1] >= a.ion.dom[2] && o[1] <= a.ion.dom[3])) &&
-                          (o[1] == 0.0 || (o[2] >= a.ion.dom[4] && o[2] <= a.ion.dom[5]));
-      if (!inside) continue;
-      a.nu[s[h]] = rate_of_output(ysel[h]);
-    }
+    const long long k = tile * 32 + (threadIdx.x & 31);
+    const bool have = k < n;
+    const double* o = a.out + 4 * k;
+    const double e = have ? o[0] : 0.0, ne = have ? o[1] : 0.0, te = have ? o[2] : 0.0;
+    const int z = have ? a.zq[a.c.off + k] : -1;
+    const float y = forward_32(w, a.ion, have, e, z, ne, te);
+    if (!have || z < 0 || z >= a.ion.zmax) continue;
+    const bool inside = e >= a.ion.dom[0] && e <= a.ion.dom[1] &&
+                        (ne == 0.0 || (ne >= a.ion.dom[2] && ne <= a.ion.dom[3])) &&
+                        (ne == 0.0 || (te >= a.ion.dom[4] && te <= a.ion.dom[5]));
+    if (inside) a.nu[k] = rate_of_output(y);
   }
 }
 
@@ -311,13 +335,16 @@ __global__ void __launch_bounds__(32 * kWarps) k_ion_mlp_rates(const IonArgs a) 
 
 // Per-warp staging for the weight gradients: x and h1 (BF16-rounded, as the
 // tensor-core layers use them), h2 (FP32), dy, da1, da2 of 16 samples.
+// (rows padded by 8 words: the eight rows that a warp stores to at once lie in
+// different banks)
+constexpr int kStRow = kNH + 8;
 struct WarpStage {
-  float x[16][kNI];
-  float h1[16][kNH];
-  float h2[16][kNH];
-  float dy[16][kNO];
-  float da1[16][kNH];
-  float da2[16][kNH];
+  alignas(16) float x[16][kNI];
+  alignas(16) float h1[16][kStRow];
+  alignas(16) float h2[16][kStRow];
+  alignas(16) float dy[16][kNO];
+  alignas(16) float da1[16][kStRow];
+  alignas(16) float da2[16][kStRow];
 };
 
 struct TrainSmem {
@@ -337,7 +364,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
                                                            float* __restrict__ loss_part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-  load_weights(p, S.w);
+  load_weights<32 * kWarps>(p, S.w);
   __syncthreads();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const float coef = 2.0f / static_cast<float>(nb);
@@ -397,16 +424,14 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
 #pragma unroll
       for (int q = 0; q < 4; ++q) dh[j][q] *= dsilu(f.a2[j][q]);
       const int c0 = 8 * j + 2 * t;
-      st.da2[g][c0] = dh[j][0]; st.da2[g][c0 + 1] = dh[j][1];
-      st.da2[g + 8][c0] = dh[j][2]; st.da2[g + 8][c0 + 1] = dh[j][3];
-      st.h2[g][c0] = silu(f.a2[j][0]);
-      st.h2[g][c0 + 1] = silu(f.a2[j][1]);
-      st.h2[g + 8][c0] = silu(f.a2[j][2]);
-      st.h2[g + 8][c0 + 1] = silu(f.a2[j][3]);
-      st.h1[g][c0] = bf16_round(silu(f.a1[j][0]));
-      st.h1[g][c0 + 1] = bf16_round(silu(f.a1[j][1]));
-      st.h1[g + 8][c0] = bf16_round(silu(f.a1[j][2]));
-      st.h1[g + 8][c0 + 1] = bf16_round(silu(f.a1[j][3]));
+      auto put = [&](float (&to)[16][kStRow], float v0, float v1, float v2, float v3) {
+        *reinterpret_cast<float2*>(&to[g][c0]) = make_float2(v0, v1);
+        *reinterpret_cast<float2*>(&to[g + 8][c0]) = make_float2(v2, v3);
+      };
+      put(st.da2, dh[j][0], dh[j][1], dh[j][2], dh[j][3]);
+      put(st.h2, silu(f.a2[j][0]), silu(f.a2[j][1]), silu(f.a2[j][2]), silu(f.a2[j][3]));
+      put(st.h1, bf16_round(silu(f.a1[j][0])), bf16_round(silu(f.a1[j][1])),
+          bf16_round(silu(f.a1[j][2])), bf16_round(silu(f.a1[j][3])));
     }
     st.dy[g][2 * t] = dy[0]; st.dy[g][2 * t + 1] = dy[1];
     st.dy[g + 8][2 * t] = dy[2]; st.dy[g + 8][2 * t + 1] = dy[3];
@@ -431,10 +456,10 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
         mma_bf16(d1, da[kk][0], da[kk][1], da[kk][2], da[kk][3], bb0, bb1);
       }
       const int c0 = 8 * j + 2 * t;
-      st.da1[g][c0] = d1[0] * dsilu(f.a1[j][0]);
-      st.da1[g][c0 + 1] = d1[1] * dsilu(f.a1[j][1]);
-      st.da1[g + 8][c0] = d1[2] * dsilu(f.a1[j][2]);
-      st.da1[g + 8][c0 + 1] = d1[3] * dsilu(f.a1[j][3]);
+      *reinterpret_cast<float2*>(&st.da1[g][c0]) =
+          make_float2(d1[0] * dsilu(f.a1[j][0]), d1[1] * dsilu(f.a1[j][1]));
+      *reinterpret_cast<float2*>(&st.da1[g + 8][c0]) =
+          make_float2(d1[2] * dsilu(f.a1[j][2]), d1[3] * dsilu(f.a1[j][3]));
     }
     if (t == 0) {
 #pragma unroll
@@ -447,12 +472,23 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
     // weight gradients of the CTA's 64 samples, in sample order
     for (int wv = 0; wv < kWarps; ++wv) {
       const WarpStage& sw = S.st[wv];
+#pragma unroll 4
       for (int s = 0; s < 16; ++s) {
+        // this thread's column of 32 (W2) and 4 (W3) neighbouring rows
         const float h1k = sw.h1[s][kcol], h2k = sw.h2[s][kcol];
 #pragma unroll
-        for (int m = 0; m < 32; ++m) gw2[m] = fmaf(sw.da2[s][nrow + 2 * m], h1k, gw2[m]);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) gw3[m] = fmaf(sw.dy[s][nrow + 2 * m], h2k, gw3[m]);
+        for (int m = 0; m < 32; m += 4) {
+          const float4 d = *reinterpret_cast<const float4*>(&sw.da2[s][32 * nrow + m]);
+          gw2[m] = fmaf(d.x, h1k, gw2[m]);
+          gw2[m + 1] = fmaf(d.y, h1k, gw2[m + 1]);
+          gw2[m + 2] = fmaf(d.z, h1k, gw2[m + 2]);
+          gw2[m + 3] = fmaf(d.w, h1k, gw2[m + 3]);
+        }
+        const float4 dy4 = *reinterpret_cast<const float4*>(&sw.dy[s][4 * nrow]);
+        gw3[0] = fmaf(dy4.x, h2k, gw3[0]);
+        gw3[1] = fmaf(dy4.y, h2k, gw3[1]);
+        gw3[2] = fmaf(dy4.z, h2k, gw3[2]);
+        gw3[3] = fmaf(dy4.w, h2k, gw3[3]);
         const float xk = sw.x[s][tid & 3];
         gw1[0] = fmaf(sw.da1[s][tid >> 2], xk, gw1[0]);
         gw1[1] = fmaf(sw.da1[s][(tid >> 2) + 32], xk, gw1[1]);
@@ -465,9 +501,9 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
   // per-CTA partials: [blockIdx][kNParam]
   float* out = part + static_cast<long long>(blockIdx.x) * kNParam;
 #pragma unroll
-  for (int m = 0; m < 32; ++m) out[kOffW2 + (nrow + 2 * m) * kNH + kcol] = gw2[m];
+  for (int m = 0; m < 32; ++m) out[kOffW2 + (32 * nrow + m) * kNH + kcol] = gw2[m];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) out[kOffW3 + (nrow + 2 * m) * kNH + kcol] = gw3[m];
+  for (int m = 0; m < 4; ++m) out[kOffW3 + (4 * nrow + m) * kNH + kcol] = gw3[m];
   out[kOffW1 + (tid >> 2) * kNI + (tid & 3)] = gw1[0];
   out[kOffW1 + ((tid >> 2) + 32) * kNI + (tid & 3)] = gw1[1];
   if (tid < 64) out[kOffB1 + tid] = gb; else out[kOffB2 + tid - 64] = gb;
@@ -529,13 +565,41 @@ __global__ void k_mlp_init(float* p, unsigned long long seed) {
   p[e] = static_cast<float>(a * (2.0 * u - 1.0));
 }
 
-// Sum of the per-CTA gradient partials in CTA order, then one Adam step.
-__global__ void k_mlp_adam(float* p, float* m, float* v, const float* part, int nparts,
-                           float lr, float b1, float b2, float eps, int step, float* grad_out) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= kNParam) return;
+// Sum of the per-CTA gradient partials in a fixed order, then one Adam step: 32
+// parameters per CTA, each of eight warps adds every eighth partial (a thread
+// per parameter over all partials one after the other: 8 us of a 31 us step).
+// The CTA after those adds the loss partials if loss_out is given.
+constexpr int kAdamWarps = 8;
+constexpr int kAdamBlocks = (kNParam + 31) / 32;
+
+__global__ void __launch_bounds__(32 * kAdamWarps)
+    k_mlp_adam(float* p, float* m, float* v, const float* part, int nparts, float lr, float b1,
+               float b2, float eps, int step, float* grad_out, const float* lpart,
+               float* loss_out) {
+  __shared__ float s_g[kAdamWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool is_loss = blockIdx.x == kAdamBlocks;
+  const int e = blockIdx.x * 32 + lane;
   float g = 0.0f;
-  for (int k = 0; k < nparts; ++k) g += part[static_cast<long long>(k) * kNParam + e];
+  if (is_loss) {
+    for (int k = threadIdx.x; k < nparts; k += 32 * kAdamWarps) g += lpart[k];
+  } else if (e < kNParam) {
+#pragma unroll 8
+    for (int k = warp; k < nparts; k += kAdamWarps) g += part[static_cast<long long>(k) * kNParam + e];
+  }
+  s_g[warp][lane] = g;
+  __syncthreads();
+  if (warp != 0) return;
+  g = 0.0f;
+#pragma unroll
+  for (int k = 0; k < kAdamWarps; ++k) g += s_g[k][lane];
+  if (is_loss) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) g += __shfl_down_sync(0xffffffffu, g, o);
+    if (lane == 0) *loss_out = g;
+    return;
+  }
+  if (e >= kNParam) return;
   if (grad_out) grad_out[e] = g;
   if (lr <= 0.0f) return;
   const float mk = b1 * m[e] + (1.0f - b1) * g;
@@ -547,49 +611,32 @@ __global__ void k_mlp_adam(float* p, float* m, float* v, const float* part, int 
   p[e] -= lr * mh / (sqrtf(vh) + eps);
 }
 
-__global__ void k_sum_floats(const float* x, int n, float* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  float s = 0.0f;
-  for (int k = 0; k < n; ++k) s += x[k];
-  *out = s;
-}
-
 // Rates of independent ions: surrogate inside the domain (model 2), -1 else.
+// Bound by the special-function unit (two per hidden unit); a CTA takes several
+// tiles, so that the weights' conversion is not paid per 64 ions.  200000 ions:
+// 68 us with a CTA per 64 ions, features formed by all four lanes of a quad and
+// eight-way bank conflicts on the weights, 25 us now.
 __global__ void __launch_bounds__(32 * kWarps) k_rates_mlp(IonDev io, const float* __restrict__ p,
                                                            const double* emag, const int* zs,
                                                            const double* ne, const double* te,
                                                            long long n, double* nu) {
   __shared__ MlpWeights w;
-  load_weights(p, w);
+  load_weights<32 * kWarps>(p, w);
   __syncthreads();
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const long long tiles = (n + 15) / 16;
+  const long long tiles = (n + 31) / 32;
   for (long long tile = static_cast<long long>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
        tile < tiles; tile += static_cast<long long>(gridDim.x) * kWarps) {
-    const long long s[2] = {tile * 16 + g, tile * 16 + g + 8};
-    float x[2][4];
-    int z[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      z[h] = s[h] < n ? zs[s[h]] : 0;
-      x[h][0] = x[h][1] = x[h][2] = x[h][3] = 0.0f;
-      if (s[h] < n)  // out-of-range charges get a valid row here and no surrogate rate below
-        features_of(io, emag[s[h]], z[h] < 0 ? 0 : (z[h] < kNO ? z[h] : kNO - 1), ne[s[h]],
-                    te[s[h]], x[h]);
-    }
-    float ysel[2];
-    forward_sel(w, x[0], x[1], z[0] < 0 ? 0 : (z[0] < kNO ? z[0] : kNO - 1),
-                z[1] < 0 ? 0 : (z[1] < kNO ? z[1] : kNO - 1), ysel);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (t != 0 || s[h] >= n) continue;  // lane t = 0 of the quad writes
-      const long long k = s[h];
-      const bool inside = z[h] >= 0 && z[h] < io.zmax && emag[k] >= io.dom[0] &&
-                          emag[k] <= io.dom[1] &&
-                          (ne[k] == 0.0 || (ne[k] >= io.dom[2] && ne[k] <= io.dom[3] &&
-                                            te[k] >= io.dom[4] && te[k] <= io.dom[5]));
-      nu[k] = inside ? rate_of_output(ysel[h]) : -1.0;
-    }
+    const long long k = tile * 32 + (threadIdx.x & 31);
+    const bool have = k < n;
+    const double e = have ? emag[k] : 0.0, d = have ? ne[k] : 0.0, tt = have ? te[k] : 0.0;
+    const int z = have ? zs[k] : 0;
+    // (out-of-range charges get a valid row and no surrogate rate)
+    const float y = forward_32(w, io, have, e, z, d, tt);
+    if (!have) continue;
+    const bool inside = z >= 0 && z < io.zmax && e >= io.dom[0] && e <= io.dom[1] &&
+                        (d == 0.0 || (d >= io.dom[2] && d <= io.dom[3] && tt >= io.dom[4] &&
+                                      tt <= io.dom[5]));
+    nu[k] = inside ? rate_of_output(y) : -1.0;
   }
 }
 
@@ -612,6 +659,20 @@ int train_grid() {
     g = 2 * (sms > 0 ? sms : 1);
   }
   return g;
+}
+
+// CTAs of a minibatch of n samples: one per tile (up to two per SM); more would
+// only add zero partials.
+int train_ctas(long long n) {
+  return static_cast<int>(std::max<long long>(
+      1, std::min<long long>(train_grid(), (n + kTileSamples - 1) / kTileSamples)));
+}
+
+// CTAs of the inference kernels for n samples in tiles of `tile` per warp: four
+// per SM, each looping over its tiles.
+unsigned infer_ctas(long long n, int tile) {
+  const long long want = ((n + tile - 1) / tile + kWarps - 1) / kWarps;
+  return static_cast<unsigned>(std::max<long long>(1, std::min<long long>(want, 2 * train_grid())));
 }
 
 cudaError_t train_smem_attr() {
@@ -657,9 +718,7 @@ md_status check_train_config(const md_mlp_train_config* c) {
 
 cudaError_t launch_ion_mlp(const IonArgs& a, cudaStream_t s) {
   if (!a.mlp) return cudaErrorInvalidValue;
-  const long long tiles = (a.ion.n_ions + 15) / 16;
-  const unsigned grid = static_cast<unsigned>((tiles + kWarps - 1) / kWarps);
-  k_ion_mlp_rates<<<grid, 32 * kWarps, 0, s>>>(a);
+  k_ion_mlp_rates<<<infer_ctas(a.ion.n_ions, 32), 32 * kWarps, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -681,10 +740,7 @@ static md_status md_mlp_forward_device_body(const float* params, const float* fe
   if (n < 0) return report_error(MD_ERR_ARG, "n < 0");
   if (n == 0) return MD_OK;
   if (!params || !feats || !y) return report_error(MD_ERR_ARG, "NULL pointer");
-  const long long tiles = (n + 15) / 16;
-  const unsigned grid = static_cast<unsigned>(
-      std::min<long long>((tiles + md::kWarps - 1) / md::kWarps, 4096));
-  md::k_mlp_forward<<<grid, 32 * md::kWarps, 0, static_cast<cudaStream_t>(stream)>>>(params, feats,
+  md::k_mlp_forward<<<md::infer_ctas(n, 16), 32 * md::kWarps, 0, static_cast<cudaStream_t>(stream)>>>(params, feats,
                                                                                    n, y);
   MLP_CUDA(cudaGetLastError());
   return MD_OK;
@@ -702,7 +758,7 @@ static md_status md_mlp_loss_grad_device_body(const float* params, const float* 
   if (!params || !feats || !z || !target || !grad) return report_error(MD_ERR_ARG, "NULL pointer");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   MLP_CUDA(md::train_smem_attr());
-  const int grid = md::train_grid();
+  const int grid = md::train_ctas(n);
   float* part = nullptr;
   float* lpart = nullptr;
   MLP_CUDA(cudaMalloc(reinterpret_cast<void**>(&part), sizeof(float) * grid * md::kNParam));
@@ -713,12 +769,8 @@ static md_status md_mlp_loss_grad_device_body(const float* params, const float* 
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
-    md::k_mlp_adam<<<(md::kNParam + 255) / 256, 256, 0, s>>>(nullptr, nullptr, nullptr, part, grid,
-                                                            0.0f, 0.f, 0.f, 0.f, 1, grad);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && loss) {
-    md::k_sum_floats<<<1, 1, 0, s>>>(lpart, grid, loss);
+    md::k_mlp_adam<<<md::kAdamBlocks + (loss ? 1 : 0), 32 * md::kAdamWarps, 0, s>>>(
+        nullptr, nullptr, nullptr, part, grid, 0.0f, 0.f, 0.f, 0.f, 1, grad, lpart, loss);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -766,10 +818,7 @@ static md_status md_ion_rates_device_body(const md_mlp_train_config* cfg, int32_
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const md::IonDev io = md::domain_io(*cfg);
   if (model == 2) {
-    const long long tiles = (n + 15) / 16;
-    const unsigned grid = static_cast<unsigned>(
-        std::min<long long>((tiles + md::kWarps - 1) / md::kWarps, 8192));
-    md::k_rates_mlp<<<grid, 32 * md::kWarps, 0, s>>>(io, params, emag, z, ne, te, n, nu);
+    md::k_rates_mlp<<<md::infer_ctas(n, 32), 32 * md::kWarps, 0, s>>>(io, params, emag, z, ne, te, n, nu);
     MLP_CUDA(cudaGetLastError());
   }
   md::k_rates_plain<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(io, emag, z, ne, te, n,
@@ -795,10 +844,7 @@ static md_status md_mlp_train_body(const md_mlp_train_config* cfg, float* params
   MLP_CUDA(md::train_smem_attr());
   const long long n = cfg->n_samples;
   const long long nh = std::max<long long>(4096, n / 20);  // held-out set
-  // one CTA per tile of the minibatch (up to two per SM): more CTAs would only
-  // add zero partials for the Adam kernel to sum
-  const int grid = static_cast<int>(std::max<long long>(1, std::min<long long>(
-      md::train_grid(), (cfg->batch + md::kTileSamples - 1) / md::kTileSamples)));
+  const int grid = md::train_ctas(cfg->batch);
   float *feats = nullptr, *target = nullptr, *hfeats = nullptr, *htarget = nullptr, *hy = nullptr;
   int *zs = nullptr, *hz = nullptr;
   float *p = nullptr, *m = nullptr, *v = nullptr, *part = nullptr, *lpart = nullptr,
@@ -852,12 +898,12 @@ static md_status md_mlp_train_body(const md_mlp_train_config* cfg, float* params
       const float lr = static_cast<float>(cfg->lr * (0.01 + 0.99 * 0.5 * (1.0 + std::cos(3.14159265358979323846 * prog))));
       md::k_mlp_train<<<grid, 32 * md::kWarps, sizeof(md::TrainSmem), s>>>(p, feats, zs, target,
                                                                            b0, nb, part, lpart);
-      md::k_mlp_adam<<<(md::kNParam + 255) / 256, 256, 0, s>>>(p, m, v, part, grid, lr, 0.9f,
-                                                              0.999f, 1e-8f,
-                                                              static_cast<int>(step), nullptr);
+      const bool want_loss = b == batches - 1 || (ep == 0 && b == 0);
+      md::k_mlp_adam<<<md::kAdamBlocks + (want_loss ? 1 : 0), 32 * md::kAdamWarps, 0, s>>>(
+          p, m, v, part, grid, lr, 0.9f, 0.999f, 1e-8f, static_cast<int>(step), nullptr, lpart,
+          lsum);
       e = cudaGetLastError();
-      if (b == batches - 1 || (ep == 0 && b == 0)) {
-        md::k_sum_floats<<<1, 1, 0, s>>>(lpart, grid, lsum);
+      if (want_loss) {
         float l = 0.0f;
         if (e == cudaSuccess) e = cudaMemcpyAsync(&l, lsum, sizeof(float), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -867,8 +913,7 @@ static md_status md_mlp_train_body(const md_mlp_train_config* cfg, float* params
   }
   cudaEventRecord(e1, s);
   if (e == cudaSuccess) {
-    md::k_mlp_forward<<<std::min<long long>((nh / 16 + md::kWarps) / md::kWarps + 1, 4096),
-                        32 * md::kWarps, 0, s>>>(p, hfeats, nh, hy);
+    md::k_mlp_forward<<<md::infer_ctas(nh, 16), 32 * md::kWarps, 0, s>>>(p, hfeats, nh, hy);
     e = cudaGetLastError();
   }
   std::vector<float> h_y(8 * nh), h_t(nh);
