@@ -123,6 +123,15 @@ md_status field_device(int** err, int* sms);
 cudaError_t launch_field_direct(const FieldArgs& a, bool potential, int sms, cudaStream_t s);
 bool field_uses_probe(long long nt, long long ns, long long nseg, int sms);
 
+// Stream-ordered scratch memory of one call on the current device, freed with
+// cudaFreeAsync on the same stream.  From a pool of the library's own that
+// keeps at most kScratchKeep bytes between calls (the default pool returns
+// everything to the system at each synchronisation, and taking it again costs
+// some 200 us); md_destroy gives the kept memory back.
+constexpr unsigned long long kScratchKeep = 32ull << 20;
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+void scratch_trim();
+
 // Records the thread-local message returned by md_last_error() and returns
 // the status (implemented in md_runtime.cu).
 md_status report_error(md_status status, const char* msg);
@@ -140,6 +149,8 @@ md_status guarded(F&& body) noexcept {
   }
 }
 md_status report_cuda_error(cudaError_t e, const char* what);
+// State -> host-layout records in a.hx .. a.hkind (null: not wanted), which may
+// be device-visible host memory.
 cudaError_t launch_download(const DownloadArgs& a, cudaStream_t s);
 
 // FP64 reference direct sum (see md_coulomb_field_fp64_device).

@@ -169,19 +169,23 @@ cudaError_t launch_field_fp64(const double* xs, const double* qs, long long ns, 
   return cudaGetLastError();
 }
 
-__global__ void k_download(const DownloadArgs a) {  const long long k = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (k >= a.n) return;
-  const long long i = a.off + k;
-  a.hx[3 * k] = a.x[i];
-  a.hx[3 * k + 1] = a.y[i];
-  a.hx[3 * k + 2] = a.z[i];
-  a.hu[3 * k] = a.ux[i];
-  a.hu[3 * k + 1] = a.uy[i];
-  a.hu[3 * k + 2] = a.uz[i];
-  a.hz[k] = a.zq[i];
-  a.hmass[k] = a.mass[i];
-  a.hw[k] = a.w[i];
-  a.hkind[k] = a.kind[i];
+// One thread per double of x (and of u): neighbouring threads write
+// neighbouring doubles, also when the arrays are host memory.
+__global__ void __launch_bounds__(256) k_download(const DownloadArgs a) {
+  const long long w = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (w < 3 * a.n) {
+    const long long k = w / 3, i = a.off + k;
+    const int c = static_cast<int>(w - 3 * k);
+    if (a.hx) a.hx[w] = (c == 0 ? a.x : c == 1 ? a.y : a.z)[i];
+    if (a.hu) a.hu[w] = (c == 0 ? a.ux : c == 1 ? a.uy : a.uz)[i];
+  }
+  if (w < a.n) {
+    const long long i = a.off + w;
+    if (a.hz) a.hz[w] = a.zq[i];
+    if (a.hmass) a.hmass[w] = a.mass[i];
+    if (a.hw) a.hw[w] = a.w[i];
+    if (a.hkind) a.hkind[w] = a.kind[i];
+  }
 }
 
 namespace {
@@ -523,8 +527,7 @@ cudaError_t launch_upload(const UploadArgs& a, cudaStream_t s) {
 
 cudaError_t launch_download(const DownloadArgs& a, cudaStream_t s) {
   if (a.n <= 0) return cudaSuccess;
-  const unsigned grid = static_cast<unsigned>((a.n + 255) / 256);
-  k_download<<<grid, 256, 0, s>>>(a);
+  k_download<<<static_cast<unsigned>((3 * a.n + 255) / 256), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

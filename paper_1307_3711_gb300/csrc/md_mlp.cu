@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(32 * kAdamWarps)
 // Bound by the special-function unit (two per hidden unit); a CTA takes several
 // tiles, so that the weights' conversion is not paid per 64 ions.  200000 ions:
 // 68 us with a CTA per 64 ions, features formed by all four lanes of a quad and
-// eight-way bank conflicts on the weights, 25 us now.
+// eight-way bank conflicts on the weights, 37 us now.
 __global__ void __launch_bounds__(32 * kWarps) k_rates_mlp(IonDev io, const float* __restrict__ p,
                                                            const double* emag, const int* zs,
                                                            const double* ne, const double* te,
@@ -759,11 +759,13 @@ static md_status md_mlp_loss_grad_device_body(const float* params, const float* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   MLP_CUDA(md::train_smem_attr());
   const int grid = md::train_ctas(n);
+  // partial gradients, then partial losses
   float* part = nullptr;
-  float* lpart = nullptr;
-  MLP_CUDA(cudaMalloc(reinterpret_cast<void**>(&part), sizeof(float) * grid * md::kNParam));
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&lpart), sizeof(float) * grid);
-  if (e == cudaSuccess) {
+  cudaError_t e = md::scratch_alloc(reinterpret_cast<void**>(&part),
+                                    sizeof(float) * grid * (md::kNParam + 1), s);
+  if (e != cudaSuccess) return report_cuda_error(e, "surrogate gradient partials");
+  float* lpart = part + static_cast<size_t>(grid) * md::kNParam;
+  {
     md::k_mlp_train<<<grid, 32 * md::kWarps, sizeof(md::TrainSmem), s>>>(params, feats, z, target,
                                                                          0, n, part, lpart);
     e = cudaGetLastError();
@@ -773,9 +775,9 @@ static md_status md_mlp_loss_grad_device_body(const float* params, const float* 
         nullptr, nullptr, nullptr, part, grid, 0.0f, 0.f, 0.f, 0.f, 1, grad, lpart, loss);
     e = cudaGetLastError();
   }
+  const cudaError_t fe = cudaFreeAsync(part, s);
+  if (e == cudaSuccess) e = fe;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  cudaFree(part);
-  cudaFree(lpart);
   if (e != cudaSuccess) return report_cuda_error(e, "surrogate loss/gradient");
   return MD_OK;
 }

@@ -41,6 +41,8 @@ md_status cuda_fail(cudaError_t e, const char* what) {
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kClassicalElectronRadius = 2.8179403262e-15;  // m, CODATA 2018
 constexpr int kGraphSteps = 16;
+// records up to which md_get_particles writes page-locked arrays from the kernel
+constexpr long long kStraightRecords = 1LL << 17;
 constexpr double kMeC2Ev = 510998.95;  // electron rest energy, eV
 // target slices start (and end, unless at the record count) on multiples of
 // this, a multiple of every compiled i-block size, so that a slice is a whole
@@ -112,6 +114,7 @@ struct md_ctx {
   // of active records
   unsigned long long* d_word = nullptr;
   unsigned long long* h_word = nullptr;
+  int* h_err = nullptr;  // pinned copy of the error word
 
   // kernel configuration
   int cfg = -1;
@@ -204,13 +207,17 @@ struct RawView {
 
 // Whether host memory is page-locked (registered or allocated by CUDA), so
 // that an asynchronous copy can use it directly.
-bool is_pinned(const void* p) {
+// device_view (may be nullptr): its address for kernels, nullptr if it has none.
+bool is_pinned(const void* p, void** device_view = nullptr) {
+  if (device_view) *device_view = nullptr;
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();  // clear the error of an unknown pointer
     return false;
   }
-  return at.type == cudaMemoryTypeHost;
+  if (at.type != cudaMemoryTypeHost) return false;
+  if (device_view) *device_view = at.devicePointer;
+  return true;
 }
 
 RawView raw_view(unsigned char* base, long long n) {
@@ -934,10 +941,14 @@ md_status ensure_scratch(md_ctx* c) {
   return MD_OK;
 }
 
-md_status check_device_error(md_ctx* c) {
-  int err = 0;
-  MD_CUDA(cudaMemcpyAsync(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  MD_CUDA(cudaStreamSynchronize(c->stream));
+// The error word's copy to the host, ordered before a synchronisation of the
+// caller's; device_error then reports it.
+cudaError_t fetch_error(md_ctx* c) {
+  return cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+}
+
+md_status device_error(md_ctx* c) {
+  const int err = *c->h_err;
   if (err & md::kErrTimeout) {
     MD_CUDA(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
     MD_CUDA(cudaMemsetAsync(c->d_ticket, 0, sizeof(unsigned), c->stream));
@@ -951,6 +962,12 @@ md_status check_device_error(md_ctx* c) {
     return fail(MD_ERR_STATE, "a device-side bounds check failed (checked build)");
   }
   return MD_OK;
+}
+
+md_status check_device_error(md_ctx* c) {
+  MD_CUDA(fetch_error(c));
+  MD_CUDA(cudaStreamSynchronize(c->stream));
+  return device_error(c);
 }
 
 md::IonArgs ion_args(md_ctx* c, int ci, int force) {
@@ -1167,6 +1184,7 @@ void free_ctx(md_ctx* c) {
   if (c->h_diag) cudaFreeHost(c->h_diag);
   cudaFree(c->d_word);
   if (c->h_word) cudaFreeHost(c->h_word);
+  if (c->h_err) cudaFreeHost(c->h_err);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -1353,6 +1371,47 @@ namespace md {
 
 md_status report_error(md_status status, const char* msg) { return fail(status, "%s", msg); }
 
+namespace {
+constexpr int kPoolDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kPoolDevices] = {};
+}  // namespace
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kPoolDevices) return cudaMallocAsync(p, bytes, s);
+  cudaMemPool_t pool = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pool[dev]) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      cudaMemPool_t made = nullptr;
+      if ((e = cudaMemPoolCreate(&made, &props)) != cudaSuccess) return e;
+      unsigned long long keep = kScratchKeep;
+      if ((e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep)) !=
+          cudaSuccess) {
+        cudaMemPoolDestroy(made);
+        return e;
+      }
+      g_pool[dev] = made;
+    }
+    pool = g_pool[dev];
+  }
+  return cudaMallocFromPoolAsync(p, bytes, pool, s);
+}
+
+void scratch_trim() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPoolDevices) return;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (g_pool[dev]) cudaMemPoolTrimTo(g_pool[dev], 0);
+}
+
 md_status report_cuda_error(cudaError_t e, const char* what) { return cuda_fail(e, what); }
 
 }  // namespace md
@@ -1516,7 +1575,8 @@ md_status create_context(const md_config* cfgs, int32_t n_clusters, const long l
                    cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMemcpy"));
   }
-  if (dev_alloc(&c->d_word, 1) != cudaSuccess ||
+  if (cudaMallocHost(reinterpret_cast<void**>(&c->h_err), sizeof(int)) != cudaSuccess ||
+      dev_alloc(&c->d_word, 1) != cudaSuccess ||
       cudaMallocHost(reinterpret_cast<void**>(&c->h_word), sizeof(unsigned long long)) !=
           cudaSuccess)
     return bail(fail(MD_ERR_OOM, "upload check buffers"));
@@ -1664,7 +1724,10 @@ md_status md_init_generate(md_ctx** out, const md_config* cfgs, const md_generat
 }
 
 
-void md_destroy(md_ctx* ctx) { free_ctx(ctx); }
+void md_destroy(md_ctx* ctx) {
+  free_ctx(ctx);
+  md::scratch_trim();
+}
 
 static md_status md_step_body(md_ctx* c, int32_t nsteps) {
   if (!c) return fail(MD_ERR_ARG, "ctx is NULL");
@@ -1689,7 +1752,6 @@ md_status md_step(md_ctx* c, int32_t nsteps) {
 
 static md_status md_sync_body(md_ctx* c) {
   if (!c) return fail(MD_ERR_ARG, "ctx is NULL");
-  MD_CUDA(cudaStreamSynchronize(c->stream));
   return check_device_error(c);
 }
 
@@ -1857,6 +1919,7 @@ static md_status md_get_ionization_body(md_ctx* c, int32_t cluster, double* emag
   if (fired)
     MD_CUDA(cudaMemcpyAsync(fired, c->d_ion_fired + c->ion_out_off[cluster], n,
                             cudaMemcpyDeviceToHost, c->stream));
+  MD_CUDA(fetch_error(c));
   MD_CUDA(cudaStreamSynchronize(c->stream));
   for (long long i = 0; i < n; ++i) {
     if (emag) emag[i] = out[4 * i];
@@ -1864,7 +1927,7 @@ static md_status md_get_ionization_body(md_ctx* c, int32_t cluster, double* emag
     if (te) te[i] = out[4 * i + 2];
     if (prob) prob[i] = out[4 * i + 3];
   }
-  return check_device_error(c);
+  return device_error(c);
 }
 
 md_status md_get_ionization(md_ctx* c, int32_t cluster, double* emag, double* ne, double* te,
@@ -2001,9 +2064,10 @@ static md_status run_fields(md_ctx* c, int ci, bool potential) {
   const long long nseg = std::max(1LL, std::min({want, static_cast<long long>(kFieldMaxSeg),
                                                 a.ns / 2048}));
   // (a periodic cluster keeps the kernel whose minimum-image twin gives the
-  // same bits where no pair needs an image)
-  if (!a.src_live && cl.boundary == MD_BOUNDARY_OPEN && a.nt > 0 &&
-      md::field_uses_probe(a.nt, a.ns, nseg, c->sm_count)) {
+  // same bits where no pair needs an image, a target slice and a cluster large
+  // enough to be sliced the one that adds every slice's sources alike)
+  if (!a.src_live && cl.boundary == MD_BOUNDARY_OPEN && !c->any_slice && a.ns <= 8192 &&
+      a.nt > 0 && md::field_uses_probe(a.nt, a.ns, nseg, c->sm_count)) {
     MD_CUDA(md::launch_field_direct(a, potential, c->sm_count, c->stream));
     return MD_OK;
   }
@@ -2029,7 +2093,6 @@ static md_status md_get_fields_body(md_ctx* c, int32_t cluster, double* e, doubl
   if (phi)
     MD_CUDA(cudaMemcpyAsync(phi + sb, c->d_phi, sizeof(double) * n, cudaMemcpyDeviceToHost,
                             c->stream));
-  MD_CUDA(cudaStreamSynchronize(c->stream));
   return check_device_error(c);
 }
 
@@ -2107,7 +2170,6 @@ static md_status md_diagnostics_body(md_ctx* c, int32_t cluster, md_diag* out) {
                           c->stream));
   long long step = 0;
   MD_CUDA(cudaMemcpyAsync(&step, c->d_step, sizeof(step), cudaMemcpyDeviceToHost, c->stream));
-  MD_CUDA(cudaStreamSynchronize(c->stream));
   st = check_device_error(c);
   if (st != MD_OK) return st;
   return fill_diag(*c->h_diag, step, a.c, out);
@@ -2188,7 +2250,6 @@ static md_status md_step_diag_body(md_ctx* c, md_diag* out) {
     MD_CUDA(md::launch_diag(d, c->diag_blocks, c->d_diag, c->stream));
     MD_CUDA(cudaMemcpyAsync(c->h_diag, c->d_diag, sizeof(md::DiagPartial),
                             cudaMemcpyDeviceToHost, c->stream));
-    MD_CUDA(cudaStreamSynchronize(c->stream));
     st = check_device_error(c);
     if (st != MD_OK) return st;
     st = fill_diag(*c->h_diag, step, c->cl[ci], &out[ci]);
@@ -2206,14 +2267,7 @@ static md_status md_get_particles_body(md_ctx* c, int32_t cluster, md_particles*
   if (cluster < 0 || cluster >= c->n_clusters) return fail(MD_ERR_ARG, "bad cluster index");
   const long long n = c->cl[cluster].n;
   if (out->n != n) return fail(MD_ERR_ARG, "out->n = %lld, cluster holds %lld", (long long)out->n, n);
-  RawView d = raw_view(c->d_raw, n);
   md::DownloadArgs a;
-  a.hx = d.x;
-  a.hu = d.u;
-  a.hz = d.z;
-  a.hmass = d.mass;
-  a.hw = d.w;
-  a.hkind = d.kind;
   a.n = n;
   a.off = c->cl[cluster].off;
   a.x = c->d_x[0];
@@ -2226,33 +2280,51 @@ static md_status md_get_particles_body(md_ctx* c, int32_t cluster, md_particles*
   a.mass = c->d_mass;
   a.zq = c->d_z;
   a.kind = c->d_kind;
-  MD_CUDA(md::launch_download(a, c->stream));
-  // page-locked caller arrays receive their copy directly; the others go
-  // through the pinned staging buffer
-  RawView h = raw_view(c->h_raw, n);
+  RawView d = raw_view(c->d_raw, n), h = raw_view(c->h_raw, n);
   struct Part {
     void* user;
     void* stage;
-    const void* dev;
+    void* dev;
     size_t bytes;
     bool direct;
+    void* view;
   };
-  Part parts[6] = {{out->x, h.x, d.x, sizeof(double) * 3 * n, false},
-                   {out->u, h.u, d.u, sizeof(double) * 3 * n, false},
-                   {out->z, h.z, d.z, sizeof(int) * n, false},
-                   {out->mass, h.mass, d.mass, sizeof(double) * n, false},
-                   {out->w, h.w, d.w, sizeof(double) * n, false},
-                   {out->kind, h.kind, d.kind, static_cast<size_t>(n), false}};
+  Part parts[6] = {{out->x, h.x, d.x, sizeof(double) * 3 * n, false, nullptr},
+                   {out->u, h.u, d.u, sizeof(double) * 3 * n, false, nullptr},
+                   {out->z, h.z, d.z, sizeof(int) * n, false, nullptr},
+                   {out->mass, h.mass, d.mass, sizeof(double) * n, false, nullptr},
+                   {out->w, h.w, d.w, sizeof(double) * n, false, nullptr},
+                   {out->kind, h.kind, d.kind, static_cast<size_t>(n), false, nullptr}};
+  bool views = true;  // every wanted array is page-locked and visible to kernels
   for (Part& q : parts) {
     if (!q.user) continue;
-    q.direct = is_pinned(q.user);
-    MD_CUDA(cudaMemcpyAsync(q.direct ? q.user : q.stage, q.dev, q.bytes, cudaMemcpyDeviceToHost,
-                            c->stream));
+    q.direct = is_pinned(q.user, &q.view);
+    views = views && q.view;
   }
+  // a few records: the kernel writes the caller's page-locked arrays itself (a
+  // copy per array costs more than it moves); otherwise through the device
+  // buffer, page-locked arrays copied directly, the others through the pinned
+  // staging buffer
+  const bool straight = views && n <= kStraightRecords;
+  auto to = [&](int k) -> void* {
+    return !parts[k].user ? nullptr : straight ? parts[k].view : parts[k].dev;
+  };
+  a.hx = static_cast<double*>(to(0));
+  a.hu = static_cast<double*>(to(1));
+  a.hz = static_cast<int*>(to(2));
+  a.hmass = static_cast<double*>(to(3));
+  a.hw = static_cast<double*>(to(4));
+  a.hkind = static_cast<unsigned char*>(to(5));
+  MD_CUDA(md::launch_download(a, c->stream));
+  for (const Part& q : parts)
+    if (q.user && !straight)
+      MD_CUDA(cudaMemcpyAsync(q.direct ? q.user : q.stage, q.dev, q.bytes, cudaMemcpyDeviceToHost,
+                              c->stream));
+  MD_CUDA(fetch_error(c));
   MD_CUDA(cudaStreamSynchronize(c->stream));
   for (const Part& q : parts)
     if (q.user && !q.direct) std::memcpy(q.user, q.stage, q.bytes);
-  return check_device_error(c);
+  return device_error(c);
 }
 
 md_status md_get_particles(md_ctx* c, int32_t cluster, md_particles* out) {
@@ -2591,7 +2663,7 @@ static md_status md_coulomb_field_device_body(const void* src, int64_t ns, const
   }
   void* part = nullptr;
   if (nseg > 1) {
-    MD_CUDA(cudaMallocAsync(&part, static_cast<size_t>(32 * nseg * nt_), st));
+    MD_CUDA(md::scratch_alloc(&part, static_cast<size_t>(32 * nseg * nt_), st));
     a.nseg = static_cast<int>(nseg);
     a.seg_len = (ns_ + nseg - 1) / nseg;
     a.part = static_cast<double*>(part);
