@@ -1610,106 +1610,136 @@ __global__ void __launch_bounds__(THREADS) k_field(const FieldArgs a) {
 
 // ------------------------------------------------------- diagnostics (K4) --
 
-template <int THREADS>
-__device__ __forceinline__ double block_sum(double v, double* red) {
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < THREADS / 32; ++k) s += red[k];
-  return s;  // valid in thread 0
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// Per-block FP64 partial sums of the diagnostics of one cluster.
+// FP64 diagnostics of one cluster, per CTA.  Bound by latency: the former
+// version kept the charge histogram in dynamically indexed registers (local
+// memory) and reduced its 42 values one after the other with two barriers each
+// (85 us at 50000 records, and 36 us for one CTA to add the CTAs' partials).
+// Here a warp adds a charge state's weights with one shuffle sum for each state
+// its 32 records hold, lane z keeping state z; every value is then reduced
+// within its warp, and the warps' sums meet in shared memory once: 10 us, and 3
+// for the CTAs' partials.  Every order is fixed.
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS) k_diag_partial(const DiagArgs a) {
-  __shared__ double red[THREADS / 32];
-  const long long step = __ldcg(a.step);
-  const double t_n = a.c.t0 + static_cast<double>(step) * a.c.dt;
-  float las[6];
-  laser_field(a.c, t_n, las);
+  constexpr int kWarps = THREADS / 32;
+  __shared__ double s_v[kWarps][kDiagVals];
+  __shared__ float s_las[6];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (!a.rec) {
+    const long long step = __ldcg(a.step);
+    if (threadIdx.x == 0) laser_field(a.c, a.c.t0 + static_cast<double>(step) * a.c.dt, s_las);
+    __syncthreads();
+  }
   const float hq = 0.5f * static_cast<float>(a.c.dt);
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  long long na = 0, nbad = 0;
-  long long hist[kHistBins];
-  double histw[kHistBins];
+  double acc[7] = {0, 0, 0, 0, 0, 0, 0};
+  int na = 0, nbad = 0;
+  int hist = 0;        // lane z: records of charge state z
+  double histw = 0.0;  // and their weight
+  const long long stride = static_cast<long long>(gridDim.x) * THREADS;
+  for (long long k0 = static_cast<long long>(blockIdx.x) * THREADS + 32 * warp; k0 < a.c.n;
+       k0 += stride) {
+    const long long k = k0 + lane, i = a.c.off + k;
+    const unsigned char kd = k < a.c.n ? a.kind[i] : 2;
+    int zb = -1;
+    double wt = 0.0;
+    if (kd != 2) {
+      ++na;
+      double ke, pe, px, py, pz;
+      bool ok;
+      if (a.rec) {
+        // recorded by a diagnostic step at t_n (the state here is t_{n+1})
+        const double2* rc = reinterpret_cast<const double2*>(a.rec + 6 * i);
+        const double2 r0 = rc[0], r1 = rc[1], r2 = rc[2];
+        ok = r0.x == 1.0;
+        ke = r0.y;
+        pe = r1.x;
+        px = r1.y;
+        py = r2.x;
+        pz = r2.y;
+      } else {
+        const double X = a.x[i], Y = a.y[i], Z = a.z[i];
+        const double Ux = a.ux[i], Uy = a.uy[i], Uz = a.uz[i];
+        ok = isfinite(X) && isfinite(Y) && isfinite(Z) && isfinite(Ux) && isfinite(Uy) &&
+             isfinite(Uz);
+        float dux, duy, duz;
+        boris_increment(static_cast<float>(Ux), static_cast<float>(Uy), static_cast<float>(Uz),
+                        static_cast<float>(a.e[3 * k]) + s_las[0],
+                        static_cast<float>(a.e[3 * k + 1]) + s_las[1],
+                        static_cast<float>(a.e[3 * k + 2]) + s_las[2], s_las[3], s_las[4],
+                        s_las[5], hq * a.qm[i], dux, duy, duz);
+        const double mx = Ux + 0.5 * dux, my = Uy + 0.5 * duy, mz = Uz + 0.5 * duz;
+        const double uu = mx * mx + my * my + mz * mz;
+        const double wm = a.w[i] * a.mass[i];
+        ke = wm * uu / (sqrt(1.0 + uu) + 1.0);
+        pe = 0.5 * a.w[i] * a.zq[i] * a.phi[k];
+        px = wm * mx;
+        py = wm * my;
+        pz = wm * mz;
+      }
+      if (!ok) {
+        ++nbad;
+      } else {
+        acc[0] += ke;
+        acc[kd == 1 ? 2 : 1] += ke;
+        acc[3] += pe;
+        acc[4] += px;
+        acc[5] += py;
+        acc[6] += pz;
+        if (kd == 0) {
+          zb = a.zq[i];
+          zb = zb < 0 ? 0 : (zb >= kHistBins ? kHistBins - 1 : zb);
+          wt = a.w[i];
+        }
+      }
+    }
+    // the charge states among these 32 records, lowest lane first
+    for (unsigned todo = __ballot_sync(0xffffffffu, zb >= 0); todo;) {
+      const int z = __shfl_sync(0xffffffffu, zb, __ffs(todo) - 1);
+      const unsigned same = __ballot_sync(0xffffffffu, zb == z);
+      const double s = warp_sum(zb == z ? wt : 0.0);
+      if (lane == z) {
+        hist += __popc(same);
+        histw += s;
+      }
+      todo &= ~same;
+    }
+  }
 #pragma unroll
-  for (int k = 0; k < kHistBins; ++k) {
-    hist[k] = 0;
-    histw[k] = 0.0;
+  for (int v = 0; v < 7; ++v) {
+    const double s = warp_sum(acc[v]);
+    if (lane == 0) s_v[warp][v] = s;
   }
-  for (long long k = static_cast<long long>(blockIdx.x) * THREADS + threadIdx.x; k < a.c.n;
-       k += static_cast<long long>(gridDim.x) * THREADS) {
-    const long long i = a.c.off + k;
-    const unsigned char kd = a.kind[i];
-    if (kd == 2) continue;
-    ++na;
-    if (a.rec) {
-      // recorded by a diagnostic step at t_n (the state here is t_{n+1})
-      const double* rc = a.rec + 6 * i;
-      if (rc[0] != 1.0) {
-        ++nbad;
-        continue;
-      }
-      acc[0] += rc[1];
-      if (kd == 1) acc[2] += rc[1]; else acc[1] += rc[1];
-      acc[3] += rc[2];
-      acc[4] += rc[3];
-      acc[5] += rc[4];
-      acc[6] += rc[5];
-    } else {
-      const double X = a.x[i], Y = a.y[i], Z = a.z[i];
-      const double Ux = a.ux[i], Uy = a.uy[i], Uz = a.uz[i];
-      if (!(isfinite(X) && isfinite(Y) && isfinite(Z) && isfinite(Ux) && isfinite(Uy) &&
-            isfinite(Uz))) {
-        ++nbad;
-        continue;
-      }
-      float dux, duy, duz;
-      boris_increment(static_cast<float>(Ux), static_cast<float>(Uy), static_cast<float>(Uz),
-                      static_cast<float>(a.e[3 * k]) + las[0],
-                      static_cast<float>(a.e[3 * k + 1]) + las[1],
-                      static_cast<float>(a.e[3 * k + 2]) + las[2], las[3], las[4], las[5],
-                      hq * a.qm[i], dux, duy, duz);
-      const double mx = Ux + 0.5 * dux, my = Uy + 0.5 * duy, mz = Uz + 0.5 * duz;
-      const double uu = mx * mx + my * my + mz * mz;
-      const double wm = a.w[i] * a.mass[i];
-      const double ke = wm * uu / (sqrt(1.0 + uu) + 1.0);
-      acc[0] += ke;
-      if (kd == 1) acc[2] += ke; else acc[1] += ke;
-      acc[3] += 0.5 * a.w[i] * a.zq[i] * a.phi[k];
-      acc[4] += wm * mx;
-      acc[5] += wm * my;
-      acc[6] += wm * mz;
-    }
-    if (kd == 0) {
-      int zb = a.zq[i];
-      zb = zb < 0 ? 0 : (zb >= kHistBins ? kHistBins - 1 : zb);
-      hist[zb] += 1;
-      histw[zb] += a.w[i];
-    }
+  na = __reduce_add_sync(0xffffffffu, na);
+  nbad = __reduce_add_sync(0xffffffffu, nbad);
+  if (lane == 0) {
+    s_v[warp][7] = 0.0;
+    s_v[warp][8] = na;
+    s_v[warp][9] = nbad;
   }
+  if (lane < kHistBins) {
+    s_v[warp][10 + lane] = hist;
+    s_v[warp][10 + kHistBins + lane] = histw;
+  }
+  __syncthreads();
+  const int v = threadIdx.x;
+  if (v >= kDiagVals) return;
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) s += s_v[w][v];  // (counts below 2^53: exact)
   DiagPartial* out = a.part + blockIdx.x;
-  for (int k = 0; k < 8; ++k) {
-    const double s = block_sum<THREADS>(acc[k], red);
-    if (threadIdx.x == 0) out->v[k] = s;
-  }
-  {
-    double s = block_sum<THREADS>(static_cast<double>(na), red);
-    if (threadIdx.x == 0) out->cnt[0] = static_cast<long long>(s);
-    s = block_sum<THREADS>(static_cast<double>(nbad), red);
-    if (threadIdx.x == 0) out->cnt[1] = static_cast<long long>(s);
-  }
-  for (int k = 0; k < kHistBins; ++k) {
-    double s = block_sum<THREADS>(static_cast<double>(hist[k]), red);
-    if (threadIdx.x == 0) out->hist[k] = static_cast<long long>(s);
-    s = block_sum<THREADS>(histw[k], red);
-    if (threadIdx.x == 0) out->histw[k] = s;
-  }
+  if (v < 8)
+    out->v[v] = s;
+  else if (v < 10)
+    out->cnt[v - 8] = static_cast<long long>(s);
+  else if (v < 10 + kHistBins)
+    out->hist[v - 10] = static_cast<long long>(s);
+  else
+    out->histw[v - 10 - kHistBins] = s;
 }
 
 }  // namespace md

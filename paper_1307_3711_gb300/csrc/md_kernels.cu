@@ -6,28 +6,26 @@
 
 namespace md {
 
-// Sums the per-block partials in block order (deterministic); one thread per
-// component.
-__global__ void k_diag_final(const DiagPartial* __restrict__ part, int nblocks,
-                             DiagPartial* __restrict__ out) {
-  const int k = threadIdx.x;
-  if (k < 8) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[b].v[k];
-    out->v[k] = s;
-  } else if (k < 10) {
+// Sum of the per-CTA partials, one warp per value: lane l adds the CTAs l, l + 32,
+// ..., then the lanes are added (a fixed order).
+__global__ void __launch_bounds__(32) k_diag_final(const DiagPartial* __restrict__ part,
+                                                   int nblocks, DiagPartial* __restrict__ out) {
+  const int k = blockIdx.x, lane = threadIdx.x;
+  if (k >= 8 && k < 10 + kHistBins) {
     long long s = 0;
-    for (int b = 0; b < nblocks; ++b) s += part[b].cnt[k - 8];
-    out->cnt[k - 8] = s;
-  } else if (k < 10 + kHistBins) {
-    long long s = 0;
-    for (int b = 0; b < nblocks; ++b) s += part[b].hist[k - 10];
-    out->hist[k - 10] = s;
-  } else if (k < 10 + 2 * kHistBins) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[b].histw[k - 10 - kHistBins];
-    out->histw[k - 10 - kHistBins] = s;
+    for (int b = lane; b < nblocks; b += 32)
+      s += k < 10 ? part[b].cnt[k - 8] : part[b].hist[k - 10];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) (k < 10 ? out->cnt[k - 8] : out->hist[k - 10]) = s;
+    return;
   }
+  double s = 0.0;
+#pragma unroll 4
+  for (int b = lane; b < nblocks; b += 32)
+    s += k < 8 ? part[b].v[k] : part[b].histw[k - 10 - kHistBins];
+  s = warp_sum(s);
+  if (lane == 0) (k < 8 ? out->v[k] : out->histw[k - 10 - kHistBins]) = s;
 }
 
 // ------------------------------------------------------------ layout glue --
@@ -349,7 +347,7 @@ cudaError_t launch_diag(const DiagArgs& a, int blocks, DiagPartial* out, cudaStr
   k_diag_partial<kDiagThreads><<<blocks, kDiagThreads, 0, s>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_diag_final<<<1, 64, 0, s>>>(a.part, blocks, out);
+  k_diag_final<<<kDiagVals, 32, 0, s>>>(a.part, blocks, out);
   return cudaGetLastError();
 }
 

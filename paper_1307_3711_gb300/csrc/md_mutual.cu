@@ -268,6 +268,13 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
     fence_mbar_init();
     s_abort = 0;
   }
+  // the clusters' laser fields for the push, one CTA each
+  if (tid == 32) {
+    for (int c = blockIdx.x; c < a.n_clusters; c += gridDim.x) {
+      const ClusterDev& cl = a.s.cl[c];
+      laser_field(cl, cl.t0 + static_cast<double>(step) * cl.dt, a.las + 6 * c);
+    }
+  }
   __syncthreads();
   const float4* __restrict__ cur = (step & 1) ? a.s.posq1 : a.s.posq0;
   unsigned it = 0;  // tiles consumed (the barrier's phase)
@@ -454,15 +461,15 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
 
 // The push of every record: its partials in a fixed order, laser, kick, drift.
 // Runs after k_mut_pairs, whose ticket it resets; its last CTA advances the
-// step.  A CTA takes 32 records: warp w adds the work units and the earlier
-// blocks' rows w, w + 8, ... in Kahan-compensated FP32, and the first warp adds
-// the eight sums in FP64 and pushes.  136 us at 200k records and 14 at 19k
-// (0.3 GB of partials at 200k); one thread per record with FP64 adds, which the
-// narrow FP64 pipe bounds, took 240 and 32.
+// step.  A CTA takes 32 records: warp w of W adds the work units and the earlier
+// blocks' rows w, w + W, ... in Kahan-compensated FP32, and the first warp adds
+// the W sums in FP64 and pushes with the laser field that the pair kernel left.
+// 99 us at 200k records (0.3 GB of partials) with W = 4, 12.5 at 19k with 8; one
+// thread per record with FP64 adds, which the narrow FP64 pipe bounds, took 240
+// and 32, the laser's sine in every CTA 136 and 14.
 constexpr int kPushRec = 32;
-constexpr int kPushWarps = 8;
 
-template <bool DET, bool POT>
+template <int kPushWarps, bool DET, bool POT>
 __global__ void __launch_bounds__(32 * kPushWarps) k_mut_push(const MutArgs a) {
   constexpr int C = POT ? 4 : 3;
   __shared__ double s_e[C][kPushWarps][kPushRec];
@@ -480,13 +487,10 @@ __global__ void __launch_bounds__(32 * kPushWarps) k_mut_push(const MutArgs a) {
   const long long j = static_cast<long long>(b.block) * a.block + k;   // in the cluster
   const bool live = j < n_pad;
   RecState st;
-  if (warp == kPushWarps - 1) {
-    if (lane == 0) {
-      s_c = *cl;
-      laser_field(s_c, s_c.t0 + static_cast<double>(step) * s_c.dt, s_las);
-    }
-    __syncwarp();
-  }
+  static_assert(sizeof(ClusterDev) % 4 == 0, "copied by words");
+  for (int q = threadIdx.x; q < static_cast<int>(sizeof(ClusterDev) / 4); q += 32 * kPushWarps)
+    reinterpret_cast<int*>(&s_c)[q] = reinterpret_cast<const int*>(cl)[q];
+  if (threadIdx.x < 6) s_las[threadIdx.x] = a.las[6 * b.cluster + threadIdx.x];
   if (live) {
     if (warp == 0) st = load_state(a.s, cl->off + j);
     float s[3] = {0.f, 0.f, 0.f}, c[3] = {0.f, 0.f, 0.f};
@@ -577,6 +581,16 @@ void launch_pairs_r(const MutArgs& a, int grid, bool pot, bool mi, cudaStream_t 
     k_mut_pairs<R, kTile, false, false><<<grid, kMutThreads, 0, s>>>(a);
 }
 
+template <int W>
+void launch_push_w(const MutArgs& a, unsigned g, bool det, bool pot, cudaStream_t s) {
+  if (det)
+    k_mut_push<W, true, false><<<g, 32 * W, 0, s>>>(a);
+  else if (pot)
+    k_mut_push<W, false, true><<<g, 32 * W, 0, s>>>(a);
+  else
+    k_mut_push<W, false, false><<<g, 32 * W, 0, s>>>(a);
+}
+
 }  // namespace
 
 cudaError_t mut_blocks_per_sm(int block, bool pot, bool mi, int* out) {
@@ -595,12 +609,12 @@ cudaError_t launch_mut_step(const MutArgs& a, int grid, bool det, bool pot, bool
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const unsigned g = static_cast<unsigned>(a.n_blks) * static_cast<unsigned>(a.block / kPushRec);
-  if (det)
-    k_mut_push<true, false><<<g, 32 * kPushWarps, 0, s>>>(a);
-  else if (pot)
-    k_mut_push<false, true><<<g, 32 * kPushWarps, 0, s>>>(a);
+  // eight warps while the CTAs are few (19k records: 12.5 us against 18 with
+  // four), four once they fill the SMs (a scan of 290k records: 81 against 125)
+  if (g >= 8u * static_cast<unsigned>(a.sms))
+    launch_push_w<4>(a, g, det, pot, s);
   else
-    k_mut_push<false, false><<<g, 32 * kPushWarps, 0, s>>>(a);
+    launch_push_w<8>(a, g, det, pot, s);
   return cudaGetLastError();
 }
 

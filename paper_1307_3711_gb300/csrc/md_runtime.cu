@@ -144,6 +144,7 @@ struct md_ctx {
   float2* d_mut_ipart = nullptr;
   float* d_mut_jpart = nullptr;
   double* d_mut_jphi = nullptr;   // allocated by the first diagnostic step
+  float* d_mut_las = nullptr;
   long long mut_jrecs = 0;        // records of all rows of jpart
   // the step of a few thousand records (md_small.cu), while small_targets > 0
   int small_targets = 0;
@@ -433,6 +434,9 @@ md::MutArgs mut_args(md_ctx* c) {
   a.ipart = c->d_mut_ipart;
   a.jpart = c->d_mut_jpart;
   a.jphi = c->d_mut_jphi;
+  a.las = c->d_mut_las;
+  a.n_clusters = c->n_clusters;
+  a.sms = c->sm_count;
   return a;
 }
 
@@ -741,6 +745,8 @@ void auto_off(md_ctx* c) {
   cudaFree(c->d_mut_ipart);
   cudaFree(c->d_mut_jpart);
   cudaFree(c->d_mut_jphi);
+  cudaFree(c->d_mut_las);
+  c->d_mut_las = nullptr;
   c->d_mut_units = nullptr;
   c->d_mut_first = nullptr;
   c->d_mut_blks = nullptr;
@@ -888,6 +894,7 @@ md_status auto_configure(md_ctx* c) {
   if (e == cudaSuccess) e = dev_alloc(&c->d_mut_units, units.size());
   if (e == cudaSuccess) e = dev_alloc(&c->d_mut_first, first.size());
   if (e == cudaSuccess) e = dev_alloc(&c->d_mut_blks, blks.size());
+  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_las, 6 * static_cast<size_t>(c->n_clusters));
   if (e != cudaSuccess) {  // no room: the step kernel needs none of this
     cudaGetLastError();
     auto_off(c);

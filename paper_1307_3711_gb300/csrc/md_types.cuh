@@ -188,6 +188,9 @@ struct MutArgs {
   float2* ipart;  // [unit][3, or 4 with the potential][block]: Kahan sum, compensation
   float* jpart;   // per block: [3][records after the block]
   double* jphi;   // per block: [records after the block] (diagnostic steps)
+  float* las;     // [n_clusters][6] laser field at t_n, from the pair kernel to the push
+  int n_clusters;
+  int sms;
 };
 
 // One CTA of the small step (md_small.cu): its cluster and first target.
