@@ -8,11 +8,19 @@
 // staged tile), the slices' sums are added in FP64 in shared memory and the
 // CTAs' through distributed shared memory by the cluster's first CTA.
 //
+// A tile is released warp by warp instead of by a CTA-wide barrier and a full
+// tile's loop has a fixed length (3 to 4 % of a large field), and the warps' sums
+// are joined as compensated FP32 pairs, for an FP64 instruction takes its pipe 16
+// cycles (every slice in FP64: 2 us more per call).  Up to four targets per SM the sources' tiles
+// are what a CTA waits for: tiles of 4096, two stages, one CTA per SM and small
+// clusters, which the SMs hold evenly (300 x 150k: 49 us with tiles of 1024 and
+// clusters of eight, 29 so).
+//
 // Measured (us, field without the potential; in brackets the field kernel with
 // its partials in memory, and the allocation-free kernel of 256-target blocks
-// that this one replaced): 300 targets x 150k sources 49 (185, 657), 1000 x
-// 4001 10.3 (237, 146), 1 x 150k 19 (171, 655), 1000 x 1M 586 (948, 4320), 3000
-// x 1M 1650 (1756, 4325), 10000 x 150k 757 (675, 1012).  One target per thread
+// that this one replaced): 300 targets x 150k sources 29 (185, 657), 1000 x
+// 4001 10.5 (237, 146), 1 x 150k 10.4 (171, 655), 1000 x 1M 559 (948, 4320), 3000
+// x 1M 1610 (1756, 4325), 10000 x 150k 711 (675, 1012).  One target per thread
 // reads a source from shared memory per pair, so where the field kernel's
 // blocks fill the SMs it stays faster (field_uses_probe).
 #include <algorithm>
@@ -31,25 +39,37 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kThreads = 512;
-constexpr int kTile = 1024;  // sources per stage
-constexpr int kStages = 3;
+constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCluster = 8;
+constexpr int kLargeTile = 4096;  // (two stages of it leave room for one CTA per SM)
 
-template <int TL, int R, bool POT>
+// Sum of two compensated sums (value s - c), with the rounding of s kept in c.
+__device__ __forceinline__ void join(float& s, float& c, float s2, float c2) {
+  const float t = s + s2, b = t - s;
+  c = (c + c2) - ((s - (t - b)) + (s2 - b));
+  s = t;
+}
+
+template <int TL, int R, bool POT, int kTile, int kStages>
 struct ProbeSmem {
   Stage<kTile, kStages> st;
-  double e[POT ? 4 : 3][kThreads / TL][TL * R];       // the slices' sums
+  float2 e[POT ? 4 : 3][kWarps][TL * R];              // the warps' sums (value x - y)
   double part[kMaxCluster][POT ? 4 : 3][TL * R];      // first CTA: the CTAs' sums
+  uint64_t empty[kStages];
   int abort;
 };
 
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // CTA (x, rank) of cluster x: targets [x kTargets, ...), sources [rank seg, ...).
-template <int TL, int R, bool POT>
+template <int TL, int R, bool POT, int kTile, int kStages>
 __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long seg) {
   constexpr int kTargets = TL * R;
   constexpr int kSlices = kThreads / TL;
   constexpr int C = POT ? 4 : 3;
-  __shared__ ProbeSmem<TL, R, POT> S;
+  __shared__ ProbeSmem<TL, R, POT, kTile, kStages> S;
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank());
   const int ranks = static_cast<int>(cluster.num_blocks());
@@ -62,13 +82,16 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
   const float4* __restrict__ src = a.src + j0;
   const int ntiles = static_cast<int>((ns + kTile - 1) / kTile);
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&S.st.full[s], 1);
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&S.st.full[s], 1);
+      mbar_init(&S.empty[s], kWarps);
+    }
     fence_mbar_init();
     S.abort = 0;
     for (int t = 0; t < kStages && t < ntiles; ++t)
       issue_tile<kTile, kStages>(S.st, static_cast<unsigned>(t), src, ns, t);
   }
-  const int tl = tid % TL, slice = tid / TL;
+  const int tl = tid % TL, slice = tid / TL, lane = tid & 31;
   const long long i0 = group * kTargets;
   float xi[R], yi[R], zi[R];
 #pragma unroll
@@ -82,20 +105,40 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
   __syncthreads();
   Acc<R, POT> acc;
   acc.zero();
+  // (a thread meets kTile / kSlices sources of a tile: several tiles to a fold)
+  constexpr int kFold = 64 * kSlices > kTile ? 64 * kSlices / kTile : 1;
+  auto stop = [&] {
+    atomicOr(a.err, kErrTimeout);
+    *reinterpret_cast<volatile int*>(&S.abort) = 1;
+  };
+  int issued = kStages < ntiles ? kStages : ntiles;  // (thread 0)
   for (int t = 0; t < ntiles; ++t) {
     const int s = t % kStages;
-    if (!mbar_wait(&S.st.full[s], (t / kStages) & 1u)) {
-      atomicOr(a.err, kErrTimeout);
-      S.abort = 1;
+    // the first thread refills the stage of the tile before this one once every
+    // warp has read it: the warps run up to a tile apart
+    if (tid == 0 && t > 0 && issued < ntiles) {
+      if (mbar_wait(&S.empty[(t - 1) % kStages], ((t - 1) / kStages) & 1u)) {
+        issue_tile<kTile, kStages>(S.st, static_cast<unsigned>(issued), src, ns, issued);
+        ++issued;
+      } else {
+        stop();
+      }
+    }
+    // (the lanes of a warp decide alike)
+    if (!__all_sync(0xffffffffu, mbar_try_wait(&S.st.full[s], (t / kStages) & 1u))) {
+      const bool go = *reinterpret_cast<volatile int*>(&S.abort) == 0 &&
+                      mbar_wait(&S.st.full[s], (t / kStages) & 1u);
+      if (!__all_sync(0xffffffffu, go)) {
+        stop();
+        break;
+      }
     }
     const long long rem = ns - static_cast<long long>(t) * kTile;
-    const int cnt = static_cast<int>(rem < kTile ? rem : kTile);
-    const uint32_t tile = smem_u32(&S.st.tile[s][0]);
-    int k = slice;
-    for (; k + 7 * kSlices < cnt; k += 8 * kSlices) {
+    const uint32_t tile = smem_u32(&S.st.tile[s][0]) + 16u * slice;
+    auto eight = [&](uint32_t from) {
 #pragma unroll
       for (int q = 0; q < 8; ++q)
-        pair<R, POT>(lds_f4(tile + 16u * (k + q * kSlices)), xi, yi, zi, a.eps2, acc);
+        pair<R, POT>(lds_f4(from + 16u * (q * kSlices)), xi, yi, zi, a.eps2, acc);
       if constexpr (POT) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -103,42 +146,61 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
           acc.ap[r] = 0.0f;
         }
       }
+    };
+    if (rem >= kTile) {
+      constexpr int kEach = kTile / kSlices;  // a full tile's sources per thread
+      static_assert(kEach % 8 == 0, "eights");
+#pragma unroll(kEach <= 32 ? kEach / 8 : 2)
+      for (int k = 0; k < kEach; k += 8) eight(tile + 16u * (k * kSlices));
+    } else {
+      const int cnt = static_cast<int>(rem);
+      int k = slice;
+      for (; k + 7 * kSlices < cnt; k += 8 * kSlices) eight(tile + 16u * (k - slice));
+      for (; k < cnt; k += kSlices)
+        pair<R, POT>(lds_f4(tile + 16u * (k - slice)), xi, yi, zi, a.eps2, acc);
     }
-    for (; k < cnt; k += kSlices)
-      pair<R, POT>(lds_f4(tile + 16u * k), xi, yi, zi, a.eps2, acc);
-    fold<R, POT>(acc);
-    if (t + kStages < ntiles) {
-      __syncthreads();  // the stage has been read by every warp
-      if (tid == 0 && !S.abort)
-        issue_tile<kTile, kStages>(S.st, static_cast<unsigned>(t + kStages), src, ns, t + kStages);
-      if (S.abort) {  // an expired wait: no further copies, those in flight are awaited
-        if (tid == 0)
-          for (int q = t + 1; q < t + kStages && q < ntiles; ++q)
-            mbar_wait(&S.st.full[q % kStages], (q / kStages) & 1u);
-        break;
-      }
-    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&S.empty[s]);
+    if ((t + 1) % kFold == 0) fold<R, POT>(acc);
   }
+  fold<R, POT>(acc);
+  // (an expired wait: no further copies, those in flight are awaited)
+  if (tid == 0 && S.abort)
+    for (int q = issued > kStages ? issued - kStages : 0; q < issued; ++q)
+      mbar_wait(&S.st.full[q % kStages], (q / kStages) & 1u);
+  auto put = [&](int c, int r, float v, float w) {
+#pragma unroll
+    for (int d = TL; d < 32; d <<= 1)
+      join(v, w, __shfl_xor_sync(0xffffffffu, v, d), __shfl_xor_sync(0xffffffffu, w, d));
+    if (lane < TL) S.e[c][tid >> 5][tl + r * TL] = make_float2(v, w);
+  };
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    S.e[0][slice][tl + r * TL] = -(static_cast<double>(acc.sx[r]) - acc.cx[r]);
-    S.e[1][slice][tl + r * TL] = -(static_cast<double>(acc.sy[r]) - acc.cy[r]);
-    S.e[2][slice][tl + r * TL] = -(static_cast<double>(acc.sz[r]) - acc.cz[r]);
-    if constexpr (POT) S.e[3][slice][tl + r * TL] = static_cast<double>(acc.sp[r]) - acc.cp[r];
+    put(0, r, acc.sx[r], acc.cx[r]);
+    put(1, r, acc.sy[r], acc.cy[r]);
+    put(2, r, acc.sz[r], acc.cz[r]);
+    if constexpr (POT) put(3, r, acc.sp[r], acc.cp[r]);
   }
   __syncthreads();
   cluster.barrier_wait(std::move(started));
-  // each value's slices: eight neighbouring lanes add every eighth, then each other's
+  // each value's warps: eight neighbouring lanes add two each, then each other's
   constexpr int kVals = C * kTargets;
   double* to = &cluster.map_shared_rank(&S.part[0][0][0], 0)[rank * kVals];
   for (int v0 = 0; v0 < kVals; v0 += kThreads / 8) {
     const int v = v0 + tid / 8, c = v / kTargets, t = v % kTargets;
-    double s = 0.0;
-    if (v < kVals)
-      for (int q = tid % 8; q < kSlices; q += 8) s += S.e[c][q][t];
+    float2 s = make_float2(0.0f, 0.0f);
+    if (v < kVals) {
+      s = S.e[c][tid % 8][t];
+      const float2 o = S.e[c][tid % 8 + 8][t];
+      join(s.x, s.y, o.x, o.y);
+    }
 #pragma unroll
-    for (int d = 4; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-    if (v < kVals && tid % 8 == 0) to[v] = s;
+    for (int d = 4; d > 0; d >>= 1)
+      join(s.x, s.y, __shfl_xor_sync(0xffffffffu, s.x, d), __shfl_xor_sync(0xffffffffu, s.y, d));
+    if (v < kVals && tid % 8 == 0) {
+      const double val = static_cast<double>(s.x) - s.y;
+      to[v] = c < 3 ? -val : val;
+    }
   }
   cluster.sync();
   if (rank != 0 || tid >= kTargets) return;
@@ -162,7 +224,7 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
   }
 }
 
-template <int TL, int R, bool POT>
+template <int TL, int R, bool POT, int TILE, int STAGES>
 cudaError_t launch_t(const FieldArgs& a, int cluster, cudaStream_t s) {
   const long long groups = (a.nt + TL * R - 1) / (TL * R);
   cudaLaunchConfig_t cfg = {};
@@ -177,12 +239,13 @@ cudaError_t launch_t(const FieldArgs& a, int cluster, cudaStream_t s) {
   cfg.numAttrs = 1;
   // whole cache lines of sources per CTA
   const long long seg = ((a.ns + cluster - 1) / cluster + 7) / 8 * 8;
-  return cudaLaunchKernelEx(&cfg, k_probe<TL, R, POT>, a, seg);
+  return cudaLaunchKernelEx(&cfg, k_probe<TL, R, POT, TILE, STAGES>, a, seg);
 }
 
-template <int TL, int R>
+template <int TL, int R, int TILE = 1024, int STAGES = 3>
 cudaError_t launch_p(const FieldArgs& a, bool potential, int cluster, cudaStream_t s) {
-  return potential ? launch_t<TL, R, true>(a, cluster, s) : launch_t<TL, R, false>(a, cluster, s);
+  return potential ? launch_t<TL, R, true, TILE, STAGES>(a, cluster, s)
+                   : launch_t<TL, R, false, TILE, STAGES>(a, cluster, s);
 }
 
 // Field of few sources at many targets, two per thread.
@@ -229,12 +292,11 @@ __global__ void __launch_bounds__(128) k_few(const FieldArgs a) {
   }
 }
 
-// With few sources for many targets a cluster per few targets costs more than
-// it sums: 30000 targets x 100 sources 13 us with k_few, 27 with clusters; 10000
-// x 100 12.7 and 14.5, 3000 x 100 11.7 and 13.3 (k_few takes 35 ns per source).
-bool few_sources(long long nt, long long ns) {
-  return ns < 512 && nt > (ns < 160 ? 1024 : 8192);
-}
+// With few sources for many targets a cluster per few targets costs more than it
+// sums: k_few takes 4.5 us + 35 ns per source (the mean of with and without the
+// potential), k_probe 6.2 us + a third of a ns per target.  30000 targets x 100
+// sources 8.4 and 17 us, 10000 x 100 8.4 and 10.4, 3000 x 100 8.4 and 6.6.
+bool few_sources(long long nt, long long ns) { return ns < 512 && 105 * ns < 5100 + nt; }
 
 }  // namespace
 
@@ -248,6 +310,19 @@ cudaError_t launch_field_direct(const FieldArgs& a, bool potential, int sms, cud
       k_few<false><<<g, 128, 0, s>>>(a);
     return cudaGetLastError();
   }
+  // up to four targets per SM and many sources: one CTA per SM with large tiles,
+  // the fewest targets per CTA that its cluster size lets run at once (clusters of
+  // two fill every SM, of four all but four SMs, of eight nine in ten)
+  if (a.ns >= 12000) {
+    const long long c8 = sms / 9, c4 = sms / 4 - 1, c2 = sms / 2;
+    if (a.nt <= 2 * c8) return launch_p<2, 1, kLargeTile, 2>(a, potential, 8, s);
+    if (a.nt <= 2 * c4) return launch_p<2, 1, kLargeTile, 2>(a, potential, 4, s);
+    if (a.nt <= 4 * c4) return launch_p<4, 1, kLargeTile, 2>(a, potential, 4, s);
+    if (a.nt <= 4 * c2) return launch_p<4, 1, kLargeTile, 2>(a, potential, 2, s);
+    // (400 x 150k: 53 us, 47 with the smaller tiles below; 400 x 30k: 14.7 and 16.7)
+    if (a.nt > (a.ns < 60000 ? 4 : 6) * c2 && a.nt <= 8 * c2)
+      return launch_p<8, 1, kLargeTile, 2>(a, potential, 2, s);
+  }
   // as many CTAs per cluster as leave each a stage of sources; then the most
   // targets per CTA that still give five CTAs to three SMs (fewer targets: the
   // sources are staged more often; fewer CTAs: idle SMs)
@@ -256,8 +331,8 @@ cudaError_t launch_field_direct(const FieldArgs& a, bool potential, int sms, cud
   const long long want = 5LL * sms / 3;
   auto ctas = [&](long long tl) { return (a.nt + tl - 1) / tl * cluster; };
   // two targets per thread halve the loads per pair once there is work for it
-  // (30000 x 30000: 489 us with one, 440 with two; 3000 x 150k: 262 and 277),
-  // and enough targets need fewer CTAs per cluster (four: 440, eight: 469)
+  // (30000 x 30000: 440 us with one, 421 with two; 10000 x 150k: 750 and 711),
+  // and enough targets need fewer CTAs per cluster (30000 x 30000: 421, eight: 450)
   if (a.nt >= 8192 && a.ns >= 8192)
     return launch_p<32, 2>(a, potential, a.nt >= 16384 ? std::min(cluster, 4) : cluster, s);
   // (many targets and few sources: no more CTAs than that; 30000 x 4001: 105 us

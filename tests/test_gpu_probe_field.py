@@ -73,3 +73,19 @@ def test_small_contexts_field_follows_oracle(md, n):
     if n > 1:
         assert summary(force_error(e, e64))["p99"] <= FORCE_P99
     np.testing.assert_allclose(phi, p64, rtol=1e-4, atol=2e-5 * max(np.abs(p64).max(), 1e-7))
+
+
+@pytest.mark.parametrize("nt,ns", [(1, 12000), (32, 66001), (33, 12001), (74, 150007), (75, 40000),
+                                   (148, 99999), (149, 12000), (304, 70001), (305, 13000),
+                                   (457, 61000), (608, 35000), (609, 35000)])
+def test_large_tiles_follow_oracle(md, nt, ns):
+    """Few targets of many sources: the target counts at which the split changes,
+    source counts of one to several stages per CTA with ragged ends."""
+    test_field_and_potential_follow_oracle(md, nt, ns, False)
+
+
+@pytest.mark.parametrize("nt,ns", [(1500, 62), (1500, 63), (32768, 360), (32768, 361), (256, 1),
+                                   (30000, 300)])
+def test_few_sources_follow_oracle(md, nt, ns):
+    """Either side of the line between the kernel for few sources and the clusters."""
+    test_field_and_potential_follow_oracle(md, nt, ns, False)
