@@ -354,8 +354,14 @@ struct TrainSmem {
 };
 
 // One minibatch [b0, b0 + nb) of the sample set: forward, backward, per-CTA
-// FP32 gradient partials (fixed accumulation order) and loss partials.
-__global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restrict__ p,
+// FP32 gradient partials (fixed accumulation order) and loss partials.  The
+// first kWarps warps run the samples through the network; all the CTA's threads
+// own gradient entries.  Bound by the serial chain of one tile: while a batch has
+// no more tiles than there are SMs the one CTA of an SM has eight warps, half the
+// entries each (loss and gradient of 8192 samples, with the host's part, 37.9 us
+// with four, 36.9 with eight, of 1000 37.7 and 35.6; the same sums in the same order).
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) k_mlp_train(const float* __restrict__ p,
                                                            const float* __restrict__ feats,
                                                            const int* __restrict__ zs,
                                                            const float* __restrict__ target,
@@ -364,108 +370,113 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
                                                            float* __restrict__ loss_part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
-  load_weights<32 * kWarps>(p, S.w);
+  load_weights<THREADS>(p, S.w);
   __syncthreads();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const float coef = 2.0f / static_cast<float>(nb);
   // owned gradient entries
-  float gw2[32], gw3[4], gw1[2], gb = 0.0f, gb3 = 0.0f;
+  constexpr int kRowsOf = THREADS / kNH;        // threads that share a column
+  constexpr int kR2 = kNH / kRowsOf, kR3 = kNO / kRowsOf, kR1 = kNH * kNI / THREADS;
+  float gw2[kR2], gw3[kR3], gw1[kR1], gb = 0.0f, gb3 = 0.0f;
 #pragma unroll
-  for (int m = 0; m < 32; ++m) gw2[m] = 0.0f;
+  for (int m = 0; m < kR2; ++m) gw2[m] = 0.0f;
 #pragma unroll
-  for (int m = 0; m < 4; ++m) gw3[m] = 0.0f;
-  gw1[0] = gw1[1] = 0.0f;
+  for (int m = 0; m < kR3; ++m) gw3[m] = 0.0f;
+#pragma unroll
+  for (int m = 0; m < kR1; ++m) gw1[m] = 0.0f;
   float lsum = 0.0f;
   const int kcol = tid & 63, nrow = tid >> 6;
   const long long iters = (nb + kTileSamples - 1) / kTileSamples;
   for (long long it = blockIdx.x; it < iters; it += gridDim.x) {
-    WarpStage& st = S.st[warp];
-    const long long base = b0 + it * kTileSamples + warp * 16;
-    const long long lim = b0 + nb;
-    const long long sg = base + g, sg8 = base + g + 8;
-    float xg[4], xg8[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      xg[k] = sg < lim ? feats[4 * sg + k] : 0.0f;
-      xg8[k] = sg8 < lim ? feats[4 * sg8 + k] : 0.0f;
-    }
-    Fwd f;
-    forward(S.w, xg, xg8, f);
-    // dL/dy: only the output of the sample's charge state
-    const int zg = sg < lim ? zs[sg] : -1, zg8 = sg8 < lim ? zs[sg8] : -1;
-    const float tg = sg < lim ? target[sg] : 0.0f, tg8 = sg8 < lim ? target[sg8] : 0.0f;
-    float dy[4];
-    dy[0] = (zg == 2 * t) ? coef * (f.y[0] - tg) : 0.0f;
-    dy[1] = (zg == 2 * t + 1) ? coef * (f.y[1] - tg) : 0.0f;
-    dy[2] = (zg8 == 2 * t) ? coef * (f.y[2] - tg8) : 0.0f;
-    dy[3] = (zg8 == 2 * t + 1) ? coef * (f.y[3] - tg8) : 0.0f;
-    if (zg == 2 * t) lsum += (f.y[0] - tg) * (f.y[0] - tg);
-    if (zg == 2 * t + 1) lsum += (f.y[1] - tg) * (f.y[1] - tg);
-    if (zg8 == 2 * t) lsum += (f.y[2] - tg8) * (f.y[2] - tg8);
-    if (zg8 == 2 * t + 1) lsum += (f.y[3] - tg8) * (f.y[3] - tg8);
-    // dh2 = dy W3 in FP32: every lane of the quad has both rows' outputs, so
-    // each forms the gradient of its own 16 columns from the selected row of W3
-    const float dsel0 = (zg >= 0 && zg < kNO) ? coef * (pick8(f.yall[0], zg) - tg) : 0.0f;
-    const float dsel1 = (zg8 >= 0 && zg8 < kNO) ? coef * (pick8(f.yall[1], zg8) - tg8) : 0.0f;
-    const int zr0 = (zg >= 0 && zg < kNO) ? zg : 0, zr1 = (zg8 >= 0 && zg8 < kNO) ? zg8 : 0;
-    float dh[8][4];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int c0 = 8 * j + 2 * t;
-      dh[j][0] = dsel0 * S.w.w3[zr0][c0];
-      dh[j][1] = dsel0 * S.w.w3[zr0][c0 + 1];
-      dh[j][2] = dsel1 * S.w.w3[zr1][c0];
-      dh[j][3] = dsel1 * S.w.w3[zr1][c0 + 1];
-    }
-    // da2 = dh2 * silu'(a2); stage h2 (FP32, as the output layer uses it), h1
-    // (BF16, as layer 2 uses it), dy, da2
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) dh[j][q] *= dsilu(f.a2[j][q]);
-      const int c0 = 8 * j + 2 * t;
-      auto put = [&](float (&to)[16][kStRow], float v0, float v1, float v2, float v3) {
-        *reinterpret_cast<float2*>(&to[g][c0]) = make_float2(v0, v1);
-        *reinterpret_cast<float2*>(&to[g + 8][c0]) = make_float2(v2, v3);
-      };
-      put(st.da2, dh[j][0], dh[j][1], dh[j][2], dh[j][3]);
-      put(st.h2, silu(f.a2[j][0]), silu(f.a2[j][1]), silu(f.a2[j][2]), silu(f.a2[j][3]));
-      put(st.h1, bf16_round(silu(f.a1[j][0])), bf16_round(silu(f.a1[j][1])),
-          bf16_round(silu(f.a1[j][2])), bf16_round(silu(f.a1[j][3])));
-    }
-    st.dy[g][2 * t] = dy[0]; st.dy[g][2 * t + 1] = dy[1];
-    st.dy[g + 8][2 * t] = dy[2]; st.dy[g + 8][2 * t + 1] = dy[3];
-    // dh1 = da2 W2 (A = da2 as BF16 fragments)
-    uint32_t da[4][4];
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      da[kk][0] = pack_bf16(dh[2 * kk][0], dh[2 * kk][1]);
-      da[kk][1] = pack_bf16(dh[2 * kk][2], dh[2 * kk][3]);
-      da[kk][2] = pack_bf16(dh[2 * kk + 1][0], dh[2 * kk + 1][1]);
-      da[kk][3] = pack_bf16(dh[2 * kk + 1][2], dh[2 * kk + 1][3]);
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      float d1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t bb0 = pair_of(S.w.w2[16 * kk + 2 * t][8 * j + g],
-                                     S.w.w2[16 * kk + 2 * t + 1][8 * j + g]);
-        const uint32_t bb1 = pair_of(S.w.w2[16 * kk + 8 + 2 * t][8 * j + g],
-                                     S.w.w2[16 * kk + 9 + 2 * t][8 * j + g]);
-        mma_bf16(d1, da[kk][0], da[kk][1], da[kk][2], da[kk][3], bb0, bb1);
-      }
-      const int c0 = 8 * j + 2 * t;
-      *reinterpret_cast<float2*>(&st.da1[g][c0]) =
-          make_float2(d1[0] * dsilu(f.a1[j][0]), d1[1] * dsilu(f.a1[j][1]));
-      *reinterpret_cast<float2*>(&st.da1[g + 8][c0]) =
-          make_float2(d1[2] * dsilu(f.a1[j][2]), d1[3] * dsilu(f.a1[j][3]));
-    }
-    if (t == 0) {
+    if (warp < kWarps) {
+      WarpStage& st = S.st[warp];
+      const long long base = b0 + it * kTileSamples + warp * 16;
+      const long long lim = b0 + nb;
+      const long long sg = base + g, sg8 = base + g + 8;
+      float xg[4], xg8[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        st.x[g][k] = bf16_round(xg[k]);
-        st.x[g + 8][k] = bf16_round(xg8[k]);
+        xg[k] = sg < lim ? feats[4 * sg + k] : 0.0f;
+        xg8[k] = sg8 < lim ? feats[4 * sg8 + k] : 0.0f;
+      }
+      Fwd f;
+      forward(S.w, xg, xg8, f);
+      // dL/dy: only the output of the sample's charge state
+      const int zg = sg < lim ? zs[sg] : -1, zg8 = sg8 < lim ? zs[sg8] : -1;
+      const float tg = sg < lim ? target[sg] : 0.0f, tg8 = sg8 < lim ? target[sg8] : 0.0f;
+      float dy[4];
+      dy[0] = (zg == 2 * t) ? coef * (f.y[0] - tg) : 0.0f;
+      dy[1] = (zg == 2 * t + 1) ? coef * (f.y[1] - tg) : 0.0f;
+      dy[2] = (zg8 == 2 * t) ? coef * (f.y[2] - tg8) : 0.0f;
+      dy[3] = (zg8 == 2 * t + 1) ? coef * (f.y[3] - tg8) : 0.0f;
+      if (zg == 2 * t) lsum += (f.y[0] - tg) * (f.y[0] - tg);
+      if (zg == 2 * t + 1) lsum += (f.y[1] - tg) * (f.y[1] - tg);
+      if (zg8 == 2 * t) lsum += (f.y[2] - tg8) * (f.y[2] - tg8);
+      if (zg8 == 2 * t + 1) lsum += (f.y[3] - tg8) * (f.y[3] - tg8);
+      // dh2 = dy W3 in FP32: every lane of the quad has both rows' outputs, so
+      // each forms the gradient of its own 16 columns from the selected row of W3
+      const float dsel0 = (zg >= 0 && zg < kNO) ? coef * (pick8(f.yall[0], zg) - tg) : 0.0f;
+      const float dsel1 = (zg8 >= 0 && zg8 < kNO) ? coef * (pick8(f.yall[1], zg8) - tg8) : 0.0f;
+      const int zr0 = (zg >= 0 && zg < kNO) ? zg : 0, zr1 = (zg8 >= 0 && zg8 < kNO) ? zg8 : 0;
+      float dh[8][4];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int c0 = 8 * j + 2 * t;
+        dh[j][0] = dsel0 * S.w.w3[zr0][c0];
+        dh[j][1] = dsel0 * S.w.w3[zr0][c0 + 1];
+        dh[j][2] = dsel1 * S.w.w3[zr1][c0];
+        dh[j][3] = dsel1 * S.w.w3[zr1][c0 + 1];
+      }
+      // da2 = dh2 * silu'(a2); stage h2 (FP32, as the output layer uses it), h1
+      // (BF16, as layer 2 uses it), dy, da2
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dh[j][q] *= dsilu(f.a2[j][q]);
+        const int c0 = 8 * j + 2 * t;
+        auto put = [&](float (&to)[16][kStRow], float v0, float v1, float v2, float v3) {
+          *reinterpret_cast<float2*>(&to[g][c0]) = make_float2(v0, v1);
+          *reinterpret_cast<float2*>(&to[g + 8][c0]) = make_float2(v2, v3);
+        };
+        put(st.da2, dh[j][0], dh[j][1], dh[j][2], dh[j][3]);
+        put(st.h2, silu(f.a2[j][0]), silu(f.a2[j][1]), silu(f.a2[j][2]), silu(f.a2[j][3]));
+        put(st.h1, bf16_round(silu(f.a1[j][0])), bf16_round(silu(f.a1[j][1])),
+            bf16_round(silu(f.a1[j][2])), bf16_round(silu(f.a1[j][3])));
+      }
+      st.dy[g][2 * t] = dy[0]; st.dy[g][2 * t + 1] = dy[1];
+      st.dy[g + 8][2 * t] = dy[2]; st.dy[g + 8][2 * t + 1] = dy[3];
+      // dh1 = da2 W2 (A = da2 as BF16 fragments)
+      uint32_t da[4][4];
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        da[kk][0] = pack_bf16(dh[2 * kk][0], dh[2 * kk][1]);
+        da[kk][1] = pack_bf16(dh[2 * kk][2], dh[2 * kk][3]);
+        da[kk][2] = pack_bf16(dh[2 * kk + 1][0], dh[2 * kk + 1][1]);
+        da[kk][3] = pack_bf16(dh[2 * kk + 1][2], dh[2 * kk + 1][3]);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        float d1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+          const uint32_t bb0 = pair_of(S.w.w2[16 * kk + 2 * t][8 * j + g],
+                                       S.w.w2[16 * kk + 2 * t + 1][8 * j + g]);
+          const uint32_t bb1 = pair_of(S.w.w2[16 * kk + 8 + 2 * t][8 * j + g],
+                                       S.w.w2[16 * kk + 9 + 2 * t][8 * j + g]);
+          mma_bf16(d1, da[kk][0], da[kk][1], da[kk][2], da[kk][3], bb0, bb1);
+        }
+        const int c0 = 8 * j + 2 * t;
+        *reinterpret_cast<float2*>(&st.da1[g][c0]) =
+            make_float2(d1[0] * dsilu(f.a1[j][0]), d1[1] * dsilu(f.a1[j][1]));
+        *reinterpret_cast<float2*>(&st.da1[g + 8][c0]) =
+            make_float2(d1[2] * dsilu(f.a1[j][2]), d1[3] * dsilu(f.a1[j][3]));
+      }
+      if (t == 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          st.x[g][k] = bf16_round(xg[k]);
+          st.x[g + 8][k] = bf16_round(xg8[k]);
+        }
       }
     }
     __syncthreads();
@@ -474,25 +485,27 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
       const WarpStage& sw = S.st[wv];
 #pragma unroll 4
       for (int s = 0; s < 16; ++s) {
-        // this thread's column of 32 (W2) and 4 (W3) neighbouring rows
+        // this thread's column of neighbouring rows of W2 and W3
         const float h1k = sw.h1[s][kcol], h2k = sw.h2[s][kcol];
 #pragma unroll
-        for (int m = 0; m < 32; m += 4) {
-          const float4 d = *reinterpret_cast<const float4*>(&sw.da2[s][32 * nrow + m]);
+        for (int m = 0; m < kR2; m += 4) {
+          const float4 d = *reinterpret_cast<const float4*>(&sw.da2[s][kR2 * nrow + m]);
           gw2[m] = fmaf(d.x, h1k, gw2[m]);
           gw2[m + 1] = fmaf(d.y, h1k, gw2[m + 1]);
           gw2[m + 2] = fmaf(d.z, h1k, gw2[m + 2]);
           gw2[m + 3] = fmaf(d.w, h1k, gw2[m + 3]);
         }
-        const float4 dy4 = *reinterpret_cast<const float4*>(&sw.dy[s][4 * nrow]);
-        gw3[0] = fmaf(dy4.x, h2k, gw3[0]);
-        gw3[1] = fmaf(dy4.y, h2k, gw3[1]);
-        gw3[2] = fmaf(dy4.z, h2k, gw3[2]);
-        gw3[3] = fmaf(dy4.w, h2k, gw3[3]);
+#pragma unroll
+        for (int m = 0; m < kR3; m += 2) {
+          const float2 d = *reinterpret_cast<const float2*>(&sw.dy[s][kR3 * nrow + m]);
+          gw3[m] = fmaf(d.x, h2k, gw3[m]);
+          gw3[m + 1] = fmaf(d.y, h2k, gw3[m + 1]);
+        }
         const float xk = sw.x[s][tid & 3];
-        gw1[0] = fmaf(sw.da1[s][tid >> 2], xk, gw1[0]);
-        gw1[1] = fmaf(sw.da1[s][(tid >> 2) + 32], xk, gw1[1]);
-        gb += (tid < 64) ? sw.da1[s][tid] : sw.da2[s][tid - 64];
+#pragma unroll
+        for (int m = 0; m < kR1; ++m)
+          gw1[m] = fmaf(sw.da1[s][(tid >> 2) + THREADS / kNI * m], xk, gw1[m]);
+        if (tid < 2 * kNH) gb += (tid < kNH) ? sw.da1[s][tid] : sw.da2[s][tid - kNH];
         if (tid < kNO) gb3 += sw.dy[s][tid];
       }
     }
@@ -501,18 +514,20 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_train(const float* __restri
   // per-CTA partials: [blockIdx][kNParam]
   float* out = part + static_cast<long long>(blockIdx.x) * kNParam;
 #pragma unroll
-  for (int m = 0; m < 32; ++m) out[kOffW2 + (32 * nrow + m) * kNH + kcol] = gw2[m];
+  for (int m = 0; m < kR2; ++m) out[kOffW2 + (kR2 * nrow + m) * kNH + kcol] = gw2[m];
 #pragma unroll
-  for (int m = 0; m < 4; ++m) out[kOffW3 + (4 * nrow + m) * kNH + kcol] = gw3[m];
-  out[kOffW1 + (tid >> 2) * kNI + (tid & 3)] = gw1[0];
-  out[kOffW1 + ((tid >> 2) + 32) * kNI + (tid & 3)] = gw1[1];
-  if (tid < 64) out[kOffB1 + tid] = gb; else out[kOffB2 + tid - 64] = gb;
+  for (int m = 0; m < kR3; ++m) out[kOffW3 + (kR3 * nrow + m) * kNH + kcol] = gw3[m];
+#pragma unroll
+  for (int m = 0; m < kR1; ++m)
+    out[kOffW1 + ((tid >> 2) + THREADS / kNI * m) * kNI + (tid & 3)] = gw1[m];
+  if (tid < kNH) out[kOffB1 + tid] = gb;
+  else if (tid < 2 * kNH) out[kOffB2 + tid - kNH] = gb;
   if (tid < kNO) out[kOffB3 + tid] = gb3;
   // loss partial: lanes hold disjoint samples, summed in lane then warp order
   float l = lsum;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) l += __shfl_down_sync(0xffffffffu, l, o);
-  if (lane == 0) S.loss[warp] = l;
+  if (lane == 0 && warp < kWarps) S.loss[warp] = l;
   __syncthreads();
   if (tid == 0) {
     float tot = 0.0f;
@@ -678,10 +693,26 @@ unsigned infer_ctas(long long n, int tile) {
 cudaError_t train_smem_attr() {
   static bool done = false;
   if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_train<32 * kWarps>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sizeof(TrainSmem)));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_mlp_train<64 * kWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(sizeof(TrainSmem)));
   if (e == cudaSuccess) done = true;
   return e;
+}
+
+void launch_train(const float* p, const float* feats, const int* zs, const float* target,
+                  long long b0, long long nb, int grid, float* part, float* lpart,
+                  cudaStream_t s) {
+  // (at most one CTA per SM: the registers of eight warps don't fit twice)
+  if (grid <= train_grid() / 2)
+    k_mlp_train<64 * kWarps><<<grid, 64 * kWarps, sizeof(TrainSmem), s>>>(p, feats, zs, target, b0,
+                                                                          nb, part, lpart);
+  else
+    k_mlp_train<32 * kWarps><<<grid, 32 * kWarps, sizeof(TrainSmem), s>>>(p, feats, zs, target, b0,
+                                                                          nb, part, lpart);
 }
 
 IonDev domain_io(const md_mlp_train_config& c) {
@@ -766,8 +797,7 @@ static md_status md_mlp_loss_grad_device_body(const float* params, const float* 
   if (e != cudaSuccess) return report_cuda_error(e, "surrogate gradient partials");
   float* lpart = part + static_cast<size_t>(grid) * md::kNParam;
   {
-    md::k_mlp_train<<<grid, 32 * md::kWarps, sizeof(md::TrainSmem), s>>>(params, feats, z, target,
-                                                                         0, n, part, lpart);
+    md::launch_train(params, feats, z, target, 0, n, grid, part, lpart, s);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) {
@@ -898,8 +928,7 @@ static md_status md_mlp_train_body(const md_mlp_train_config* cfg, float* params
       // cosine decay of the learning rate to 1 % at the end
       const double prog = (step - 1) / static_cast<double>(total);
       const float lr = static_cast<float>(cfg->lr * (0.01 + 0.99 * 0.5 * (1.0 + std::cos(3.14159265358979323846 * prog))));
-      md::k_mlp_train<<<grid, 32 * md::kWarps, sizeof(md::TrainSmem), s>>>(p, feats, zs, target,
-                                                                           b0, nb, part, lpart);
+      md::launch_train(p, feats, zs, target, b0, nb, grid, part, lpart, s);
       const bool want_loss = b == batches - 1 || (ep == 0 && b == 0);
       md::k_mlp_adam<<<md::kAdamBlocks + (want_loss ? 1 : 0), 32 * md::kAdamWarps, 0, s>>>(
           p, m, v, part, grid, lr, 0.9f, 0.999f, 1e-8f, static_cast<int>(step), nullptr, lpart,
