@@ -101,6 +101,7 @@ int ion_fix_targets_per_cta();
 cudaError_t ion_fix_blocks_per_sm(int* out);
 // Shape of the field-only pass kernel (clusters whose moments come from the
 // cell list).
+int ion_sum_tile();
 int ion_sum_targets_per_cta();
 cudaError_t ion_sum_blocks_per_sm(int* out);
 

@@ -386,10 +386,19 @@ __global__ void __launch_bounds__(THREADS) k_ion_field(const IonArgs a) {
 // uses atomic counters.  The near test is the field pass's: the FP32
 // r^2 + eps^2 of the j-stream positions against r_loc^2 + eps^2.
 
+constexpr int kSumTile = 512;  // sources per stage of the field-only kernel
+
+// Records of the cluster below the next free electron slot.
+__device__ __forceinline__ long long live_records(const IonArgs& a) {
+  long long n = __ldcg(a.next_slot);
+  n = n > a.ion.slot_base ? n : a.ion.slot_base;
+  return n < a.c.n_pad ? (n > 0 ? n : 0) : a.c.n_pad;
+}
+
 // Field of the live records at the ions: CTA (x, y) sums segment y of the
 // live records for R x THREADS ions and writes its field to the scratch of
-// segment y.  4000 ions, 34000 live records: 168 us with 17 segments of whole
-// tiles (68 CTAs), 60 us with 112.
+// segment y.  4000 ions, 34000 live records: 168 us with 17 segments (68 CTAs),
+// 66 us with a tile to a segment.
 template <int THREADS, int R, int TILE, int STAGES, bool PACK>
 __global__ void __launch_bounds__(THREADS) k_ion_field_sum(const IonArgs a) {
   __shared__ Stage<TILE, STAGES> sm;
@@ -405,13 +414,10 @@ __global__ void __launch_bounds__(THREADS) k_ion_field_sum(const IonArgs a) {
   }
   __syncthreads();
   const float4* __restrict__ cur = (step & 1) ? a.posq1 : a.posq0;
-  long long n_live = __ldcg(a.next_slot);
-  n_live = n_live > a.ion.slot_base ? n_live : a.ion.slot_base;
-  n_live = n_live < a.c.n_pad ? (n_live > 0 ? n_live : 0) : a.c.n_pad;
+  const long long n_live = live_records(a);
   const long long per_seg = (n_live + gridDim.y - 1) / gridDim.y;
-  // whole tiles, unless the segments are that short
-  const long long unit = per_seg >= 4 * TILE ? TILE : 64;
-  const long long seg_len = (per_seg + unit - 1) / unit * unit;
+  // whole tiles: a tile's FP32 sum is then the same for any number of segments
+  const long long seg_len = (per_seg + TILE - 1) / TILE * TILE;
   const long long j0 = static_cast<long long>(blockIdx.y) * seg_len;
   const long long ns = (j0 >= n_live) ? 0 : ((n_live - j0 < seg_len) ? n_live - j0 : seg_len);
   const long long t0 = static_cast<long long>(blockIdx.x) * (THREADS * R);
@@ -907,11 +913,16 @@ __global__ void __launch_bounds__(256) k_ion_inputs(const IonArgs a) {
   ion_outputs(a, t, f, lax, lay, W, S, Q);
 }
 
-// After the field-only kernel and the cell list's moments: 32 ions per CTA,
-// each of eight warps adds every eighth segment, the first warp the eight sums
-// (4000 ions: 23 us with a thread per ion over the strided segments).
+// After the field-only kernel and the cell list's moments: 32 ions per CTA, its
+// eight warps share the segments, whose fields are then added in order.  With a
+// tile to a segment in the scratch (sum_segs > 0) the sum_segs segments of whole
+// tiles are formed here, by the compensated sum that the source loop would have
+// made of their tiles: the pass's field does not depend on how its kernel was
+// spread over the SMs.  (4000 ions: 23 us with a thread per ion over the strided
+// segments, 12.6 now.)
 __global__ void __launch_bounds__(256) k_ion_inputs_sum(const IonArgs a) {
-  __shared__ double s_f[3][8][32];
+  __shared__ double s_seg[3][kIonMaxSeg][32];
+  __shared__ double s_f[3][32];
   __shared__ double s_las[2];
   const long long step = __ldcg(a.step);
   if (!pass_active(a, step)) return;
@@ -920,25 +931,43 @@ __global__ void __launch_bounds__(256) k_ion_inputs_sum(const IonArgs a) {
   if (t == 0 && warp == 0) *a.pass_slot = *a.next_slot;
   if (threadIdx.x == 255) s_las[0] = laser_ax(a.c, a.c.t0 + static_cast<double>(step) * a.c.dt,
                                               &s_las[1]);
-  double f[3] = {0.0, 0.0, 0.0};
+  const int nseg = a.sum_segs > 0 ? a.sum_segs : a.nseg;
+  const long long n_live = live_records(a);
+  const int tiles = static_cast<int>((n_live + kSumTile - 1) / kSumTile);
+  const int per = static_cast<int>(((n_live + nseg - 1) / nseg + kSumTile - 1) / kSumTile);
   if (t < nn) {
-#pragma unroll 4
-    for (int sg = warp; sg < a.nseg; sg += 8) {
+    for (int sg = warp; sg < nseg; sg += 8) {
       const double* sc = a.scratch + 3 * static_cast<long long>(sg) * nn + t;
+      if (a.sum_segs <= 0) {
 #pragma unroll
-      for (int c = 0; c < 3; ++c) f[c] += sc[c * nn];
+        for (int c = 0; c < 3; ++c) s_seg[c][sg][lane] = sc[c * nn];
+        continue;
+      }
+      float sum[3] = {0.0f, 0.0f, 0.0f}, comp[3] = {0.0f, 0.0f, 0.0f};
+      const int end = (sg + 1) * per < tiles ? (sg + 1) * per : tiles;
+#pragma unroll 4
+      for (int k = sg * per; k < end; ++k) {
+        const double* tk = a.scratch + 3 * static_cast<long long>(k) * nn + t;
+        const double v[3] = {tk[0], tk[nn], tk[2 * nn]};
+        // (a tile without live or charged records was never folded)
+        if (v[0] == 0.0 && v[1] == 0.0 && v[2] == 0.0) continue;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) kahan_add(sum[c], comp[c], -static_cast<float>(v[c]));
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        s_seg[c][sg][lane] = -(static_cast<double>(sum[c]) - comp[c]);
     }
   }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) s_f[c][warp][lane] = f[c];
+  __syncthreads();
+  if (warp < 3) {
+    double f = 0.0;
+    for (int sg = 0; sg < nseg; ++sg) f += s_seg[warp][sg][lane];
+    s_f[warp][lane] = f;
+  }
   __syncthreads();
   if (warp != 0 || t >= nn) return;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    f[c] = s_f[c][0][lane];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) f[c] += s_f[c][w][lane];
-  }
+  const double f[3] = {s_f[0][lane], s_f[1][lane], s_f[2][lane]};
   const double* m = a.scratch + 3 * static_cast<long long>(a.nseg) * nn + kIonMom * t;
   const double S[3] = {m[1], m[2], m[3]};
   ion_outputs(a, t, f, s_las[0], s_las[1], m[0], S, m[4]);
@@ -1252,7 +1281,6 @@ constexpr int kIonTile = 512;
 // packed source loop
 constexpr int kSumThreads = 128;
 constexpr int kSumR = 8;
-constexpr int kSumTile = 512;
 constexpr bool kSumPacked = true;
 // the charge-change field: the step kernel's packed source loop (eight
 // targets per thread); the minimum-image twin is scalar (four per thread)
@@ -1276,6 +1304,8 @@ int ion_field_targets_per_cta() { return kIonThreads * kIonR; }
 
 int ion_fix_targets_per_cta() { return kFixThreads * kFixR; }
 
+int ion_sum_tile() { return kSumTile; }
+
 int ion_sum_targets_per_cta() { return kSumThreads * kSumR; }
 
 cudaError_t ion_sum_blocks_per_sm(int* out) {
@@ -1296,7 +1326,9 @@ cudaError_t ion_fix_blocks_per_sm(int* out) {
 cudaError_t launch_ion_pass(const IonArgs& a, cudaStream_t s) {
   if (a.ion.n_ions <= 0) return cudaSuccess;
   const bool sum_only = !a.min_image && a.cells.count;
-  if (a.nseg < 1 || a.nseg > (sum_only ? kIonSumSeg : kIonMaxSeg)) return cudaErrorInvalidValue;
+  if (a.nseg < 1 || a.nseg > (sum_only && a.sum_segs > 0 ? kIonSumSeg : kIonMaxSeg) ||
+      a.sum_segs > kIonMaxSeg)
+    return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
   if (!sum_only) {
     // field and moments in one source loop

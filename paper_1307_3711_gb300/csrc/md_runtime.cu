@@ -769,8 +769,8 @@ constexpr long long kMutBigRecords = 40000;
 constexpr long long kMutMinTiles = 2;
 
 // Pairs (records squared, summed over the clusters) up to which the small step
-// is taken: 24.6 us per step at 5000 records against 31 with each pair once,
-// 42.3 against 41.2 at 8000, 66 against 55 at 10000.
+// is taken: 23.8 us per step at 5000 records against 31 with each pair once,
+// 41.5 against 41.2 at 8000, 66 against 55 at 10000.
 constexpr double kSmallMaxPairs = 9.0e3 * 9.0e3;
 
 // The small step, if the context is that small: 16 or 32 targets per CTA,
@@ -1011,11 +1011,8 @@ md::IonArgs ion_args(md_ctx* c, int ci, int force) {
     const long long ion_blocks = (a.ion.n_ions + per - 1) / per;
     const long long cap = std::max(1LL, static_cast<long long>(
         sum_only ? c->ion_sum_bps : c->ion_field_bps) * c->sm_count);
-    // (the field-only kernel: segments of 256 records or more, so that a few
-    // thousand ions, a handful of blocks, still cover the SMs)
-    const long long by_len = std::max(1LL, static_cast<long long>(a.c.n_pad) / (sum_only ? 256 : 2048));
-    const int smax = static_cast<int>(
-        std::min<long long>(sum_only ? md::kIonSumSeg : md::kIonMaxSeg, by_len));
+    const long long by_len = std::max(1LL, static_cast<long long>(a.c.n_pad) / 2048);
+    const int smax = static_cast<int>(std::min<long long>(md::kIonMaxSeg, by_len));
     double best = -1.0;
     a.nseg = 1;
     for (int sg = 1; sg <= smax; ++sg) {
@@ -1026,6 +1023,14 @@ md::IonArgs ion_args(md_ctx* c, int ci, int force) {
         best = score;
         a.nseg = sg;
       }
+    }
+    // a few thousand ions are a handful of blocks: a CTA per tile covers the SMs,
+    // and the tiles' sums are added as those segments would have been
+    a.sum_segs = 0;
+    const long long tiles = (a.c.n_pad + md::ion_sum_tile() - 1) / md::ion_sum_tile();
+    if (sum_only && tiles <= md::kIonSumSeg && tiles > a.nseg && ion_blocks * a.nseg < cap) {
+      a.sum_segs = a.nseg;
+      a.nseg = static_cast<int>(tiles);
     }
   }
   a.out = c->d_ion_out + 4 * c->ion_out_off[ci];

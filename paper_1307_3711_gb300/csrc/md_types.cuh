@@ -250,6 +250,7 @@ struct IonArgs {
                       // sw du_z, sw du^2, u_ref (3) of each source segment (du = u -
                       // u_ref, u_ref = the segment's first local electron's u)
   int nseg;           // source segments of the field pass (equal shares of the live records)
+  int sum_segs;       // > 0: the scratch holds a tile per segment, to be added in sum_segs segments
   int* blk_fired;     // fired ions per block of 64 of the decision
   long long* pass_slot;  // first free slot at the start of the pass
   double* out;        // [n_ions][4]: |E|, ne (cm^-3), Te (eV), P
