@@ -327,6 +327,13 @@ struct Acc {
   }
 };
 
+// Sum of two compensated sums (value s - c), with the rounding of s kept in c.
+__device__ __forceinline__ void join_sums(float& s, float& c, float s2, float c2) {
+  const float t = s + s2, b = t - s;
+  c = (c + c2) - ((s - (t - b)) + (s2 - b));
+  s = t;
+}
+
 __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
   const float y = v - c;
   const float t = s + y;

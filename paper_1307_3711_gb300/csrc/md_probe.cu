@@ -43,13 +43,6 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kMaxCluster = 8;
 constexpr int kLargeTile = 4096;  // (two stages of it leave room for one CTA per SM)
 
-// Sum of two compensated sums (value s - c), with the rounding of s kept in c.
-__device__ __forceinline__ void join(float& s, float& c, float s2, float c2) {
-  const float t = s + s2, b = t - s;
-  c = (c + c2) - ((s - (t - b)) + (s2 - b));
-  s = t;
-}
-
 template <int TL, int R, bool POT, int kTile, int kStages>
 struct ProbeSmem {
   Stage<kTile, kStages> st;
@@ -171,7 +164,7 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
   auto put = [&](int c, int r, float v, float w) {
 #pragma unroll
     for (int d = TL; d < 32; d <<= 1)
-      join(v, w, __shfl_xor_sync(0xffffffffu, v, d), __shfl_xor_sync(0xffffffffu, w, d));
+      join_sums(v, w, __shfl_xor_sync(0xffffffffu, v, d), __shfl_xor_sync(0xffffffffu, w, d));
     if (lane < TL) S.e[c][tid >> 5][tl + r * TL] = make_float2(v, w);
   };
 #pragma unroll
@@ -192,11 +185,11 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
     if (v < kVals) {
       s = S.e[c][tid % 8][t];
       const float2 o = S.e[c][tid % 8 + 8][t];
-      join(s.x, s.y, o.x, o.y);
+      join_sums(s.x, s.y, o.x, o.y);
     }
 #pragma unroll
     for (int d = 4; d > 0; d >>= 1)
-      join(s.x, s.y, __shfl_xor_sync(0xffffffffu, s.x, d), __shfl_xor_sync(0xffffffffu, s.y, d));
+      join_sums(s.x, s.y, __shfl_xor_sync(0xffffffffu, s.x, d), __shfl_xor_sync(0xffffffffu, s.y, d));
     if (v < kVals && tid % 8 == 0) {
       const double val = static_cast<double>(s.x) - s.y;
       to[v] = c < 3 ? -val : val;

@@ -5,15 +5,17 @@
 // Here a CTA takes kTargets targets, few enough that the CTAs cover the SMs,
 // and all its warps share them: every (target lane, slice) thread sums the
 // sources j = slice, slice + kSlices, ... of each staged tile, the slices' sums
-// are added in a fixed order in FP64 through shared memory, and the targets are
+// are added in a fixed order as compensated FP32 pairs (an FP64 instruction takes
+// its pipe 16 cycles) through shared memory, and the targets are
 // pushed by the CTA that summed them: one launch, no partial sums
 // in memory, no ticket.  The laser's FP64 envelope and sine run in two warps of
 // their own beside the sums, the targets' state is loaded before them, and the
 // step counter is advanced while they run.
 //
-// Measured (graph replay, us per step): 8.0 at 2000 records (53 with the step
-// kernel's default configuration), 6.5 at 1000, 12.7 at 3000, 15.5 at 4000,
-// 42 at 8000; about 6 us of each are the launch, the loads and the push.  More
+// Measured (graph replay, us per step): 6.8 at 2000 records (53 with the step
+// kernel's default configuration; 8.1 with the slices' sums in FP64 and the last
+// few sources of a tile one by one), 5.4 at 1000, 11.9 at 3000, 14.9 at 4000, 41.5
+// at 8000; about 5 us of each are the launch, the loads and the push.  More
 // threads per CTA (512, 768), two or four targets per thread, 8 targets per
 // CTA, two stages, a register cap for a fourth CTA per SM and programmatic
 // launches were slower or no faster.
@@ -30,8 +32,8 @@ constexpr int kStages = 4;
 template <int THREADS, int TL, int R, bool POT>
 struct SmallSmem {
   Stage<kTile, kStages> st;
-  double e[POT ? 4 : 3][THREADS / TL][TL * R];  // the slices' sums
-  double sum[POT ? 4 : 3][TL * R];
+  float2 e[POT ? 4 : 3][THREADS / 32][TL * R];  // the warps' sums (value x - y)
+  float2 sum[POT ? 4 : 3][TL * R];
   ClusterDev c;
   double amp, sn, cs;  // the laser at t_n
   int abort;
@@ -115,11 +117,7 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
         }
         const int rem = n_pad - t * kTile, cnt = rem < kTile ? rem : kTile;
         const uint32_t tile = smem_u32(&S.st.tile[s][0]);
-        int k = slice;
-        for (; k + 7 * kSlices < cnt; k += 8 * kSlices) {
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            pair<R, POT>(lds_f4(tile + 16u * (k + q * kSlices)), xi, yi, zi, eps2, acc);
+        auto fold_phi = [&] {
           if constexpr (POT) {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -127,9 +125,25 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
               acc.ap[r] = 0.0f;
             }
           }
+        };
+        int k = slice;
+        for (; k + 7 * kSlices < cnt; k += 8 * kSlices) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            pair<R, POT>(lds_f4(tile + 16u * (k + q * kSlices)), xi, yi, zi, eps2, acc);
+          fold_phi();
         }
-        for (; k < cnt; k += kSlices)
-          pair<R, POT>(lds_f4(tile + 16u * k), xi, yi, zi, eps2, acc);
+        if (k < cnt) {
+          // the last few at once too: past the end the tile's last source, uncharged
+#pragma unroll
+          for (int q = 0; q < 7; ++q) {
+            const int j = k + q * kSlices;
+            float4 p = lds_f4(tile + 16u * (j < cnt ? j : cnt - 1));
+            p.w = j < cnt ? p.w : 0.0f;
+            pair<R, POT>(p, xi, yi, zi, eps2, acc);
+          }
+          fold_phi();
+        }
         fold<R, POT>(acc);
       }
     }
@@ -143,26 +157,39 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
     }
   }
   if (tid < THREADS) {
+    auto put = [&](int c, int r, float v, float w) {
+#pragma unroll
+      for (int d = TL; d < 32; d <<= 1)
+        join_sums(v, w, __shfl_xor_sync(0xffffffffu, v, d), __shfl_xor_sync(0xffffffffu, w, d));
+      if ((tid & 31) < TL) S.e[c][tid >> 5][tl + r * TL] = make_float2(v, w);
+    };
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      S.e[0][slice][tl + r * TL] = -(static_cast<double>(acc.sx[r]) - acc.cx[r]);
-      S.e[1][slice][tl + r * TL] = -(static_cast<double>(acc.sy[r]) - acc.cy[r]);
-      S.e[2][slice][tl + r * TL] = -(static_cast<double>(acc.sz[r]) - acc.cz[r]);
-      if constexpr (POT) S.e[3][slice][tl + r * TL] = static_cast<double>(acc.sp[r]) - acc.cp[r];
+      put(0, r, acc.sx[r], acc.cx[r]);
+      put(1, r, acc.sy[r], acc.cy[r]);
+      put(2, r, acc.sz[r], acc.cz[r]);
+      if constexpr (POT) put(3, r, acc.sp[r], acc.cp[r]);
     }
   }
   __syncthreads();
   if (S.abort) return;
-  for (int k = tid; tid < THREADS && k < C * kTargets; k += THREADS) {
-    const int c = k / kTargets, t = k % kTargets;
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    static_assert(kSlices % 4 == 0, "four interleaved sums");
+  // each value's warps: kJoin neighbouring lanes add some each, then each other's
+  constexpr int kWarps = THREADS / 32, kJoin = THREADS / (4 * kTargets);
+  static_assert(kJoin >= 1 && kJoin <= kWarps, "lanes per value");
+  if (tid < THREADS) {
+    const int k = tid / kJoin, c = k / kTargets, t = k % kTargets;
+    float2 v = make_float2(0.0f, 0.0f);
+    if (k < C * kTargets) {
+      v = S.e[c][tid % kJoin][t];
 #pragma unroll
-    for (int s = 0; s < kSlices; s += 4) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) v[q] += S.e[c][s + q][t];
+      for (int w = tid % kJoin + kJoin; w < kWarps; w += kJoin)
+        join_sums(v.x, v.y, S.e[c][w][t].x, S.e[c][w][t].y);
     }
-    S.sum[c][t] = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+    for (int d = kJoin / 2; d > 0; d >>= 1)
+      join_sums(v.x, v.y, __shfl_xor_sync(0xffffffffu, v.x, d),
+                __shfl_xor_sync(0xffffffffu, v.y, d));
+    if (k < C * kTargets && tid % kJoin == 0) S.sum[c][t] = v;
   }
   __syncthreads();
   if (pushes) {
@@ -170,13 +197,16 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
     float las[6];
     laser_of(S.amp, S.sn, S.cs, S.c.pol, las);
     const double t_next = S.c.t0 + static_cast<double>(step + 1) * S.c.dt;
+    auto value = [&](int c) {
+      const float2 v = S.sum[c][tid];
+      return static_cast<double>(v.x) - static_cast<double>(v.y);
+    };
     if constexpr (POT) {
-      const double ph = S.sum[3][tid] - static_cast<double>(cur[i].w * rsqrt_mufu(S.c.eps2));
-      push_loaded<DET, true>(a, S.c, i, st, S.sum[0][tid], S.sum[1][tid], S.sum[2][tid], las,
-                             t_next, cur, nxt, ph);
+      const double ph = value(3) - static_cast<double>(cur[i].w * rsqrt_mufu(S.c.eps2));
+      push_loaded<DET, true>(a, S.c, i, st, -value(0), -value(1), -value(2), las, t_next, cur,
+                             nxt, ph);
     } else {
-      push_loaded<DET>(a, S.c, i, st, S.sum[0][tid], S.sum[1][tid], S.sum[2][tid], las, t_next,
-                       cur, nxt);
+      push_loaded<DET>(a, S.c, i, st, -value(0), -value(1), -value(2), las, t_next, cur, nxt);
     }
   }
 }
