@@ -19,6 +19,7 @@ import argparse
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -36,11 +37,16 @@ from paper_1307_3711_gb300 import synth  # noqa: E402
 METRIC = "Coulomb pair interactions/s & steps/s at N=200k on 1 GB300; force err vs FP64"
 UNIT = "pair/s"
 RECORD_BYTES = 3 * 8 + 3 * 8 + 4 + 8 + 8 + 1   # x, u, z, mass, w, kind per record
+# FP32 instructions per counted pair: a kernel that sums every ordered pair (k_step)
+# issues 12, one that evaluates a pair once for both its records (k_mut_pairs) 14
+# per two of them
 FP32_INSTR_PER_PAIR = 12
+FP32_INSTR_PER_PAIR_ONCE = 7
 # DRAM bytes (read + write) per launch of the step kernel, from one 1-pass ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of the named workload
 # at full size in the named kernel configuration (threads, r, tile, packed,
-# jsplit); reported only when the timed run uses that configuration.
+# jsplit); reported only when the timed run's step is k_step in that
+# configuration.
 STEP_TRAFFIC_BYTES = {("xe3_200k", 200000, 128, 8, 512, True, 9): 15.77e6,
                       ("xe3_200k", 200000, 128, 8, 256, True, -4): 20.16e6}
 L2_FLUSH_BYTES = 512 << 20
@@ -280,10 +286,7 @@ def ionizing_context(md, n, rates, rank, stream, train=None):
               "r_create", "ip_ev", "q_outer"):
         setattr(cfg, f, getattr(ion, f))
     ctx = md.Context([cfg], [md.HostParticles.from_cluster(c)], stream=stream)
-    # ion field, inputs, (surrogate rates,) decision, apply, charge-change
-    # correction, ion push, step
-    info = {"rates": rates, "t0": w.t0,
-            "kernels_per_step": 7 + (1 if model == md.RATES_MLP else 0)}
+    info = {"rates": rates, "t0": w.t0}
     if model == md.RATES_MLP:
         if train is None:
             tc = md.mlp_train_config(synth.ARGON, n_samples=10 << 20, epochs=80, batch=8192,
@@ -337,10 +340,9 @@ def precision_study(md, ctx, w, n_targets=10000, n_oracle=2000, seed=0):
             "metric": "|E - E_fp64| / max(|E_fp64|, rms|E_fp64|), state after the timed steps"}
 
 
-def driven_precision(md, args, rank, stream, tuning):
+def driven_precision(md, args, rank, stream):
     """The precision case's driven run: the same 1M-particle cluster with the
-    laser on (a0 = 0.1, 100 fs sin^2, from the envelope's peak), the same
-    kernel configuration, as many
+    laser on (a0 = 0.1, 100 fs sin^2, from the envelope's peak), as many
     steps as the timed run; then the FP32/Kahan field against the FP64 GPU
     reference (and the oracle) on the state the laser has pulled apart, and
     the energy the laser has put in."""
@@ -349,7 +351,6 @@ def driven_precision(md, args, rank, stream, tuning):
     wd.t0 = 0.5 * wd.tau          # from the peak of the sin^2 envelope
     with md.Context([md.config_from_workload(wd)], [md.HostParticles.from_cluster(wd.cluster)],
                     stream=stream.cuda_stream) as cd:
-        cd.set_tuning(tuning[0], tuning[1], tuning[2], 0, tuning[4], tuning[5], tuning[6])
         d0 = cd.diagnostics(0)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(stream)
@@ -384,16 +385,43 @@ def event_steps(ctx, stream, flush, steps, after=None):
     return ms, extra
 
 
-def alu_frac(pairs_per_s: float, sms: int, clocks: dict) -> dict:
-    """Fraction of the FP32 roofline (128 lanes x SMs x clock / 12) at the
-    median SM clock sampled during the run and at the maximum clock."""
+def step_kernels(ctx) -> dict:
+    """The library's kernels of one further step of the context, with their counts
+    (a profiler's record, taken after the timed parts)."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    out = {}
+    for _ in range(3):  # (the profiler's first session in a process may record nothing)
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            ctx.step(1)
+            torch.cuda.synchronize()
+        for e in p.key_averages():
+            m = re.search(r"md::(?:\(anonymous namespace\)::)?(k_\w+)", e.key)
+            if m:
+                out[m.group(1)] = out.get(m.group(1), 0) + e.count
+        if out:
+            break
+    return out or {"not recorded (at least one)": 1}
+
+
+def instr_per_pair(kernels: dict) -> int:
+    return FP32_INSTR_PER_PAIR_ONCE if "k_mut_pairs" in kernels else FP32_INSTR_PER_PAIR
+
+
+def alu_frac(pairs_per_s: float, sms: int, clocks: dict, kernels: dict) -> dict:
+    """Fraction of the FP32 roofline (128 lanes x SMs x clock / instructions per
+    counted pair) at the median SM clock sampled during the run and at the
+    maximum clock."""
     clk = clocks.get("sm_mhz") or 2070.0
-    peak = 128.0 * sms * clk * 1e6 / FP32_INSTR_PER_PAIR
+    instr = instr_per_pair(kernels)
+    peak = 128.0 * sms * clk * 1e6 / instr
     return {"frac": pairs_per_s / peak, "peak_gpair_s": peak / 1e9, "sm_mhz": clk,
-            "frac_at_max_clock": pairs_per_s / (128.0 * sms * 2070e6 / FP32_INSTR_PER_PAIR)}
+            "fp32_instr_per_pair": instr, "step_kernels": kernels,
+            "frac_at_max_clock": pairs_per_s / (128.0 * sms * 2070e6 / instr)}
 
 
-def secondary_measurements(md, stream, flush, sms, gpu_id, tuning, steps=3, warmup=2):
+def secondary_measurements(md, stream, flush, sms, gpu_id, steps=3, warmup=2):
     """Driver-visible numbers of the other configurations, each timed with
     CUDA events (L2 flushed between steps, outside the events) and its own
     nvidia-smi clock record:
@@ -404,9 +432,9 @@ def secondary_measurements(md, stream, flush, sms, gpu_id, tuning, steps=3, warm
                       both on the same seed;
       precision_1m -- 500k Ar+ + 500k e: the step time, and the FP32/Kahan
                       field against the FP64 GPU reference and the oracle.
-    The 1M context runs the step kernel configuration and source split that
-    the headline's autotuner chose (`tuning`); the ionizing contexts run
-    IONIZING_TUNING with a segment count chosen for balance."""
+    The 1M context runs the plan that the library chooses by itself; the
+    ionizing contexts run IONIZING_TUNING with a segment count chosen for
+    balance."""
     import torch
     out = {}
     cs = stream.cuda_stream
@@ -432,12 +460,15 @@ def secondary_measurements(md, stream, flush, sms, gpu_id, tuning, steps=3, warm
         ms, _ = event_steps(ctx, stream, flush, 2 * steps)
         clocks = sampler.stop()
         tun = ctx.tuning()
+        kernels = step_kernels(ctx)
     rate = pairs / (statistics.mean(ms) / 1e3)
     out["scan256"] = dict({"clusters": 256, "records": int(sum(p.n for p in parts)),
                            "pairs_per_step": pairs, "steps": len(ms),
                            "ms_per_step": statistics.mean(ms), "pairs_per_s": rate,
-                           "tuning": list(tun), "clocks": clocks, "gpu_launches": len(ms),
-                           "wall_s": time.perf_counter() - t_wall}, **alu_frac(rate, sms, clocks))
+                           "tuning": list(tun), "clocks": clocks,
+                           "gpu_launches": len(ms) * sum(kernels.values()),
+                           "wall_s": time.perf_counter() - t_wall},
+                          **alu_frac(rate, sms, clocks, kernels))
 
     # ar_ionize, plain rates then the surrogate, same seed
     n_atoms = 200000
@@ -456,6 +487,7 @@ def secondary_measurements(md, stream, flush, sms, gpu_id, tuning, steps=3, warm
             ms, act = event_steps(ctx, stream, flush, steps, after=lambda c: c.count_active(0))
             clocks = sampler.stop()
             d = ctx.diagnostics(0)
+            kernels = step_kernels(ctx)
         pairs = float(np.mean([float(a) ** 2 for a in act]))
         rate = pairs / (statistics.mean(ms) / 1e3)
         ent = dict({"atoms": n_atoms, "records": ws[0].cluster.n, "steps": steps,
@@ -464,9 +496,9 @@ def secondary_measurements(md, stream, flush, sms, gpu_id, tuning, steps=3, warm
                     "pairs_per_s": rate,
                     "pairs_counted": "(active records after each step's ionization pass)^2",
                     "charge_fractions": (d["charge_count"][:9] / n_atoms).tolist(),
-                    "clocks": clocks, "gpu_launches": steps * info["kernels_per_step"],
+                    "clocks": clocks, "gpu_launches": steps * sum(kernels.values()),
                     "wall_s": time.perf_counter() - t_wall},
-                   **alu_frac(rate, sms, clocks))
+                   **alu_frac(rate, sms, clocks, kernels))
         if "surrogate_training" in info:
             ent["surrogate_training"] = info["surrogate_training"]
         out[f"ar_ionize_{rates}"] = ent
@@ -481,22 +513,22 @@ def secondary_measurements(md, stream, flush, sms, gpu_id, tuning, steps=3, warm
     w = synth.precision_1m(seed=0, a0=0.0)
     with md.Context([md.config_from_workload(w)], [md.HostParticles.from_cluster(w.cluster)],
                     stream=cs) as ctx:
-        ctx.set_tuning(tuning[0], tuning[1], tuning[2], 0, tuning[4], tuning[5], tuning[6])
         ctx.step(1)
         sampler = ClockSampler(gpu_id)
         time.sleep(0.3)
         ms, _ = event_steps(ctx, stream, flush, 2)
         clocks = sampler.stop()
         tun = ctx.tuning()
+        kernels = step_kernels(ctx)
         prec = precision_study(md, ctx, w, n_targets=10000, n_oracle=1000)
     pairs = float(w.cluster.n) ** 2
     rate = pairs / (statistics.mean(ms) / 1e3)
     out["precision_1m"] = dict({"n_particles": w.cluster.n, "steps": len(ms),
                                 "ms_per_step": statistics.mean(ms), "pairs_per_s": rate,
                                 "tuning": list(tun), "clocks": clocks,
-                                "gpu_launches": len(ms), "precision": prec,
-                                "wall_s": time.perf_counter() - t_wall},
-                               **alu_frac(rate, sms, clocks))
+                                "gpu_launches": len(ms) * sum(kernels.values()),
+                                "precision": prec, "wall_s": time.perf_counter() - t_wall},
+                               **alu_frac(rate, sms, clocks, kernels))
     torch.cuda.synchronize()
     return out
 
@@ -596,10 +628,11 @@ def run_nscale(args):
                 ms.append(e0.elapsed_time(e1))
             t = statistics.mean(ms)
             pairs = float(n) ** 2
-            peak = 128.0 * sms * 2070e6 / FP32_INSTR_PER_PAIR
+            kernels = step_kernels(ctx)
+            peak = 128.0 * sms * 2070e6 / instr_per_pair(kernels)
             rows.append({"n": n, "ms_per_step": t, "pairs_per_s": pairs / (t / 1e3),
                          "frac_at_max_clock": pairs / (t / 1e3) / peak,
-                         "tuning": list(ctx.tuning())})
+                         "step_kernels": kernels, "tuning": list(ctx.tuning())})
     cpu = None if args.no_cpu_baseline else oracle_step_scaling()
     print(json.dumps({"workload": "nscale: xe3 clusters at the density of the 400k case",
                       "device": gpu_name, "l2": "flushed between timed steps",
@@ -716,6 +749,7 @@ def run_iedf(args):
             done += kk
         zs = ctx.get_particles(0).z[:n]
         det, inside = ctx.iedf(0)
+        kernels = step_kernels(ctx)
     if rank != 0:
         return
     centers = (np.arange(nb) + 0.5) * e_max / nb
@@ -738,8 +772,7 @@ def run_iedf(args):
                        "mean_charge": float(zs.mean())},
         "iedf": iedf, "ions_inside": int(inside.sum()),
         "inside_mean_kev": float((hin * centers).sum() / max(hin.sum(), 1.0) / 1e3),
-        # ion field, inputs, decision, apply, charge-change correction, ion push, step
-        "gpu_launches": 7 * nsteps,
+        "gpu_launches": sum(kernels.values()) * nsteps,
     }
     print(json.dumps(line), flush=True)
 
@@ -839,7 +872,7 @@ def run_native(args):
             "steps": args.steps, "dt": w.dt, "laser": "off",
             "what": "(E_total after - before) / |PE before| over the timed steps (the cluster "
                     "starts cold: KE = 0), FP64 sums, m_e c^2 units"}
-        precision["driven"] = driven_precision(md, args, rank, stream, tuning)
+        precision["driven"] = driven_precision(md, args, rank, stream)
     ion_state = None
     if ionizing:
         # the state the timed steps reached (the end-to-end leg below repeats
@@ -856,13 +889,10 @@ def run_native(args):
                                        + ("surrogate rates, " if args.rates == "mlp" else "")
                                        + "decision, fused Coulomb/laser/push step")
 
-    # FP32 roofline of the step kernel (the only kernel of a step)
+    # FP32 roofline of the step's pair sum
     ffma_per_s, ffma2_per_s = md.measure_fp32_peak(stream.cuda_stream)
     achieved = pairs_local / (statistics.mean(step_ms) / 1e3)
-    peak_probe = max(ffma_per_s, ffma2_per_s) / FP32_INSTR_PER_PAIR
     clk = clocks.get("sm_mhz") or None
-    peak_clock = 128.0 * sms * clk * 1e6 / FP32_INSTR_PER_PAIR if clk else None
-    peak_max = 128.0 * sms * 2070e6 / FP32_INSTR_PER_PAIR
 
     # end to end through the C ABI with host buffers: upload, step, download.
     # An ionizing run repeats one step from the state its timed steps reached.
@@ -909,12 +939,16 @@ def run_native(args):
                "steps_per_s": rate / (float(w.cluster.n) ** 2),
                "single_thread": single_thread_rate(w, 3.0)}
 
-    launches_per_step = info.get("kernels_per_step", 1)
+    kernels = step_kernels(ctx)
+    instr = instr_per_pair(kernels)
+    peak_probe = max(ffma_per_s, ffma2_per_s) / instr
+    peak_clock = 128.0 * sms * clk * 1e6 / instr if clk else None
+    peak_max = 128.0 * sms * 2070e6 / instr
     ctx.close()
     secondary = None
     if (rank == 0 and world == 1 and args.workload == "xe3_200k" and not args.no_secondary):
         t_sec = time.perf_counter()
-        secondary = secondary_measurements(md, stream, flush, sms, gpu_id_for(local), tuning)
+        secondary = secondary_measurements(md, stream, flush, sms, gpu_id_for(local))
         secondary["wall_s"] = time.perf_counter() - t_sec
     dist.close()
     if rank != 0:
@@ -958,15 +992,19 @@ def run_native(args):
             "peak": (peak_clock or peak_max) / 1e9,
             "unit": "Gpair/s",
             "frac": achieved / (peak_clock or peak_max),
-            "peak_basis": ("128 FP32 lanes x SMs x median SM clock under load / 12 FP32 "
-                           "instructions per pair" if peak_clock else
-                           "128 FP32 lanes x SMs x 2070 MHz / 12"),
+            "peak_basis": (f"128 FP32 lanes x SMs x median SM clock under load / {instr} FP32 "
+                           "instructions per counted pair" if peak_clock else
+                           f"128 FP32 lanes x SMs x 2070 MHz / {instr}")
+                          + (" (each pair evaluated once for both its records)"
+                             if instr == FP32_INSTR_PER_PAIR_ONCE else ""),
+            "step_kernels": kernels,
             "frac_at_max_clock": achieved / peak_max,
             "frac_of_measured_ffma": achieved / peak_probe,
             "measured_ffma_tflops": 2 * ffma_per_s / 1e12,
             "measured_packed_f32x2_fma_tflops": 2 * ffma2_per_s / 1e12,
-            "traffic": STEP_TRAFFIC_BYTES.get((args.workload, n, tuning[0], tuning[1],
-                                                tuning[2], bool(tuning[5]), tuning[4])),
+            "traffic": (STEP_TRAFFIC_BYTES.get((args.workload, n, tuning[0], tuning[1], tuning[2],
+                                                bool(tuning[5]), tuning[4]))
+                        if "k_step" in kernels else None),
             "traffic_unit": "B per launch (dram read + write, ncu)",
         },
         "clocks": clocks,
@@ -974,7 +1012,7 @@ def run_native(args):
                 "d2h_bytes_per_step": RECORD_BYTES * n, "wall_s_per_step": e2e_max,
                 "what": "md_set_particles + md_step(1) + md_get_particles from pinned host "
                         "arrays, wall clock"},
-        "gpu_launches": args.steps * launches_per_step,
+        "gpu_launches": args.steps * sum(kernels.values()),
         "cpu_baseline": cpu,
         "force_err_vs_fp64": force_err,
         "precision_study": precision,
