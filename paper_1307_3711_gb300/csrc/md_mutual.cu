@@ -462,17 +462,18 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
 // The push of every record: its partials in a fixed order, laser, kick, drift.
 // Runs after k_mut_pairs, whose ticket it resets; its last CTA advances the
 // step.  A CTA takes 32 records: warp w of W adds the work units and the earlier
-// blocks' rows w, w + W, ... in Kahan-compensated FP32, and the first warp adds
-// the W sums in FP64 and pushes with the laser field that the pair kernel left.
-// 99 us at 200k records (0.3 GB of partials) with W = 4, 12.5 at 19k with 8; one
-// thread per record with FP64 adds, which the narrow FP64 pipe bounds, took 240
-// and 32, the laser's sine in every CTA 136 and 14.
+// blocks' rows w, w + W, ... in Kahan-compensated FP32, and the first warp joins
+// the W sums and pushes with the laser field that the pair kernel left.  86 us at
+// 200k records (0.3 GB of partials) with W = 4, 10.9 at 19k with 8; one thread per
+// record with FP64 adds, which the narrow FP64 pipe bounds, took 240 and 32, the
+// laser's sine in every CTA 136 and 14, the W sums in FP64 99 and 12.2.
 constexpr int kPushRec = 32;
 
 template <int kPushWarps, bool DET, bool POT>
 __global__ void __launch_bounds__(32 * kPushWarps) k_mut_push(const MutArgs a) {
   constexpr int C = POT ? 4 : 3;
-  __shared__ double s_e[C][kPushWarps][kPushRec];
+  __shared__ float2 s_e[3][kPushWarps][kPushRec];  // the warps' sums (value x - y)
+  __shared__ double s_ph[POT ? kPushWarps : 1][kPushRec];
   __shared__ ClusterDev s_c;
   __shared__ float s_las[6];
   const long long step = __ldcg(a.s.step);
@@ -524,18 +525,25 @@ __global__ void __launch_bounds__(32 * kPushWarps) k_mut_push(const MutArgs a) {
       if constexpr (POT) ph += __ldcg(a.jphi + b.jbase + skipped + col);
     }
 #pragma unroll
-    for (int m = 0; m < 3; ++m) s_e[m][warp][lane] = static_cast<double>(s[m]) - c[m];
-    if constexpr (POT) s_e[3][warp][lane] = ph;
+    for (int m = 0; m < 3; ++m) s_e[m][warp][lane] = make_float2(s[m], c[m]);
+    if constexpr (POT) s_ph[warp][lane] = ph;
   }
   __syncthreads();
   if (warp == 0) {
     if (live) {
       double e[C];
 #pragma unroll
-      for (int m = 0; m < C; ++m) {
-        e[m] = 0.0;
+      for (int m = 0; m < 3; ++m) {
+        float2 v = s_e[m][0][lane];
 #pragma unroll
-        for (int w = 0; w < kPushWarps; ++w) e[m] += s_e[m][w][lane];
+        for (int w = 1; w < kPushWarps; ++w)
+          join_sums(v.x, v.y, s_e[m][w][lane].x, s_e[m][w][lane].y);
+        e[m] = static_cast<double>(v.x) - v.y;
+      }
+      if constexpr (POT) {
+        e[3] = 0.0;
+#pragma unroll
+        for (int w = 0; w < kPushWarps; ++w) e[3] += s_ph[w][lane];
       }
       const float4* __restrict__ cur = (step & 1) ? a.s.posq1 : a.s.posq0;
       float4* __restrict__ nxt = (step & 1) ? a.s.posq0 : a.s.posq1;
@@ -610,7 +618,8 @@ cudaError_t launch_mut_step(const MutArgs& a, int grid, bool det, bool pot, bool
   if (e != cudaSuccess) return e;
   const unsigned g = static_cast<unsigned>(a.n_blks) * static_cast<unsigned>(a.block / kPushRec);
   // eight warps while the CTAs are few (19k records: 12.5 us against 18 with
-  // four), four once they fill the SMs (a scan of 290k records: 81 against 125)
+  // four), four once they fill the SMs (a scan of 290k records: 81 against 125;
+  // both sides with the warps' sums in FP64, now 10.9 and 59)
   if (g >= 8u * static_cast<unsigned>(a.sms))
     launch_push_w<4>(a, g, det, pot, s);
   else
