@@ -755,7 +755,7 @@ void auto_off(md_ctx* c) {
   c->d_mut_jphi = nullptr;
 }
 
-// Rows of jpart at most: 16 GB (1.6M records in one cluster); a larger context
+// Rows of jpart at most: 16 GB (2.1M records in one cluster); a larger context
 // keeps the step kernel.
 constexpr long long kMutMaxRecs = (16LL << 30) / 12;
 // Records from which a cluster with minimum-image forces takes it.  Another
