@@ -9,6 +9,8 @@
 #include <string>
 #include <vector>
 
+#include <cuda.h>
+
 #include "md.h"
 #include "md_internal.h"
 
@@ -208,16 +210,39 @@ struct RawView {
 
 // Whether host memory is page-locked (registered or allocated by CUDA), so
 // that an asynchronous copy can use it directly.
-// device_view (may be nullptr): its address for kernels, nullptr if it has none.
-bool is_pinned(const void* p, void** device_view = nullptr) {
-  if (device_view) *device_view = nullptr;
+bool is_pinned(const void* p) {
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();  // clear the error of an unknown pointer
     return false;
   }
-  if (at.type != cudaMemoryTypeHost) return false;
-  if (device_view) *device_view = at.devicePointer;
+  return at.type == cudaMemoryTypeHost;
+}
+
+// Whether all `bytes` bytes of a host array lie in one page-locked block, and
+// in *view the address through which kernels reach it.  A copy checks its range;
+// a kernel's stores would run on into whatever follows the block.
+bool is_pinned(void* p, size_t bytes, uintptr_t* view) {
+  using GetAttribute = CUresult(CUDAAPI*)(void*, CUpointer_attribute, CUdeviceptr);
+  static const GetAttribute get = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault,
+                                         &found) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<GetAttribute>(f);
+  }();
+  CUdeviceptr at = 0, base = 0;
+  size_t size = 0;
+  if (!get || !is_pinned(p) ||
+      get(&at, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, reinterpret_cast<CUdeviceptr>(p)) ||
+      get(&base, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, at) ||
+      get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, at) || at < base || bytes > size ||
+      at - base > size - bytes)
+    return false;
+  *view = static_cast<uintptr_t>(at);
   return true;
 }
 
@@ -2297,29 +2322,30 @@ static md_status md_get_particles_body(md_ctx* c, int32_t cluster, md_particles*
     void* user;
     void* stage;
     void* dev;
-    size_t bytes;
+    size_t bytes, element;
     bool direct;
-    void* view;
+    uintptr_t view;
   };
-  Part parts[6] = {{out->x, h.x, d.x, sizeof(double) * 3 * n, false, nullptr},
-                   {out->u, h.u, d.u, sizeof(double) * 3 * n, false, nullptr},
-                   {out->z, h.z, d.z, sizeof(int) * n, false, nullptr},
-                   {out->mass, h.mass, d.mass, sizeof(double) * n, false, nullptr},
-                   {out->w, h.w, d.w, sizeof(double) * n, false, nullptr},
-                   {out->kind, h.kind, d.kind, static_cast<size_t>(n), false, nullptr}};
-  bool views = true;  // every wanted array is page-locked and visible to kernels
+  Part parts[6] = {{out->x, h.x, d.x, sizeof(double) * 3 * n, sizeof(double), false, 0},
+                   {out->u, h.u, d.u, sizeof(double) * 3 * n, sizeof(double), false, 0},
+                   {out->z, h.z, d.z, sizeof(int) * n, sizeof(int), false, 0},
+                   {out->mass, h.mass, d.mass, sizeof(double) * n, sizeof(double), false, 0},
+                   {out->w, h.w, d.w, sizeof(double) * n, sizeof(double), false, 0},
+                   {out->kind, h.kind, d.kind, static_cast<size_t>(n), 1, false, 0}};
+  // a few records: the kernel writes the caller's page-locked arrays itself (a
+  // copy per array costs more than it moves) if every element lies on a
+  // multiple of its size, which a copy does not need; otherwise through the
+  // device buffer, page-locked arrays copied directly, the others through the
+  // pinned staging buffer
+  bool straight = n <= kStraightRecords;
   for (Part& q : parts) {
     if (!q.user) continue;
-    q.direct = is_pinned(q.user, &q.view);
-    views = views && q.view;
+    q.direct = is_pinned(q.user, q.bytes, &q.view);
+    straight = straight && q.direct && q.view % q.element == 0;
   }
-  // a few records: the kernel writes the caller's page-locked arrays itself (a
-  // copy per array costs more than it moves); otherwise through the device
-  // buffer, page-locked arrays copied directly, the others through the pinned
-  // staging buffer
-  const bool straight = views && n <= kStraightRecords;
   auto to = [&](int k) -> void* {
-    return !parts[k].user ? nullptr : straight ? parts[k].view : parts[k].dev;
+    return !parts[k].user ? nullptr
+                          : straight ? reinterpret_cast<void*>(parts[k].view) : parts[k].dev;
   };
   a.hx = static_cast<double*>(to(0));
   a.hu = static_cast<double*>(to(1));
