@@ -376,8 +376,11 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
           }
         }
         __syncthreads();
-        // an expired wait: no other copy is in flight (one stage)
-        if (*reinterpret_cast<volatile int*>(&s_abort)) return;
+        // an expired wait: the one copy in flight is awaited once more (bounded)
+        if (*reinterpret_cast<volatile int*>(&s_abort)) {
+          if (tid == 0) mbar_wait(&sm.full[0], it & 1u);
+          return;
+        }
         if (tid == 0 && t + 1 < t_end) issue_tile<TILE, 1>(sm, it + 1, blk, left, t + 1);
         const u64 qq = f2_pack(qt, qt);
         const bool mutual = t * TILE >= kBlock;

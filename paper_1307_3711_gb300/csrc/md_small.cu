@@ -10,7 +10,11 @@
 // pushed by the CTA that summed them: one launch, no partial sums
 // in memory, no ticket.  The laser's FP64 envelope and sine run in two warps of
 // their own beside the sums, the targets' state is loaded before them, and the
-// step counter is advanced while they run.
+// step counter is advanced beside the push.
+//
+// A wait that runs out: the CTA pushes nothing, waits (bounded) for its copies
+// still in flight and leaves; the step does not advance, and the launches that
+// follow (of the same graph) find the error bit and push nothing.
 //
 // Measured (graph replay, us per step): 6.8 at 2000 records (53 with the step
 // kernel's default configuration; 8.1 with the slices' sums in FP64 and the last
@@ -36,7 +40,6 @@ struct SmallSmem {
   float2 sum[POT ? 4 : 3][TL * R];
   ClusterDev c;
   double amp, sn, cs;  // the laser at t_n
-  int abort;
 };
 
 // One target group: TL lanes x R targets, THREADS / TL slices of the sources.
@@ -57,7 +60,6 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
   if (tid == THREADS) {
     for (int s = 0; s < kStages; ++s) mbar_init(&S.st.full[s], 1);
     fence_mbar_init();
-    S.abort = 0;
   }
   const long long step = __ldcg(a.step);
   const float4* __restrict__ cur = ((step & 1) ? a.posq1 : a.posq0);
@@ -89,17 +91,19 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
     if (pushes) st = load_state(a, off + b.t0 + tid);
   }
   __syncthreads();  // the first copies are issued, the descriptor is in place
+  // the tiles of the group from t0 on, before their CTA leaves
+  auto drain = [&](int t0) {
+    if (tid == THREADS)
+      for (int t = t0; t < ntiles && t < t0 + kStages; ++t)
+        mbar_wait(&S.st.full[t % kStages], (t / kStages) & 1u);
+  };
+  // a wait of this thread ran out, or (the thread that asks) one of an earlier launch
+  bool late = false;
   if (tid >= THREADS) {
     const double t_n = S.c.t0 + static_cast<double>(step) * S.c.dt;
     if (tid == THREADS) {
-      // every thread of this CTA has read the step: the last CTA to get here
-      // advances it
-      const unsigned prev = atomicAdd(a.done, 1u);
-      if (prev == gridDim.x - 1) {
-        atomicExch(a.done, 0u);
-        *reinterpret_cast<volatile long long*>(a.step) = step + 1;
-      }
       S.amp = S.c.a0 * envelope(t_n, S.c.env, S.c.tau);
+      late = __ldcg(a.err) & kErrTimeout;
     } else if (tid == THREADS + 32) {
       sincos(t_n, &S.sn, &S.cs);
     }
@@ -112,7 +116,7 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
         const int s = t % kStages;
         if (!mbar_wait(&S.st.full[s], (t / kStages) & 1u)) {
           atomicOr(a.err, kErrTimeout);
-          S.abort = 1;
+          late = true;
           break;
         }
         const int rem = n_pad - t * kTile, cnt = rem < kTile ? rem : kTile;
@@ -149,8 +153,10 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
     }
     if (t0 + kStages < ntiles) {
       // every stage is read: refill (a cluster of more than kStages tiles)
-      __syncthreads();
-      if (S.abort) return;
+      if (__syncthreads_or(late)) {
+        drain(t0);
+        return;
+      }
       if (tid == THREADS)
         for (int t = t0 + kStages; t < ntiles && t < t0 + 2 * kStages; ++t)
           issue_tile<kTile, kStages>(S.st, static_cast<unsigned>(t), src, n_pad, t);
@@ -171,12 +177,26 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
       if constexpr (POT) put(3, r, acc.sp[r], acc.cp[r]);
     }
   }
-  __syncthreads();
-  if (S.abort) return;
+  if (__syncthreads_or(late)) {
+    drain((ntiles - 1) / kStages * kStages);
+    return;
+  }
+  if (tid >= THREADS) {
+    // every thread of this CTA has read the step, and its sums are complete: the
+    // last CTA to get here advances it (beside the join and the push of the others)
+    if (tid == THREADS) {
+      const unsigned prev = atomicAdd(a.done, 1u);
+      if (prev == gridDim.x - 1) {
+        atomicExch(a.done, 0u);
+        *reinterpret_cast<volatile long long*>(a.step) = step + 1;
+      }
+    }
+    return;
+  }
   // each value's warps: kJoin neighbouring lanes add some each, then each other's
   constexpr int kWarps = THREADS / 32, kJoin = THREADS / (4 * kTargets);
   static_assert(kJoin >= 1 && kJoin <= kWarps, "lanes per value");
-  if (tid < THREADS) {
+  {
     const int k = tid / kJoin, c = k / kTargets, t = k % kTargets;
     float2 v = make_float2(0.0f, 0.0f);
     if (k < C * kTargets) {
@@ -191,7 +211,7 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
                 __shfl_xor_sync(0xffffffffu, v.y, d));
     if (k < C * kTargets && tid % kJoin == 0) S.sum[c][t] = v;
   }
-  __syncthreads();
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");  // the summing threads
   if (pushes) {
     const long long i = off + b.t0 + tid;
     float las[6];
