@@ -2081,6 +2081,7 @@ static md_status run_fields(md_ctx* c, int ci, bool potential) {
   a.ns = cl.n_pad;
   a.tgt = cur + sb;
   a.nt = std::max(0LL, se - sb);
+  if (a.nt == 0) return MD_OK;  // an empty slice has no targets
   a.eps2 = cl.eps2;
   a.self_offset = sb;
   a.e = c->d_e;
@@ -2104,7 +2105,7 @@ static md_status run_fields(md_ctx* c, int ci, bool potential) {
   // same bits where no pair needs an image, a target slice and a cluster large
   // enough to be sliced the one that adds every slice's sources alike)
   if (!a.src_live && cl.boundary == MD_BOUNDARY_OPEN && !c->any_slice && a.ns <= 8192 &&
-      a.nt > 0 && md::field_uses_probe(a.nt, a.ns, nseg, c->sm_count)) {
+      md::field_uses_probe(a.nt, a.ns, nseg, c->sm_count)) {
     MD_CUDA(md::launch_field_direct(a, potential, c->sm_count, c->stream));
     return MD_OK;
   }
