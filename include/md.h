@@ -411,7 +411,8 @@ md_status md_get_step(md_ctx *ctx, int64_t *step);
  * Until then (and after md_autotune, if it was the fastest) a context without
  * ionizing clusters or target slices takes the step that evaluates each pair
  * of records once for both, where it has room for its partial sums (12 bytes
- * per 1024 or 1536 pairs, at most 16 GB); its sums have another order.
+ * per 1024 or 1536 pairs, 20 from the first md_step_diag on; at most 16 GB and
+ * half of the free device memory); its sums have another order.
  * md_get_tuning: the step kernel configuration in use, or the one that would
  * be without that step.
  * md_autotune: times every configuration over `steps` steps on the

@@ -145,7 +145,7 @@ struct md_ctx {
   int mut_shares = 0, mut_blks = 0, mut_grid = 0, mut_block = 0;
   float2* d_mut_ipart = nullptr;
   float* d_mut_jpart = nullptr;
-  double* d_mut_jphi = nullptr;   // allocated by the first diagnostic step
+  double* d_mut_jphi = nullptr;   // allocated by the first diagnostic step, if there is room
   float* d_mut_las = nullptr;
   long long mut_jrecs = 0;        // records of all rows of jpart
   // the step of a few thousand records (md_small.cu), while small_targets > 0
@@ -914,6 +914,15 @@ md_status auto_configure(md_ctx* c) {
   }
   const long long G = static_cast<long long>(first.size()) - 1;
   for (size_t i = 1; i < first.size(); ++i) first[i] += first[i - 1];
+  // Not more than half of the memory that is free (a query only where it counts):
+  // diagnosed steps, other contexts and the autotuner's copy of the state want some.
+  const size_t need = 20 * static_cast<size_t>(jrecs) +
+                      4 * sizeof(float2) * static_cast<size_t>(B) * units.size();
+  if (need > (64u << 20)) {
+    size_t free = 0, total = 0;
+    MD_CUDA(cudaMemGetInfo(&free, &total));
+    if (need > free / 2) return MD_OK;
+  }
   cudaError_t e = dev_alloc(&c->d_mut_jpart, 3 * static_cast<size_t>(jrecs));
   if (e == cudaSuccess) e = dev_alloc(&c->d_mut_ipart, 4 * static_cast<size_t>(B) * units.size());
   if (e == cudaSuccess) e = dev_alloc(&c->d_mut_units, units.size());
@@ -2222,14 +2231,21 @@ md_status md_diagnostics(md_ctx* c, int32_t cluster, md_diag* out) {
 // the field and records every record's diagnostics from its own kick, and an
 // O(N) reduction per cluster adds them in a fixed order.  Contexts with
 // ionization, detectors or minimum-image forces take the diagnostics call
-// and md_step(1) instead.
+// and md_step(1) instead, and so does the pair-once step where there is no room
+// for its partial potentials.
 static md_status md_step_diag_body(md_ctx* c, md_diag* out) {
   if (!c || !out) return fail(MD_ERR_ARG, "NULL argument");
   int ncfg = 0;
   const md::KernelConfig* cfgs = md::step_configs(&ncfg);
   const md::KernelConfig& k = cfgs[c->cfg];
   md_status st = MD_OK, worst = MD_OK;
-  if (c->any_ion || c->det_on || c->any_mi || !k.launch_step_pot) {
+  bool apart = c->any_ion || c->det_on || c->any_mi || !k.launch_step_pot;
+  if (!apart && c->mut_on && !c->d_mut_jphi &&
+      dev_alloc(&c->d_mut_jphi, static_cast<size_t>(c->mut_jrecs)) != cudaSuccess) {
+    cudaGetLastError();
+    apart = true;
+  }
+  if (apart) {
     for (int ci = 0; ci < c->n_clusters; ++ci) {
       st = md_diagnostics(c, ci, &out[ci]);
       if (st == MD_ERR_NONFINITE) worst = st;
@@ -2242,9 +2258,7 @@ static md_status md_step_diag_body(md_ctx* c, md_diag* out) {
   if (st != MD_OK) return st;
   const size_t nt = static_cast<size_t>(c->n_total);
   if (!c->d_diag_rec) MD_CUDA(dev_alloc(&c->d_diag_rec, 6 * nt));
-  if (c->mut_on) {
-    if (!c->d_mut_jphi) MD_CUDA(dev_alloc(&c->d_mut_jphi, static_cast<size_t>(c->mut_jrecs)));
-  } else if (!c->small_targets && c->nseg_used > 1 && c->part_phi_seg < c->nseg_used) {
+  if (!c->mut_on && !c->small_targets && c->nseg_used > 1 && c->part_phi_seg < c->nseg_used) {
     cudaFree(c->d_part_phi);
     c->d_part_phi = nullptr;
     MD_CUDA(dev_alloc(&c->d_part_phi, static_cast<size_t>(c->nseg_used) * nt));
