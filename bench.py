@@ -977,7 +977,9 @@ def run_native(args):
             "l2": f"flushed between timed steps ({L2_FLUSH_BYTES >> 20} MB write outside the "
                   "timed events)",
             "tuning": {"threads": tuning[0], "r": tuning[1], "tile": tuning[2],
-                       "source_split": (f"equal shares, {-tuning[4]} per resident CTA"
+                       "source_split": ("the step chosen for the context's size"
+                                        if tuning[4] == md.JSPLIT_AUTO else
+                                        f"equal shares, {-tuning[4]} per resident CTA"
                                         if tuning[4] < 0 else
                                         f"{tuning[4]} segments per i-block"),
                        "jsplit": tuning[4], "packed_f32x2": bool(tuning[5]),

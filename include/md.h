@@ -173,12 +173,18 @@ typedef struct {
                            equal shares they may.  md_get_tuning reports -k for equal shares,
                            else the largest segment count of any cluster; md_autotune
                            tries 0 for every configuration and -2, -4 for the two
-                           fastest. */
+                           fastest.
+                           MD_JSPLIT_AUTO: no piece of this kernel, but the step that
+                           suits the context's size (see md_set_tuning) */
     int32_t packed;     /* 1: pair arithmetic in packed f32x2 (two i-particles per
                            instruction, bit-identical results), 0: scalar FP32 */
     int32_t min_blocks; /* register budget: 64K / (threads x min_blocks); 0 = left to the
                            compiler.  On input to md_set_tuning, -1 matches any value */
 } md_tuning;
+
+/* md_tuning.jsplit of a context that takes its steps with the kernels chosen
+ * for its size. */
+enum { MD_JSPLIT_AUTO = 128 };
 
 /* ---- context life cycle -------------------------------------------------
  * md_init: creates a context holding n_clusters independent clusters (a
@@ -409,12 +415,17 @@ md_status md_get_step(md_ctx *ctx, int64_t *step);
  * configurations into list (may be NULL) and returns their number.
  * md_set_tuning: uses the given configuration of the step kernel from now on.
  * Until then (and after md_autotune, if it was the fastest) a context without
- * ionizing clusters or target slices takes the step that evaluates each pair
+ * ionizing clusters or target slices takes the step that suits its size: one
+ * launch for a few thousand records, or the step that evaluates each pair
  * of records once for both, where it has room for its partial sums (12 bytes
  * per 1024 or 1536 pairs, 20 from the first md_step_diag on; at most 16 GB and
  * half of the free device memory); its sums have another order.
- * md_get_tuning: the step kernel configuration in use, or the one that would
- * be without that step.
+ * With jsplit MD_JSPLIT_AUTO it goes back to that choice, and the configuration
+ * (with jsplit 0) serves where it is not taken.
+ * md_get_tuning: the step kernel configuration in use; while the context takes
+ * the step chosen for its size, the one that would be, with jsplit
+ * MD_JSPLIT_AUTO.  Setting what md_get_tuning returned, in this context or
+ * another, takes the same kind of step.
  * md_autotune: times every configuration over `steps` steps on the
  * context's own state (restored afterwards), with jsplit 0 and, for the two
  * fastest, jsplit -2 and -4 (no ionizing cluster), then the step that takes

@@ -2427,14 +2427,16 @@ static md_status md_set_tuning_body(md_ctx* c, const md_tuning* t) {
         (t->min_blocks < 0 || cfgs[i].min_blocks == t->min_blocks)) {
       if (t->ctas_per_sm < 0) return fail(MD_ERR_ARG, "ctas_per_sm < 0");
       MD_CUDA(cudaStreamSynchronize(c->stream));
-      const bool was = c->forced;
-      c->forced = true;
-      const md_status st = configure(c, i, t->ctas_per_sm, t->jsplit);
-      if (st == MD_OK)
-        auto_off(c);
-      else
+      const bool was = c->forced, automatic = t->jsplit == MD_JSPLIT_AUTO;
+      c->forced = !automatic;
+      const md_status st = configure(c, i, t->ctas_per_sm, automatic ? 0 : t->jsplit);
+      if (st != MD_OK) {
         c->forced = was;
-      return st;
+        return st;
+      }
+      if (automatic) return auto_configure(c);
+      auto_off(c);
+      return MD_OK;
     }
   }
   return fail(MD_ERR_ARG, "no compiled configuration threads=%d r=%d tile=%d packed=%d",
@@ -2453,7 +2455,8 @@ static md_status md_get_tuning_body(md_ctx* c, md_tuning* t) {
   t->r = cfgs[c->cfg].r;
   t->tile = cfgs[c->cfg].tile;
   t->ctas_per_sm = c->ctas_per_sm;
-  t->jsplit = c->jsplit < 0 ? c->jsplit : c->nseg_used;
+  t->jsplit = c->mut_on || c->small_targets ? static_cast<int32_t>(MD_JSPLIT_AUTO)
+                                            : c->jsplit < 0 ? c->jsplit : c->nseg_used;
   t->packed = cfgs[c->cfg].packed;
   t->min_blocks = cfgs[c->cfg].min_blocks;
   return MD_OK;

@@ -25,6 +25,7 @@ MD_OK, MD_ERR_ARG, MD_ERR_OOM, MD_ERR_CUDA, MD_ERR_TIMEOUT, MD_ERR_NONFINITE, MD
 ENV_GAUSS, ENV_SIN2, ENV_LITERAL_EQ3, ENV_FLAT = 0, 1, 2, 3
 BOUNDARY_OPEN, BOUNDARY_PERIODIC, BOUNDARY_MIXED = 0, 1, 2
 KIND_ION, KIND_ELECTRON, KIND_INACTIVE = 0, 1, 2
+JSPLIT_AUTO = 128  # jsplit of a context that takes the step chosen for its size
 
 
 class MDError(RuntimeError):
@@ -468,7 +469,9 @@ class Context:
     def set_tuning(self, threads, r, tile, ctas_per_sm=0, jsplit=0, packed=0, min_blocks=-1):
         """md_set_tuning: one of tuning_list()'s configurations; jsplit > 0 that
         many source segments per i-block, 0 a count chosen for balance, -k equal
-        shares, k per resident CTA (md_tuning in md.h)."""
+        shares, k per resident CTA; JSPLIT_AUTO the step chosen for the context's
+        size (md_tuning in md.h).  ``set_tuning(*other.tuning())`` takes over
+        another context's choice."""
         t = Tuning(threads, r, tile, ctas_per_sm, jsplit, packed, min_blocks)
         _check(_lib.md_set_tuning(self._h, C.byref(t)))
 
