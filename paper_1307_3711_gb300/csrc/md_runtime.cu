@@ -793,14 +793,52 @@ constexpr long long kMutMinImageRecords = 11000;
 constexpr long long kMutBigRecords = 40000;
 constexpr long long kMutMinTiles = 2;
 
+// What a step takes in us with the step kernel as a context starts with it (128
+// x 4 targets), with the small step and with each pair once.  Each is a fixed
+// part, a part per i-block (or CTA) and one per pair, fitted to the timings below.
+// Where clusters hold a few hundred records the blocks are mostly empty (1024
+// targets of the pair-once step) or mostly launch and push (16 or 32 targets of
+// the small step), and the step kernel's 512 targets are the better ones.
+//   clusters x records   step kernel   small    each pair once
+//   700 x 300                63.3       131
+//   5000 x 100              143         313
+//   100 x 800                71.7        63.1
+//   20000 x 16              207         183
+//   1 x 8000                 79.5        41.6
+//   1000 x 300               85.3                  179
+//   10000 x 100             287                    866
+//   250 x 600                95.3                   87.4
+//   100 x 1500              119                    120
+//   64 x 2500               219                    176
+//   1680 x 891..1518       1197                   1116
+//   1 x 15000               149                     86
+double step_kernel_us(const md_ctx* c) {
+  double t = 0.0, longest = 0.0;
+  for (const md::ClusterDev& cl : c->cl) {
+    t += (cl.n_pad + 511) / 512 * (0.008 + 0.000225 * cl.n_pad);
+    longest = std::max(longest, static_cast<double>(cl.n_pad));
+  }
+  return 0.87 * (10.0 + 0.05 * std::min(longest, 700.0) + t);
+}
+
+double small_step_us(const md_ctx* c, int per) {
+  double t = 0.0;
+  for (const md::ClusterDev& cl : c->cl)
+    t += (cl.n_pad + per - 1) / per * (0.008 + 4.2e-7 * per * cl.n_pad);
+  return 4.0 + t;
+}
+
+// (lanes: FP32 lane operations, 11 and 14 per pair of a one-sided and of a mutual tile)
+double mut_step_us(double blocks, double lanes) { return 21.0 + 0.06 * blocks + lanes / 2.8e7; }
+
 // Pairs (records squared, summed over the clusters) up to which the small step
 // is taken: 23.8 us per step at 5000 records against 31 with each pair once,
 // 41.5 against 41.2 at 8000, 66 against 55 at 10000.
 constexpr double kSmallMaxPairs = 9.0e3 * 9.0e3;
 
-// The small step, if the context is that small: 16 or 32 targets per CTA,
-// whichever leaves the busiest SM fewer targets (equal: 32, whose CTAs stage
-// the sources half as often).
+// The small step, if the context is that small and its clusters are not many and
+// tiny: 16 or 32 targets per CTA, whichever leaves the busiest SM fewer targets
+// (equal: 32, whose CTAs stage the sources half as often).
 md_status small_configure(md_ctx* c) {
   double pairs = 0.0;
   for (const md::ClusterDev& cl : c->cl) pairs += static_cast<double>(cl.n_pad) * cl.n_pad;
@@ -813,6 +851,7 @@ md_status small_configure(md_ctx* c) {
   }
   const int pick = load[1] <= load[0] ? 1 : 0;
   const int per = pick ? 32 : 16;
+  if (small_step_us(c, per) > step_kernel_us(c)) return MD_OK;
   if (c->n_clusters > 1) {
     std::vector<md::SmallBlk> blks;
     for (int ci = 0; ci < c->n_clusters; ++ci)
@@ -830,8 +869,8 @@ md_status small_configure(md_ctx* c) {
 
 // Sets up the step that suits the context's size, if it can take it (no
 // ionizing cluster, no target slice): the small step, or each pair evaluated
-// once if there is room for the partial sums; otherwise the configured step
-// kernel stays.
+// once if there is room for the partial sums; the configured step kernel stays
+// where neither is faster.
 md_status auto_configure(md_ctx* c) {
   MD_CUDA(cudaStreamSynchronize(c->stream));
   auto_off(c);
@@ -851,6 +890,7 @@ md_status auto_configure(md_ctx* c) {
   const long long slots = static_cast<long long>(bps) * c->sm_count;
   std::vector<md::MutBlk> blks;
   long long jrecs = 0, weight = 0, tiles = 0;
+  double lanes = 0.0;
   for (int ci = 0; ci < c->n_clusters; ++ci) {
     const long long n = c->cl[ci].n_pad, nb = (n + B - 1) / B;
     const long long base = jrecs;
@@ -860,8 +900,11 @@ md_status auto_configure(md_ctx* c) {
       jrecs += std::max(0LL, n - (b + 1) * B);
       weight += md::kMutWeightOwn * own + md::kMutWeightPair * (nt - own);
       tiles += nt;
+      const double left = static_cast<double>(n - b * B);
+      lanes += B * (14.0 * left - 3.0 * std::min<double>(left, B));
     }
   }
+  if (mut_step_us(static_cast<double>(blks.size()), lanes) > step_kernel_us(c)) return MD_OK;
   if (jrecs > kMutMaxRecs || blks.size() > (1u << 27)) return MD_OK;
   // Shares in rounds of one per resident CTA: a round takes three eighths of
   // the work that is left.  The CTAs of an SM do not advance alike (one share
