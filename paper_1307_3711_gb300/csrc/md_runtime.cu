@@ -2076,8 +2076,12 @@ static md_status md_set_slice_body(md_ctx* c, int32_t cluster, int64_t i_begin, 
   if (c->any_ion || c->det_on)
     return fail(MD_ERR_STATE, "target slices need a context without ionization or detectors");
   MD_CUDA(cudaStreamSynchronize(c->stream));
+  const long long end = i_end == cl.n ? cl.n_pad : i_end;
+  // the slice that it has: the plan of its steps stands (a new one costs 0.2 to
+  // 1.2 ms with the partial sums of the pair-once step)
+  if (c->slice_b[cluster] == i_begin && c->slice_e[cluster] == end) return MD_OK;
   c->slice_b[cluster] = i_begin;
-  c->slice_e[cluster] = i_end == cl.n ? cl.n_pad : i_end;
+  c->slice_e[cluster] = end;
   bool any = false;
   for (int ci = 0; ci < c->n_clusters; ++ci)
     any = any || c->slice_b[ci] > 0 || c->slice_e[ci] < c->cl[ci].n_pad;
