@@ -77,6 +77,9 @@ cudaError_t launch_generate(const GenerateArgs& g, cudaStream_t s);
 // Count of the records [off, off + n) that are not INACTIVE, into *out.
 cudaError_t launch_count_active(const unsigned char* kind, long long off, long long n,
                                 unsigned long long* out, cudaStream_t s);
+// Number of the runs of kMutTile among n j-stream records that hold a charge.
+cudaError_t launch_count_charged(const float4* posq, long long n, unsigned long long* out,
+                                 cudaStream_t s);
 
 // Launches one CTA whose mbarrier wait can never complete (bounded by budget).
 cudaError_t launch_wait_selftest(long long budget, int* err, cudaStream_t s);

@@ -441,6 +441,23 @@ cudaError_t launch_count_active(const unsigned char* kind, long long off, long l
   return cudaGetLastError();
 }
 
+// Runs of kMutTile j-stream records that hold a charge, added to *out.
+__global__ void __launch_bounds__(kMutTile) k_count_charged(const float4* posq, long long n,
+                                                            unsigned long long* out) {
+  const long long k = static_cast<long long>(blockIdx.x) * kMutTile + threadIdx.x;
+  const int any = __syncthreads_or(k < n && posq[k].w != 0.0f);
+  if (threadIdx.x == 0 && any) atomicAdd(out, 1ull);
+}
+
+cudaError_t launch_count_charged(const float4* posq, long long n, unsigned long long* out,
+                                 cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), s);
+  if (e != cudaSuccess || n <= 0) return e;
+  k_count_charged<<<static_cast<unsigned>((n + kMutTile - 1) / kMutTile), kMutTile, 0, s>>>(posq, n,
+                                                                                           out);
+  return cudaGetLastError();
+}
+
 // Records of a generated cluster (Sec. II: atoms at random inside the sphere
 // of radius R0; Eq. 1: macro weight w).  Record k is an ion (k < n_ions), an
 // electron (k < n_ions + n_electrons) or an inactive slot.

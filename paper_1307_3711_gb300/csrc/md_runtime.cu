@@ -905,7 +905,20 @@ md_status auto_configure(md_ctx* c) {
     }
   }
   if (mut_step_us(static_cast<double>(blks.size()), lanes) > step_kernel_us(c)) return MD_OK;
-  if (jrecs > kMutMaxRecs || blks.size() > (1u << 27)) return MD_OK;
+  if (jrecs > kMutMaxRecs || blks.size() > (1u << 25)) return MD_OK;
+  // A large context of mostly uncharged records (unused slots): its few charged
+  // blocks fall into few large shares.  Below a third of charged tiles the step
+  // kernel is no slower (200k records, the rest unused slots behind the charged
+  // ones, ms per step, step kernel / pair-once: 40 % charged 6.85 / 6.71, 30 % 5.40 /
+  // 5.57, 20 % 3.95 / 4.18, 10 % 2.59 / 4.24); up to 35000 records pair-once is
+  // the faster one down to 2 % (0.133 / 0.099).
+  if (c->max_n >= kMutBigRecords) {
+    MD_CUDA(md::launch_count_charged(c->d_posq[0], c->n_total, c->d_word, c->stream));
+    MD_CUDA(cudaMemcpyAsync(c->h_word, c->d_word, sizeof(unsigned long long),
+                            cudaMemcpyDeviceToHost, c->stream));
+    MD_CUDA(cudaStreamSynchronize(c->stream));
+    if (3 * static_cast<long long>(*c->h_word) < c->n_total / T) return MD_OK;
+  }
   // Shares in rounds of one per resident CTA: a round takes three eighths of
   // the work that is left.  The CTAs of an SM do not advance alike (one share
   // each, all equal: 10.8 ms per step at 200k records; eight rounds of equal
