@@ -245,10 +245,11 @@ __device__ __forceinline__ void forward_sel(const MlpWeights& w, uint32_t x0, ui
   ysel[1] = p1 + w.b3[z1];
 }
 
-// One warp, 32 samples, lane l holding sample l's inputs: the output of its
+// One warp, 16 H samples, lane l holding sample l's inputs: the output of its
 // charge state z (clamped to the network's).  The features are formed once per
-// sample and reach the two 16-row tiles' fragments by shuffles.
-__device__ __forceinline__ float forward_32(const MlpWeights& w, const IonDev& io, bool have,
+// sample and reach the H 16-row tiles' fragments by shuffles.
+template <int H>
+__device__ __forceinline__ float forward_tiles(const MlpWeights& w, const IonDev& io, bool have,
                                             double emag, int z, double ne, double te) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int zc = z < 0 ? 0 : (z < kNO ? z : kNO - 1);
@@ -257,7 +258,7 @@ __device__ __forceinline__ float forward_32(const MlpWeights& w, const IonDev& i
   const uint32_t f01 = pack_bf16(x[0], x[1]), f23 = pack_bf16(x[2], x[3]);
   float y = 0.0f;
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < H; ++h) {
     uint32_t xr[2];
     int zr[2];
 #pragma unroll
@@ -306,6 +307,7 @@ __global__ void __launch_bounds__(32 * kWarps) k_mlp_forward(const float* __rest
 
 // Ionization pass, rate_model 2: for every ion inside the training domain
 // the surrogate rate nu = 10^(15 y_z - 15); ions outside keep use_plain = 1.
+template <int H>
 __global__ void __launch_bounds__(32 * kWarps) k_ion_mlp_rates(const IonArgs a) {
   __shared__ MlpWeights w;
   const long long step = __ldcg(a.step);
@@ -314,15 +316,16 @@ __global__ void __launch_bounds__(32 * kWarps) k_ion_mlp_rates(const IonArgs a) 
   load_weights<32 * kWarps>(a.mlp, w);
   __syncthreads();
   const long long n = a.ion.n_ions;
-  const long long tiles = (n + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  const long long tiles = (n + 16 * H - 1) / (16 * H);
   for (long long tile = static_cast<long long>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
        tile < tiles; tile += static_cast<long long>(gridDim.x) * kWarps) {
-    const long long k = tile * 32 + (threadIdx.x & 31);
-    const bool have = k < n;
+    const long long k = tile * 16 * H + lane;
+    const bool have = lane < 16 * H && k < n;
     const double* o = a.out + 4 * k;
     const double e = have ? o[0] : 0.0, ne = have ? o[1] : 0.0, te = have ? o[2] : 0.0;
     const int z = have ? a.zq[a.c.off + k] : -1;
-    const float y = forward_32(w, a.ion, have, e, z, ne, te);
+    const float y = forward_tiles<H>(w, a.ion, have, e, z, ne, te);
     if (!have || z < 0 || z >= a.ion.zmax) continue;
     const bool inside = e >= a.ion.dom[0] && e <= a.ion.dom[1] &&
                         (ne == 0.0 || (ne >= a.ion.dom[2] && ne <= a.ion.dom[3])) &&
@@ -630,7 +633,9 @@ __global__ void __launch_bounds__(32 * kAdamWarps)
 // Bound by the special-function unit (two per hidden unit); a CTA takes several
 // tiles, so that the weights' conversion is not paid per 64 ions.  200000 ions:
 // 68 us with a CTA per 64 ions, features formed by all four lanes of a quad and
-// eight-way bank conflicts on the weights, 37 us now.
+// eight-way bank conflicts on the weights, 37 us now.  A warp takes two 16-row
+// tiles, one (H = 1) while that gives an SM two CTAs at most (rates_per_warp).
+template <int H>
 __global__ void __launch_bounds__(32 * kWarps) k_rates_mlp(IonDev io, const float* __restrict__ p,
                                                            const double* emag, const int* zs,
                                                            const double* ne, const double* te,
@@ -638,15 +643,16 @@ __global__ void __launch_bounds__(32 * kWarps) k_rates_mlp(IonDev io, const floa
   __shared__ MlpWeights w;
   load_weights<32 * kWarps>(p, w);
   __syncthreads();
-  const long long tiles = (n + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  const long long tiles = (n + 16 * H - 1) / (16 * H);
   for (long long tile = static_cast<long long>(blockIdx.x) * kWarps + (threadIdx.x >> 5);
        tile < tiles; tile += static_cast<long long>(gridDim.x) * kWarps) {
-    const long long k = tile * 32 + (threadIdx.x & 31);
-    const bool have = k < n;
+    const long long k = tile * 16 * H + lane;
+    const bool have = lane < 16 * H && k < n;
     const double e = have ? emag[k] : 0.0, d = have ? ne[k] : 0.0, tt = have ? te[k] : 0.0;
     const int z = have ? zs[k] : 0;
     // (out-of-range charges get a valid row and no surrogate rate)
-    const float y = forward_32(w, io, have, e, z, d, tt);
+    const float y = forward_tiles<H>(w, io, have, e, z, d, tt);
     if (!have) continue;
     const bool inside = z >= 0 && z < io.zmax && e >= io.dom[0] && e <= io.dom[1] &&
                         (d == 0.0 || (d >= io.dom[2] && d <= io.dom[3] && tt >= io.dom[4] &&
@@ -689,6 +695,11 @@ unsigned infer_ctas(long long n, int tile) {
   const long long want = ((n + tile - 1) / tile + kWarps - 1) / kWarps;
   return static_cast<unsigned>(std::max<long long>(1, std::min<long long>(want, 2 * train_grid())));
 }
+
+// Ions per warp of the surrogate's rates: the two tiles of a warp run one after
+// the other, so few ions take one.  (us per call with one and two tiles: 1000 ions
+// 14.4 and 18.5, 9700 14.4 and 18.5; the same bits.)
+int rates_per_warp(long long n) { return n <= 16LL * kWarps * train_grid() ? 16 : 32; }
 
 cudaError_t train_smem_attr() {
   static bool done = false;
@@ -749,7 +760,12 @@ md_status check_train_config(const md_mlp_train_config* c) {
 
 cudaError_t launch_ion_mlp(const IonArgs& a, cudaStream_t s) {
   if (!a.mlp) return cudaErrorInvalidValue;
-  k_ion_mlp_rates<<<infer_ctas(a.ion.n_ions, 32), 32 * kWarps, 0, s>>>(a);
+  const int per = rates_per_warp(a.ion.n_ions);
+  const unsigned grid = infer_ctas(a.ion.n_ions, per);
+  if (per == 16)
+    k_ion_mlp_rates<1><<<grid, 32 * kWarps, 0, s>>>(a);
+  else
+    k_ion_mlp_rates<2><<<grid, 32 * kWarps, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -850,7 +866,12 @@ static md_status md_ion_rates_device_body(const md_mlp_train_config* cfg, int32_
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const md::IonDev io = md::domain_io(*cfg);
   if (model == 2) {
-    md::k_rates_mlp<<<md::infer_ctas(n, 32), 32 * md::kWarps, 0, s>>>(io, params, emag, z, ne, te, n, nu);
+    const int per = md::rates_per_warp(n);
+    const unsigned grid = md::infer_ctas(n, per);
+    if (per == 16)
+      md::k_rates_mlp<1><<<grid, 32 * md::kWarps, 0, s>>>(io, params, emag, z, ne, te, n, nu);
+    else
+      md::k_rates_mlp<2><<<grid, 32 * md::kWarps, 0, s>>>(io, params, emag, z, ne, te, n, nu);
     MLP_CUDA(cudaGetLastError());
   }
   md::k_rates_plain<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(io, emag, z, ne, te, n,
