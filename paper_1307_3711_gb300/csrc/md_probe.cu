@@ -24,7 +24,6 @@
 // reads a source from shared memory per pair, so where the field kernel's
 // blocks fill the SMs it stays faster (field_uses_probe).
 #include <algorithm>
-#include <cmath>
 #include <utility>
 
 #include <cooperative_groups.h>
@@ -324,10 +323,31 @@ cudaError_t launch_field_direct(const FieldArgs& a, bool potential, int sms, cud
   const long long want = 5LL * sms / 3;
   auto ctas = [&](long long tl) { return (a.nt + tl - 1) / tl * cluster; };
   // two targets per thread halve the loads per pair once there is work for it
-  // (30000 x 30000: 440 us with one, 421 with two; 10000 x 150k: 750 and 711),
-  // and enough targets need fewer CTAs per cluster (30000 x 30000: 421, eight: 450)
-  if (a.nt >= 8192 && a.ns >= 8192)
-    return launch_p<32, 2>(a, potential, a.nt >= 16384 ? std::min(cluster, 4) : cluster, s);
+  // (30000 x 30000: 440 us with one, 421 with two; 10000 x 150k: 750 and 711), with
+  // the cluster size that loads the busiest SM least: it holds L of the CTAs, each
+  // 1.6 us and 4.3 ns per source of its part, the fewer the less they hide of each
+  // other's waits (us with clusters of one, two, four and eight: 8192 x 30000 133,
+  // 134, 138, 140; 10000 x 30000 257, 196, 166, 158; 14000 x 17000 150, 116, 119, 140;
+  // 20000 x 80000 998, 835, 758, 771; 30000 x 89000 1289 with two, 1207 with four;
+  // 28000 x 16000 209, 210, 219, 247; with the potential 8192 x 200k 1012, 955, 964, 936)
+  if (a.nt >= 8192 && a.ns >= 8192) {
+    const long long groups = (a.nt + 63) / 64;
+    int best = 1;
+    double least = 0.0;
+    for (int c = 1; c <= cluster; c *= 2) {
+      // (clusters of four leave four SMs empty, of eight a dozen, whose CTAs are
+      // many and even out)
+      const long long on = c == 4 ? sms - 4 : sms;
+      const double L = c == 8 ? 8.0 * groups / (sms - 12) + 0.4
+                              : static_cast<double>((groups * c + on - 1) / on);
+      const double t = (L + 0.08) * (1.6 + 0.0043 * static_cast<double>(a.ns) / c);
+      if (c == 1 || t < least) {
+        least = t;
+        best = c;
+      }
+    }
+    return launch_p<32, 2>(a, potential, best, s);
+  }
   // (many targets and few sources: no more CTAs than that; 30000 x 4001: 105 us
   // with clusters of four, 74 without)
   while (cluster > 1 && ctas(32) >= 4 * want) cluster /= 2;
@@ -338,17 +358,25 @@ cudaError_t launch_field_direct(const FieldArgs& a, bool potential, int sms, cud
 }
 
 // Whether launch_field_direct is the faster of the two for nt targets and ns
-// sources in nseg segments of the field kernel.  Estimates in us from the
-// timings above: this kernel 7 + 0.53 per million pairs; the field kernel 12 +
-// (8 + 49 k) ns per source of a segment, k = 1024-target CTAs per SM (three
-// run at once).
+// sources in nseg segments of the field kernel; the same with and without the
+// potential, so that the field has the same bits.  Estimates in us from the
+// timings above: this kernel 7 + 0.53 per million pairs, with few sources per
+// target 7 + 0.25 ns per target + 0.4 per million pairs (the clusters' start and
+// join); k_few 4.5 + 35 ns per source or 8 + 16.3 for each of the busiest SM's CTAs;
+// the field kernel 10.5 + (3.5 + 56.2 k) ns per source of a segment, k = 1024-target
+// CTAs per SM (three run at once).  Either side of the lines, us, field kernel and this
+// one: 100000 x 520 41 and 49, x 1300 88 and 84, 200000 x 800 103 and 117, 50000 x 600
+// 45 and 34; field kernel and k_few 300000 x 510 68 and 74, 527000 x 307 81 and 77.
 bool field_uses_probe(long long nt, long long ns, long long nseg, int sms) {
-  const double pairs = static_cast<double>(nt) * static_cast<double>(ns);
-  const double k = static_cast<double>((nt + 1023) / 1024 * nseg) / sms;
-  const double at_once = k < 3.0 ? std::ceil(k) : 3.0, rounds = k < 3.0 ? 1.0 : k / 3.0;
-  const double split = 12.0 + static_cast<double>(ns) / static_cast<double>(nseg) *
-                                  (0.008 + 0.049 * at_once) * rounds;
-  return few_sources(nt, ns) || 7.0 + 5.3e-7 * pairs < split;
+  const double t = static_cast<double>(nt), n = static_cast<double>(ns), pairs = t * n;
+  const long long k = ((nt + 1023) / 1024 * nseg + sms - 1) / sms;
+  const double each = 0.172 * (k / 3) + (k % 3 ? 0.0035 + 0.0562 * (k % 3) : 0.0);
+  const double split = 10.5 + each * n / static_cast<double>(nseg);
+  if (few_sources(nt, ns)) {
+    const double L = static_cast<double>(((nt + 255) / 256 + sms - 1) / sms);
+    return 4.5 + std::max(0.035, 0.008 + 0.0163 * L) * n < split;
+  }
+  return 7.0 + std::max(5.3e-7 * pairs, 2.5e-4 * t + 4.0e-7 * pairs) < split;
 }
 
 }  // namespace md
