@@ -139,6 +139,7 @@ struct md_ctx {
   // partial sums, while `mut_on`
   bool forced = false;  // md_set_tuning or md_autotune chose: no automatic choice
   bool mut_on = false;
+  unsigned char* d_mut = nullptr;  // one block for all but the potentials
   md::MutUnit* d_mut_units = nullptr;
   int* d_mut_first = nullptr;
   md::MutBlk* d_mut_blks = nullptr;
@@ -764,13 +765,9 @@ void auto_off(md_ctx* c) {
   c->small_targets = 0;
   cudaFree(c->d_small_blks);
   c->d_small_blks = nullptr;
-  cudaFree(c->d_mut_units);
-  cudaFree(c->d_mut_first);
-  cudaFree(c->d_mut_blks);
-  cudaFree(c->d_mut_ipart);
-  cudaFree(c->d_mut_jpart);
+  cudaFree(c->d_mut);
   cudaFree(c->d_mut_jphi);
-  cudaFree(c->d_mut_las);
+  c->d_mut = nullptr;
   c->d_mut_las = nullptr;
   c->d_mut_units = nullptr;
   c->d_mut_first = nullptr;
@@ -970,32 +967,44 @@ md_status auto_configure(md_ctx* c) {
   }
   const long long G = static_cast<long long>(first.size()) - 1;
   for (size_t i = 1; i < first.size(); ++i) first[i] += first[i - 1];
+  // one block (an allocation costs 20 to 30 us, and another when it is given
+  // back): the lists, which are copied as one, then the partial sums
+  size_t bytes = 0;
+  auto place = [&](size_t size) {
+    const size_t at = bytes;
+    bytes += (size + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_units = place(units.size() * sizeof(md::MutUnit));
+  const size_t o_first = place(first.size() * sizeof(int));
+  const size_t o_blks = place(blks.size() * sizeof(md::MutBlk));
+  std::vector<unsigned char> lists(bytes);
+  std::memcpy(&lists[o_units], units.data(), units.size() * sizeof(md::MutUnit));
+  std::memcpy(&lists[o_first], first.data(), first.size() * sizeof(int));
+  std::memcpy(&lists[o_blks], blks.data(), blks.size() * sizeof(md::MutBlk));
+  const size_t o_las = place(6 * sizeof(float) * static_cast<size_t>(c->n_clusters));
+  const size_t o_jpart = place(3 * sizeof(float) * static_cast<size_t>(jrecs));
+  const size_t o_ipart = place(4 * sizeof(float2) * static_cast<size_t>(B) * units.size());
   // Not more than half of the memory that is free (a query only where it counts):
   // diagnosed steps, other contexts and the autotuner's copy of the state want some.
-  const size_t need = 20 * static_cast<size_t>(jrecs) +
-                      4 * sizeof(float2) * static_cast<size_t>(B) * units.size();
+  const size_t need = bytes + sizeof(double) * static_cast<size_t>(jrecs);
   if (need > (64u << 20)) {
     size_t free = 0, total = 0;
     MD_CUDA(cudaMemGetInfo(&free, &total));
     if (need > free / 2) return MD_OK;
   }
-  cudaError_t e = dev_alloc(&c->d_mut_jpart, 3 * static_cast<size_t>(jrecs));
-  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_ipart, 4 * static_cast<size_t>(B) * units.size());
-  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_units, units.size());
-  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_first, first.size());
-  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_blks, blks.size());
-  if (e == cudaSuccess) e = dev_alloc(&c->d_mut_las, 6 * static_cast<size_t>(c->n_clusters));
-  if (e != cudaSuccess) {  // no room: the step kernel needs none of this
+  if (dev_alloc(&c->d_mut, bytes) != cudaSuccess) {  // no room: the step kernel needs none of this
     cudaGetLastError();
-    auto_off(c);
     return MD_OK;
   }
-  MD_CUDA(cudaMemcpyAsync(c->d_mut_units, units.data(), units.size() * sizeof(md::MutUnit),
-                          cudaMemcpyHostToDevice, c->stream));
-  MD_CUDA(cudaMemcpyAsync(c->d_mut_first, first.data(), first.size() * sizeof(int),
-                          cudaMemcpyHostToDevice, c->stream));
-  MD_CUDA(cudaMemcpyAsync(c->d_mut_blks, blks.data(), blks.size() * sizeof(md::MutBlk),
-                          cudaMemcpyHostToDevice, c->stream));
+  c->d_mut_units = reinterpret_cast<md::MutUnit*>(c->d_mut + o_units);
+  c->d_mut_first = reinterpret_cast<int*>(c->d_mut + o_first);
+  c->d_mut_blks = reinterpret_cast<md::MutBlk*>(c->d_mut + o_blks);
+  c->d_mut_las = reinterpret_cast<float*>(c->d_mut + o_las);
+  c->d_mut_jpart = reinterpret_cast<float*>(c->d_mut + o_jpart);
+  c->d_mut_ipart = reinterpret_cast<float2*>(c->d_mut + o_ipart);
+  MD_CUDA(cudaMemcpyAsync(c->d_mut, lists.data(), lists.size(), cudaMemcpyHostToDevice,
+                          c->stream));
   MD_CUDA(cudaStreamSynchronize(c->stream));
   c->mut_shares = static_cast<int>(G);
   c->mut_blks = static_cast<int>(blks.size());
