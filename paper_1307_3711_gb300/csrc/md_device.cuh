@@ -1154,6 +1154,7 @@ __device__ __forceinline__ void push_loaded(const StepArgs& a, const ClusterDev&
                                             const RecState& st, double ex, double ey, double ez,
                                             const float* las, double t_next, const float4* cur,
                                             float4* nxt, double phi = 0.0) {
+  if (!MD_IN_RANGE(a.err, i, c.off, c.off + c.n_pad)) return;
   double X = st.X, Y = st.Y, Z = st.Z;
   double Ux = st.Ux, Uy = st.Uy, Uz = st.Uz;
   const float h = 0.5f * static_cast<float>(c.dt) * st.qm;

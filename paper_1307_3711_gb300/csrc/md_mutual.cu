@@ -292,6 +292,23 @@ __global__ void __launch_bounds__(kMutThreads) k_mut_pairs(const MutArgs a) {
         s_c = a.s.cl[s_un.cluster];
       }
       __syncthreads();
+      // (checked build; the whole CTA decides alike) the unit, and its tiles in the cluster
+      if (!MD_IN_RANGE(a.s.err, u, 0, a.n_units) ||
+          !MD_IN_RANGE(a.s.err, s_un.cluster, 0, a.n_clusters) ||
+          !MD_IN_RANGE(a.s.err, static_cast<long long>(s_un.block) * kBlock, 0, s_c.n_pad) ||
+          !MD_IN_RANGE(a.s.err, s_un.t0, 0, s_un.t0 + s_un.nt) ||
+          !MD_IN_RANGE(a.s.err,
+                       static_cast<long long>(s_un.block) * kBlock +
+                           static_cast<long long>(s_un.t0 + s_un.nt - 1) * TILE,
+                       0, s_c.n_pad) ||
+          !MD_IN_RANGE(a.s.err, s_c.off + s_c.n_pad, 1, a.s.n_total + 1) ||
+          !MD_IN_RANGE(a.s.err, s_un.jrow, 0, a.n_jrecs + 1) ||
+          !MD_IN_RANGE(a.s.err,
+                       s_un.jrow + s_c.n_pad - static_cast<long long>(s_un.block + 1) * kBlock,
+                       -kBlock, a.n_jrecs + 1)) {
+        __syncthreads();
+        continue;
+      }
       const long long i0 = static_cast<long long>(s_un.block) * kBlock;
       const float4* __restrict__ blk = cur + s_c.off + i0;
       const int left = s_c.n_pad - static_cast<int>(i0);  // records from this block on
@@ -513,7 +530,9 @@ __global__ void __launch_bounds__(32 * kPushWarps) k_mut_push(const MutArgs a) {
   const int n_pad = cl->n_pad;
   const int k = static_cast<int>(blockIdx.x % per) * kPushRec + lane;  // in the block
   const long long j = static_cast<long long>(b.block) * a.block + k;   // in the cluster
-  const bool live = j < n_pad;
+  const bool live = j < n_pad && MD_IN_RANGE(a.s.err, cl->off + j, 0, a.s.n_total) &&
+                    MD_IN_RANGE(a.s.err, b.unit0, 0, a.n_units) &&
+                    MD_IN_RANGE(a.s.err, b.unit0 + b.units, 1, a.n_units + 1);
   RecState st;
   static_assert(sizeof(ClusterDev) % 4 == 0, "copied by words");
   for (int q = threadIdx.x; q < static_cast<int>(sizeof(ClusterDev) / 4); q += 32 * kPushWarps)
@@ -546,6 +565,9 @@ __global__ void __launch_bounds__(32 * kPushWarps) k_mut_push(const MutArgs a) {
                                 static_cast<long long>(a.block) * I * (I + 1) / 2;
       const long long later = n_pad - static_cast<long long>(I + 1) * a.block;
       const long long col = j - static_cast<long long>(I + 1) * a.block;
+      if (!MD_IN_RANGE(a.s.err, col, 0, later) ||
+          !MD_IN_RANGE(a.s.err, b.jbase + skipped + later, 1, a.n_jrecs + 1))
+        continue;
       const float* row = a.jpart + 3 * (b.jbase + skipped) + col;
 #pragma unroll
       for (int m = 0; m < 3; ++m) kahan_add(s[m], c[m], __ldcg(row + m * later));

@@ -72,7 +72,10 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
   const long long j0 = rank * seg;
   const long long ns = j0 >= a.ns ? 0 : (a.ns - j0 < seg ? a.ns - j0 : seg);
   const float4* __restrict__ src = a.src + j0;
-  const int ntiles = static_cast<int>((ns + kTile - 1) / kTile);
+  // (checked build: sources outside the array are left out)
+  const int ntiles = ns > 0 && MD_IN_RANGE(a.err, j0 + ns, 1, a.ns + 1)
+                         ? static_cast<int>((ns + kTile - 1) / kTile)
+                         : 0;
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&S.st.full[s], 1);
@@ -197,7 +200,7 @@ __global__ void __launch_bounds__(kThreads) k_probe(const FieldArgs a, long long
   cluster.sync();
   if (rank != 0 || tid >= kTargets) return;
   const long long i = i0 + tid;
-  if (i >= a.nt) return;
+  if (i >= a.nt || !MD_IN_RANGE(a.err, i, 0, a.nt)) return;
   double e[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) {

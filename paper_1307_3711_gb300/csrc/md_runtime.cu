@@ -143,7 +143,7 @@ struct md_ctx {
   md::MutUnit* d_mut_units = nullptr;
   int* d_mut_first = nullptr;
   md::MutBlk* d_mut_blks = nullptr;
-  int mut_shares = 0, mut_blks = 0, mut_grid = 0, mut_block = 0;
+  int mut_shares = 0, mut_units = 0, mut_blks = 0, mut_grid = 0, mut_block = 0;
   float2* d_mut_ipart = nullptr;
   float* d_mut_jpart = nullptr;
   double* d_mut_jphi = nullptr;   // allocated by the first diagnostic step, if there is room
@@ -454,6 +454,8 @@ md::MutArgs mut_args(md_ctx* c) {
   a.units = c->d_mut_units;
   a.share_first = c->d_mut_first;
   a.n_shares = c->mut_shares;
+  a.n_units = c->mut_units;
+  a.n_jrecs = c->mut_jrecs;
   a.blks = c->d_mut_blks;
   a.n_blks = c->mut_blks;
   a.block = c->mut_block;
@@ -1007,6 +1009,7 @@ md_status auto_configure(md_ctx* c) {
                           c->stream));
   MD_CUDA(cudaStreamSynchronize(c->stream));
   c->mut_shares = static_cast<int>(G);
+  c->mut_units = static_cast<int>(units.size());
   c->mut_blks = static_cast<int>(blks.size());
   c->mut_grid = static_cast<int>(std::min(G, slots));
   c->mut_jrecs = jrecs;

@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(THREADS + 64) k_step_small(const StepArgs a,
   const int tl = tid % TL, slice = tid / TL;
   float xi[R], yi[R], zi[R];
   RecState st;
-  const bool pushes = tid < kTargets && b.t0 + tid < n_pad;
+  const bool pushes = tid < kTargets && b.t0 + tid < n_pad &&
+                      MD_IN_RANGE(a.err, off + b.t0 + tid, 0, a.n_total);
   if (tid >= THREADS) {
     if (tid == THREADS)
       for (int t = 0; t < lead; ++t)

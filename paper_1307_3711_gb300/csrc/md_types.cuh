@@ -182,6 +182,8 @@ struct MutArgs {
   const MutUnit* units;
   const int* share_first;  // first unit of every share, n_shares + 1
   int n_shares;
+  int n_units;
+  long long n_jrecs;  // records of all rows of jpart
   const MutBlk* blks;
   int n_blks;
   int block;      // records per i-block
