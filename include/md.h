@@ -241,8 +241,8 @@ md_status md_init_generate(md_ctx **out, const md_config *cfgs, const md_generat
 
 /* md_step: advances every cluster by nsteps full steps (Sec. II): softened
  * Coulomb field at x^n + laser at t_n, relativistic Boris kick, FP64 drift,
- * boundary.  One fused kernel per step; runs of steps are replayed from a
- * captured CUDA graph.  Asynchronous.  nsteps >= 0. */
+ * boundary.  One fused kernel per step, or two where each pair of records is
+ * evaluated once for both; runs of steps are replayed from a captured CUDA graph.  Asynchronous.  nsteps >= 0. */
 md_status md_step(md_ctx *ctx, int32_t nsteps);
 
 /* md_sync: waits for the context's stream and reports device-side errors
@@ -428,10 +428,11 @@ md_status md_get_step(md_ctx *ctx, int64_t *step);
  * another, takes the same kind of step.
  * md_autotune: times every configuration over `steps` steps on the
  * context's own state (restored afterwards), with jsplit 0 and, for the two
- * fastest, jsplit -2 and -4 (no ionizing cluster), then the step that takes
- * each pair once, and keeps the fastest; the
- * per-configuration best mean step times in ms go to times_ms (cap entries,
- * may be NULL; -1 for a configuration not timed). */
+ * fastest, jsplit -2 and -4 (no ionizing cluster), then the step chosen for
+ * the context's size, and keeps the fastest; the per-configuration best mean
+ * step times in ms go to times_ms (cap entries, may be NULL; -1 for a
+ * configuration not timed).  The step chosen for the size has no entry there:
+ * md_get_tuning reports MD_JSPLIT_AUTO where it was the fastest. */
 int32_t md_tuning_list(md_tuning *list, int32_t cap);
 md_status md_set_tuning(md_ctx *ctx, const md_tuning *t);
 md_status md_get_tuning(md_ctx *ctx, md_tuning *t);

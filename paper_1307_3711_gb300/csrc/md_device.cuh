@@ -195,9 +195,9 @@ __device__ __forceinline__ double e1_series(double x) {  // sum_{k >= K} c_k x^(
 // few thousand ions, 336 us for 50000.  Largest relative error over [1e-6, 500]
 // against 40 digits: 7e-15 (Lentz and a series up to 1: 8e-15).
 __device__ inline double expint_e1(double x) {
-  if (!(x > 0.0)) return __longlong_as_double(0x7ff0000000000000LL);  // +inf
+  if (!(x > 0.0)) return __longlong_as_double(0x7ff0000000000000LL);  // +inf (NaN too)
   if (x <= 2.0) return -kEulerGamma - log(x) + x * e1_series<1>(x);
-  if (x > 745.0) return 0.0 * x;  // e^-x underflows (and NaN stays NaN)
+  if (x > 745.0) return 0.0 * x;  // e^-x underflows (NaN at infinity)
   const int n = static_cast<int>(90.0f / static_cast<float>(x)) + 8;
   double a0 = 0.0, a1 = 1.0, b0 = 1.0, b1 = x + 1.0, b = b1, k2 = 1.0, dk = 3.0;
   for (int k = 1; k < n; ++k) {  // k2 = k^2
@@ -1133,13 +1133,6 @@ __device__ __forceinline__ void detect(unsigned long long* hist, unsigned char* 
 }
 
 // The integrator state of one record.
-// (push_record loads it; push_loaded takes it from a caller that loaded it early.)
-// Laser + Boris kick (FP32 increment) + FP64 drift + boundary for record i
-// with Coulomb field (ex, ey, ez); writes x, u and the next j-stream entry.
-// DIAG (diagnostic steps): also the record's diagnostics at t_n, as
-// k_diag_partial forms them from the same kick: status (1 active, 2
-// non-finite; inactive records are left at 0), kinetic energy at the
-// integer-time u = u^{n-1/2} + du/2, potential energy w z phi / 2, momentum.
 struct RecState {
   double X, Y, Z, Ux, Uy, Uz;
   float qm;
@@ -1149,6 +1142,13 @@ __device__ __forceinline__ RecState load_state(const StepArgs& a, long long i) {
   return {a.x[i], a.y[i], a.z[i], a.ux[i], a.uy[i], a.uz[i], a.qm[i]};
 }
 
+// Laser + Boris kick (FP32 increment) + FP64 drift + boundary for record i
+// with Coulomb field (ex, ey, ez); writes x, u and the next j-stream entry.
+// DIAG (diagnostic steps): also the record's diagnostics at t_n, as
+// k_diag_partial forms them from the same kick: status (1 active, 2
+// non-finite; inactive records are left at 0), kinetic energy at the
+// integer-time u = u^{n-1/2} + du/2, potential energy w z phi / 2, momentum.
+// (push_record loads the state; push_loaded takes it from a caller that loaded it early.)
 template <bool DET, bool DIAG = false>
 __device__ __forceinline__ void push_loaded(const StepArgs& a, const ClusterDev& c, long long i,
                                             const RecState& st, double ex, double ey, double ez,

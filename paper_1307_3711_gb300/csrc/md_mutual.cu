@@ -31,9 +31,9 @@
 //     adds a record's partials in a fixed order and pushes it.  The traffic is
 //     12 bytes per i-block and later record each way: 0.24 GB written and read
 //     per step at 200k records, 1 % of its time.
-//   * Work units are runs of tiles of one i-block, cut into equal shares of the
-//     whole context's tiles (a mutual tile weighs 4, a one-sided tile 3) that
-//     a ticket hands out, as in the step kernel.
+//   * Work units are runs of tiles of one i-block.  The whole context's tiles (a
+//     mutual tile weighs 4, a one-sided tile 3) are cut into shares that a ticket
+//     hands out, in rounds of three eighths of the work that is left (auto_configure).
 #include <algorithm>
 
 #include "md_device.cuh"
@@ -47,8 +47,9 @@ constexpr int kMutThreads = 128;
 constexpr int kMutWarps = kMutThreads / 32;
 constexpr int kTile = kMutTile;
 
-// Far away from every record, where a source adds exactly 0 to a sum:
-// r^2 = 3e36 is finite and 1/r^3 underflows to 0.
+// Far away from every record, where a source adds exactly 0 to a field: r^2 =
+// 3e36 is finite and 1/r^3 underflows to 0 (to a potential, before its charge of 0
+// or the tile's is applied, 6e-19).
 constexpr float kFar = 1.0e18f;
 
 // A source tile expanded for packed use, (x,x | y,y) and (z,z | q,q) apart, so

@@ -5,13 +5,13 @@
 // fields through memory: at a few hundred targets most of its lanes hold none.
 // Here a cluster of CTAs takes kTargets targets; its CTAs share the sources,
 // the warps of a CTA share its part (every TL lanes another source of the
-// staged tile), the slices' sums are added in FP64 in shared memory and the
-// CTAs' through distributed shared memory by the cluster's first CTA.
+// staged tile), the warps' sums are joined as compensated FP32 pairs through
+// shared memory, and the CTAs' are added in FP64 by the cluster's first CTA, which
+// receives them through distributed shared memory.
 //
 // A tile is released warp by warp instead of by a CTA-wide barrier and a full
-// tile's loop has a fixed length (3 to 4 % of a large field), and the warps' sums
-// are joined as compensated FP32 pairs, for an FP64 instruction takes its pipe 16
-// cycles (every slice in FP64: 2 us more per call).  Up to four targets per SM the sources' tiles
+// tile's loop has a fixed length (3 to 4 % of a large field); FP32 pairs, for an
+// FP64 instruction takes its pipe 16 cycles (every slice in FP64: 2 us more per call).  Up to four targets per SM the sources' tiles
 // are what a CTA waits for: tiles of 4096, two stages, one CTA per SM and small
 // clusters, which the SMs hold evenly (300 x 150k: 49 us with tiles of 1024 and
 // clusters of eight, 29 so).

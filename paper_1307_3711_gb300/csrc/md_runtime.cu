@@ -782,12 +782,15 @@ void auto_off(md_ctx* c) {
 // Rows of jpart at most: 16 GB (2.1M records in one cluster); a larger context
 // keeps the step kernel.
 constexpr long long kMutMaxRecs = (16LL << 30) / 12;
-// Records from which a cluster with minimum-image forces takes it.  Another
-// order of the sums moves next step's FP32 positions by an ulp here and there,
-// and a pair half a box apart then takes its other image: a kick of up to
-// 8 K_C dt / L^2.  At the density of a solid cluster that stays below 1e-3 of a
-// 10 eV electron's momentum from 11000 records on; smaller periodic clusters
-// keep the step kernel and its order.
+// Records from which a cluster with minimum-image forces takes it; a context with
+// a smaller one keeps the step kernel.  Not a matter of accuracy or of speed:
+// another order of the sums moves next step's FP32 positions by an ulp here and
+// there, and a pair half a box apart then takes its other image, which is as near
+// to the FP64 sum.  It is a kick of up to 8 K_C dt / L^2, at unit charges, dt = 0.02
+// and 400000 records per (16 nm)^3 4e-4 of a 10 eV electron's momentum at 11000
+// records and 2e-3 at 1000; below, trajectories stay those of the step kernel.
+// us per step of a singly charged gas, step kernel and pair-once: 1000 records 94 and
+// 26, 4000 76 and 33, 8000 113 and 49, 11000 166 and 80, 12000 168 and 81.
 constexpr long long kMutMinImageRecords = 11000;
 constexpr long long kMutBigRecords = 40000;
 constexpr long long kMutMinTiles = 2;
