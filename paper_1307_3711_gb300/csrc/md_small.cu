@@ -16,9 +16,9 @@
 // still in flight and leaves; the step does not advance, and the launches that
 // follow (of the same graph) find the error bit and push nothing.
 //
-// Measured (graph replay, us per step): 6.8 at 2000 records (53 with the step
+// Measured (graph replay, us per step): 7.0 at 2000 records (53 with the step
 // kernel's default configuration; 8.1 with the slices' sums in FP64 and the last
-// few sources of a tile one by one), 5.4 at 1000, 11.9 at 3000, 14.9 at 4000, 41.5
+// few sources of a tile one by one), 5.1 at 1000, 11.9 at 3000, 14.6 at 4000, 41.6
 // at 8000; about 5 us of each are the launch, the loads and the push.  More
 // threads per CTA (512, 768), two or four targets per thread, 8 targets per
 // CTA, two stages, a register cap for a fourth CTA per SM and programmatic
