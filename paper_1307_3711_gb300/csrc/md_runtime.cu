@@ -139,6 +139,7 @@ struct md_ctx {
   // partial sums, while `mut_on`
   bool forced = false;  // md_set_tuning or md_autotune chose: no automatic choice
   bool mut_on = false;
+  bool few_charged = false;  // not taken: too few of the records carry charge
   unsigned char* d_mut = nullptr;  // one block for all but the potentials
   md::MutUnit* d_mut_units = nullptr;
   int* d_mut_first = nullptr;
@@ -869,6 +870,21 @@ md_status small_configure(md_ctx* c) {
   return MD_OK;
 }
 
+// Whether a large context holds mostly uncharged records (unused slots): the few
+// charged blocks of the pair-once step fall into few large shares.  Below a third
+// of charged tiles the step kernel is no slower (200k records, the rest unused
+// slots behind the charged ones, ms per step, step kernel / pair-once: 40 % charged
+// 6.85 / 6.71, 30 % 5.40 / 5.57, 20 % 3.95 / 4.18, 10 % 2.59 / 4.24); up to 35000
+// records pair-once is the faster one down to 2 % (0.133 / 0.099).
+md_status count_charged(md_ctx* c) {
+  MD_CUDA(md::launch_count_charged(c->d_posq[0], c->n_total, c->d_word, c->stream));
+  MD_CUDA(cudaMemcpyAsync(c->h_word, c->d_word, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+                          c->stream));
+  MD_CUDA(cudaStreamSynchronize(c->stream));
+  c->few_charged = 3 * static_cast<long long>(*c->h_word) < c->n_total / md::kMutTile;
+  return MD_OK;
+}
+
 // Sets up the step that suits the context's size, if it can take it (no
 // ionizing cluster, no target slice): the small step, or each pair evaluated
 // once if there is room for the partial sums; the configured step kernel stays
@@ -876,6 +892,7 @@ md_status small_configure(md_ctx* c) {
 md_status auto_configure(md_ctx* c) {
   MD_CUDA(cudaStreamSynchronize(c->stream));
   auto_off(c);
+  c->few_charged = false;
   if (c->any_ion || c->any_slice) return MD_OK;
   const md_status small = small_configure(c);
   if (small != MD_OK || c->small_targets) return small;
@@ -908,18 +925,9 @@ md_status auto_configure(md_ctx* c) {
   }
   if (mut_step_us(static_cast<double>(blks.size()), lanes) > step_kernel_us(c)) return MD_OK;
   if (jrecs > kMutMaxRecs || blks.size() > (1u << 25)) return MD_OK;
-  // A large context of mostly uncharged records (unused slots): its few charged
-  // blocks fall into few large shares.  Below a third of charged tiles the step
-  // kernel is no slower (200k records, the rest unused slots behind the charged
-  // ones, ms per step, step kernel / pair-once: 40 % charged 6.85 / 6.71, 30 % 5.40 /
-  // 5.57, 20 % 3.95 / 4.18, 10 % 2.59 / 4.24); up to 35000 records pair-once is
-  // the faster one down to 2 % (0.133 / 0.099).
   if (c->max_n >= kMutBigRecords) {
-    MD_CUDA(md::launch_count_charged(c->d_posq[0], c->n_total, c->d_word, c->stream));
-    MD_CUDA(cudaMemcpyAsync(c->h_word, c->d_word, sizeof(unsigned long long),
-                            cudaMemcpyDeviceToHost, c->stream));
-    MD_CUDA(cudaStreamSynchronize(c->stream));
-    if (3 * static_cast<long long>(*c->h_word) < c->n_total / T) return MD_OK;
+    const md_status st = count_charged(c);
+    if (st != MD_OK || c->few_charged) return st;
   }
   // Shares in rounds of one per resident CTA: a round takes three eighths of
   // the work that is left.  The CTAs of an SM do not advance alike (one share
@@ -2465,8 +2473,13 @@ static md_status md_set_particles_body(md_ctx* c, int32_t cluster, const md_part
   if (!c->ion[cluster].rate_model) {
     // the per-record checks run on the staged copy in device memory
     md_status st = check_block(*in, cluster, c->cl[cluster].n);
-    if (st != MD_OK) return st;
-    return upload_cluster(c, cluster, *in, true);
+    if (st == MD_OK) st = upload_cluster(c, cluster, *in, true);
+    // records that carry charge now, in a context that held too few of them
+    if (st == MD_OK && c->few_charged && !c->forced && !c->any_slice) {
+      st = count_charged(c);
+      if (st == MD_OK && !c->few_charged) st = auto_configure(c);
+    }
+    return st;
   }
   md_status st = validate_particles(*in, cluster, c->cl[cluster].n);
   if (st != MD_OK) return st;

@@ -156,3 +156,31 @@ def test_large_contexts_of_slots_keep_the_step_kernel(md, n, charged, chosen):
         e64 = oracle.coulomb_field(x[idx], x, (w * z).astype(float), EPS,
                                    oracle.coulomb_constant(0.8), self_idx=idx, nthreads=NTHREADS)
         assert summary(force_error(kick, e64))["p99"] <= FORCE_P99
+
+
+def test_charged_records_set_later_take_the_choice_up(md):
+    """A large context made of neutral atoms keeps the step kernel until
+    md_set_particles gives it charges, and a forced tuning beyond that."""
+    n = 41000
+    recs = _records(n, "last", "charged", md)
+    x, u, z, mass, w, kind = recs
+    w = np.ones(n)
+    neutral = (x, u, np.zeros(n, np.int32), mass, w, np.zeros(n, np.uint8))
+    charged = (x, u, z, mass, w, kind)
+    for forced in (False, True):
+        with md.Context([_cfg(md)], [md.HostParticles(*neutral)]) as ctx:
+            assert ctx.tuning()[4] != md.JSPLIT_AUTO
+            ctx.step(2)
+            if forced:
+                ctx.set_tuning(*FORCED)
+            ctx.set_particles(0, md.HostParticles(*neutral))
+            assert ctx.tuning()[4] != md.JSPLIT_AUTO
+            ctx.set_particles(0, md.HostParticles(*charged))
+            assert (ctx.tuning()[4] == md.JSPLIT_AUTO) != forced
+            ctx.step(1)
+            got = ctx.get_particles(0).u
+        with md.Context([_cfg(md)], [md.HostParticles(*charged)]) as ctx:
+            if forced:
+                ctx.set_tuning(*FORCED)
+            ctx.step(1)
+            assert np.array_equal(ctx.get_particles(0).u, got)
